@@ -151,6 +151,25 @@ int sim_reset(qsim *s, uint64_t basis);
  * complex64 norm control then starts afresh after it. */
 int sim_apply(qsim *s, const double *matrix, const int *targets, int t, const int *controls, int c);
 
+/* Gates by name (sim_apply_gates): the gates of the paper's examples (H, X,
+ * Z and Rx of Sec. 4, R of Appendix A.3) and the standard Y, S, T, SWAP, RY,
+ * RZ and U3(theta, phi, lambda). */
+enum qsim_gate_kind {
+    QSIM_G_H = 0, QSIM_G_X, QSIM_G_Y, QSIM_G_Z, QSIM_G_S, QSIM_G_T, QSIM_G_SWAP, /* no parameter */
+    QSIM_G_RX, QSIM_G_RY, QSIM_G_RZ, QSIM_G_R,                                   /* one angle */
+    QSIM_G_U3                                                                    /* three angles */
+};
+
+/* Queue `count` gates by name, as `count` calls of sim_apply with their
+ * matrices: a whole circuit in one call (the paper's engines hand commands
+ * on in lists, Sec. 3).  Gate i has kind kinds[i], nt[i] targets (1; 2 for
+ * SWAP) and nc[i] controls; targets, controls and params hold those of all
+ * gates one after the other.  Stops at the first gate that sim_apply would
+ * refuse and returns its status, the gates before it queued; *queued (may
+ * be NULL) receives their number. */
+int sim_apply_gates(qsim *s, int count, const int *kinds, const int *nt, const int *nc, const int *targets,
+                    const int *controls, const double *params, int *queued);
+
 /* Execute every queued gate: eng.flush() of Sec. 4, listing 1. */
 int sim_flush(qsim *s);
 

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdlib>
@@ -149,8 +150,9 @@ int block_kmax(const qsim *s) {
 // Launch one planned item.  With profiling: events around it; in mode 2
 // also its features and its host time (building the block matrix, the
 // operand record, staging and launching), for the cost model.
-int execute_item(qsim *s, const PlanItem &it) {
+int execute_item(qsim *s, PlanItem &it) {
     const auto h0 = std::chrono::steady_clock::now();
+    const double built_ms = it.host_ms;  // before this call
     int rc;
     size_t ev0 = 0, ev1 = 0;
     // with profiling on, an NVTX range per planned item (visible in a
@@ -186,6 +188,7 @@ int execute_item(qsim *s, const PlanItem &it) {
         cls = gate_class(g);
     } else if (it.diag_block) {
         cls = KC_BLOCK_DIAG;
+        if (it.dtab.empty()) block_matrix(s->queue, it);
         rc = launch_block_diag(s, it.dmask, it.dtab.data());
         bytes = 2.0 * (double)amp_bytes(s) * std::ldexp(1.0, s->n);
     } else if (it.prod_block) {
@@ -196,21 +199,22 @@ int execute_item(qsim *s, const PlanItem &it) {
         s->stats.passes += npasses > 0 ? npasses - 1 : 0;  // one is counted below
     } else if (it.perm_block) {
         int qubits[64], m = 0, kind = 0;
+        if (it.ptab.empty()) block_matrix(s->queue, it);
         for (int b = 0; b < s->n; ++b)
             if ((it.pmask >> b) & 1ull) qubits[m++] = b;
         rc = launch_permutation(s, it.ptab.data(), qubits, m, it.pmask, 0, &kind);
         cls = kind == 2 ? KC_PERMUTE_BULK : kind == 1 ? KC_PERMUTE_CYCLES : KC_PERMUTE;
         bytes = 2.0 * (double)amp_bytes(s) * std::ldexp(1.0, s->n);
     } else {
-        rc = QSIM_ENOTSUP;
-        cls = KC_BLOCK_TC;
-        if (it.k == 6) {
-            cls = KC_BLOCK_TC6;
-            rc = launch_block_tmem(s, it.qubits, 6, it.m.data());
-        } else if (s->prec == QSIM_C64 && it.k >= 4)
-            rc = launch_block_tc(s, it.qubits, it.k, it.m.data());
-        if (rc == QSIM_ENOTSUP) {
+        int q[6];
+        if (const int K = tmem_block_qubits(s, it, q)) {
+            cls = K == 6 ? KC_BLOCK_TC6 : KC_BLOCK_TC;
+            PlanItem *const one = &it;
+            rc = it.operand ? QSIM_OK : build_operands(s, &one, 1);
+            if (!rc) rc = launch_block_tmem(s, it);
+        } else {
             cls = KC_BLOCK_DENSE;
+            if (it.m.empty()) block_matrix(s->queue, it);
             rc = launch_block_dense(s, it.qubits, it.k, it.m.data());
         }
         bytes = 2.0 * (double)amp_bytes(s) * std::ldexp(1.0, s->n);
@@ -228,7 +232,7 @@ int execute_item(qsim *s, const PlanItem &it) {
             s->pending_feats.resize(s->pending_feats.size() + kFeatures);
             item_features(it, s->queue, s->n, s->prec, s->tc_enabled, s->c128_df, &s->pending_feats[feat]);
         }
-        const double host_ms = it.host_ms + std::chrono::duration<double, std::milli>(h1 - h0).count();
+        const double host_ms = built_ms + std::chrono::duration<double, std::milli>(h1 - h0).count();
         s->pending.push_back({cls, ev0, bytes, feat, (float)host_ms});
     }
     s->stats.passes++;
@@ -236,11 +240,48 @@ int execute_item(qsim *s, const PlanItem &it) {
     return QSIM_OK;
 }
 
-int execute_plan(qsim *s, const std::vector<PlanItem> &plan) {
-    for (const PlanItem &it : plan)
+int execute_plan(qsim *s, std::vector<PlanItem> &plan) {
+    for (PlanItem &it : plan)
         if (const int rc = execute_item(s, it)) return rc;
     return QSIM_OK;
 }
+
+// Runs the items of a plan as they come, the operand images of up to
+// kMaxGroup tensor-core blocks built in one launch: the first block at once,
+// then 2, 4, ... so that the device has work while the host plans on.  With
+// profiling on each block's image is built on its own, inside its events.
+struct GroupRunner {
+    // records of a group fit the staging buffer (at most 64 KB each), and its
+    // images and the records of its other items (at most kMaxHeld of 64 KB)
+    // a fraction of the ring, so that none is overwritten before its pass
+    static constexpr int kMaxGroup = 16, kMaxHeld = 64;
+    qsim *s;
+    std::vector<PlanItem> held;
+    int blocks = 0, group = 1;
+    int add(PlanItem &it) {
+        int q[6];
+        const bool tc = tmem_block_qubits(s, it, q) != 0;
+        if ((!tc && held.empty()) || s->profiling) return execute_item(s, it);
+        held.push_back(std::move(it));
+        blocks += tc;
+        return blocks >= group || held.size() >= (size_t)kMaxHeld ? run() : QSIM_OK;
+    }
+    int run() {
+        std::vector<PlanItem *> tc;
+        int q[6];
+        for (PlanItem &it : held)
+            if (tmem_block_qubits(s, it, q)) tc.push_back(&it);
+        if (const int rc = build_operands(s, tc.data(), (int)tc.size())) return rc;
+        const int rc = execute_plan(s, held);
+        held.clear();
+        blocks = 0;
+        group = std::min(2 * group, kMaxGroup);
+        return rc;
+    }
+};
+static_assert(GroupRunner::kMaxGroup * (64u << 10) < kStageBytes &&
+                  GroupRunner::kMaxGroup * (160u << 10) + 2 * GroupRunner::kMaxHeld * (64u << 10) < kWsRingBytes,
+              "a group's records and images stay valid until its passes are issued");
 
 int flush(qsim *s) {
     if (s->queue.empty()) return QSIM_OK;
@@ -263,28 +304,26 @@ int flush(qsim *s) {
             [&](PlanItem &it) {
                 const bool fuse = idx < ch.fuse.size() && ch.fuse[idx];
                 ++idx;
-                if (!it.fused) return execute_item(s, it);
-                if (fuse) {
-                    block_matrix(q, it);
-                    return execute_item(s, it);
+                if (!it.fused || fuse) return execute_item(s, it);
+                for (int gi : it.members) {
+                    PlanItem one = single_item(q, s->n, gi);
+                    if (const int r = execute_item(s, one)) return r;
                 }
-                for (int gi : it.members)
-                    if (const int r = execute_item(s, single_item(q, s->n, gi))) return r;
                 return 0;
             },
             kMaxDiagQubits, false, s->perm_blocks ? perm_min_width(s->prec, ch.kmax) : 0);
     } else {
-        // greedy: each block is launched as soon as it is formed, so the
-        // host's planning of the next blocks overlaps the device's work.
-        // Where planning the queue twice costs less than a tenth of one pass
-        // over the state (about 1 us per gate against 2^n amplitudes read
-        // and written at some 6.5 TB/s), both dense tie rules are planned
-        // first and the one with fewer passes is launched
+        // greedy: blocks are launched as they are formed, so the host's
+        // planning of the next ones overlaps the device's work.  Where
+        // planning the queue twice costs less than a tenth of one pass over
+        // the state (about 1 us per gate against 2^n amplitudes read and
+        // written at some 6.5 TB/s), both dense tie rules are planned first
+        // and the plan with fewer passes is launched
         const bool prod = s->prod_passes && s->prec == QSIM_C64 && s->n >= 12;
         const int perm_min = s->perm_blocks ? perm_min_width(s->prec, block_kmax(s)) : 0;
         const int prod_min = prod ? block_kmax(s) + 1 : 0;
         const double pass_us = 2.0 * (double)amp_bytes(s) * std::ldexp(1.0, s->n) / 6.5e6;
-        int tie = 0;
+        GroupRunner run{s};
         if (2.0 * (double)q.size() < 0.1 * pass_us) {
             std::vector<PlanItem> p0, p1;
             plan_greedy(q, s->n, block_kmax(s), p0, kMaxDiagQubits, false, perm_min, prod_min, 0);
@@ -294,11 +333,15 @@ int flush(qsim *s) {
                 for (const PlanItem &it : p) c += it.prod_block ? (size_t)product_pass_count(it.qmask_prod) : 1;
                 return c;
             };
-            if (passes(p1) < passes(p0)) tie = 1;
+            rc = QSIM_OK;
+            for (PlanItem &it : passes(p1) < passes(p0) ? p1 : p0)
+                if ((rc = run.add(it))) break;
+        } else {
+            rc = plan_greedy_each(
+                s->queue, s->n, block_kmax(s), [&run](PlanItem &it) { return run.add(it); }, kMaxDiagQubits, false,
+                perm_min, prod_min, 0);
         }
-        rc = plan_greedy_each(
-            s->queue, s->n, block_kmax(s), [s](PlanItem &it) { return execute_item(s, it); }, kMaxDiagQubits, true,
-            perm_min, prod_min, tie);
+        if (!rc) rc = run.run();
     }
     s->queue.clear();
     return rc;
@@ -306,32 +349,121 @@ int flush(qsim *s) {
 
 bool is_finite(double x) { return std::isfinite(x); }
 
+// Validate a gate and append it to the queue.
+int queue_gate(qsim *s, const double *matrix, const int *targets, int t, const int *controls, int c) {
+    if (t + c > s->n) return set_err(s, QSIM_ERANGE, "more qubits than the register has");
+    GateRec g;
+    int rc = validate_qubits(s, targets, t, controls, c, &g.tmask, &g.cmask);
+    if (rc) return rc;
+    const int D = 1 << t;
+    for (int i = 0; i < 2 * D * D; ++i)
+        if (!is_finite(matrix[i])) return set_err(s, QSIM_ENONFINITE, "non-finite matrix entry");
+    g.t = t;
+    for (int j = 0; j < t; ++j) g.targets[j] = targets[j];
+    g.controls.assign(controls, controls + c);
+    g.m.resize((size_t)D * D);
+    for (int i = 0; i < D * D; ++i) g.m[i] = cd(matrix[2 * i], matrix[2 * i + 1]);
+    g.kind = classify(g);
+    g.unitary = is_unitary(g);
+    g.perm = perm_map(g, g.pmap);
+    g.diag = true;
+    for (int r = 0; r < D && g.diag; ++r)
+        for (int col = 0; col < D; ++col)
+            if (r != col && g.m[(size_t)r * D + col] != 0.0) {
+                g.diag = false;
+                break;
+            }
+    s->queue.push_back(std::move(g));
+    s->stats.gates++;
+    return QSIM_OK;
+}
+
+// Parameters of a named gate; -1 for an unknown kind.
+int named_params(int kind) {
+    if (kind < QSIM_G_H || kind > QSIM_G_U3) return -1;
+    return kind < QSIM_G_RX ? 0 : kind == QSIM_G_U3 ? 3 : 1;
+}
+
+// The matrix of a named gate, row-major, interleaved: the standard
+// definitions, as paper_1612_08091_gb300/gates.py has them.
+void named_matrix(int kind, const double *p, double *m) {
+    const double pi = 3.14159265358979323846, r = std::sqrt(0.5);
+    std::fill_n(m, kind == QSIM_G_SWAP ? 32 : 8, 0.0);
+    auto set = [&](int e, double re, double im) {
+        m[2 * e] = re;
+        m[2 * e + 1] = im;
+    };
+    switch (kind) {
+    case QSIM_G_H:
+        set(0, r, 0), set(1, r, 0), set(2, r, 0), set(3, -r, 0);
+        return;
+    case QSIM_G_X: set(1, 1, 0), set(2, 1, 0); return;
+    case QSIM_G_Y: set(1, 0, -1), set(2, 0, 1); return;
+    case QSIM_G_Z: set(0, 1, 0), set(3, -1, 0); return;
+    case QSIM_G_S: set(0, 1, 0), set(3, std::cos(pi / 2), std::sin(pi / 2)); return;
+    case QSIM_G_T: set(0, 1, 0), set(3, std::cos(pi / 4), std::sin(pi / 4)); return;
+    case QSIM_G_SWAP: set(0, 1, 0), set(6, 1, 0), set(9, 1, 0), set(15, 1, 0); return;
+    case QSIM_G_R: set(0, 1, 0), set(3, std::cos(p[0]), std::sin(p[0])); return;
+    default: break;
+    }
+    const double c = std::cos(0.5 * p[0]), s = std::sin(0.5 * p[0]);
+    switch (kind) {
+    case QSIM_G_RX: set(0, c, 0), set(1, 0, -s), set(2, 0, -s), set(3, c, 0); return;
+    case QSIM_G_RY: set(0, c, 0), set(1, -s, 0), set(2, s, 0), set(3, c, 0); return;
+    case QSIM_G_RZ: set(0, c, -s), set(3, c, s); return;
+    default: break;  // U3(theta, phi, lambda)
+    }
+    const double phi = p[1], lam = p[2];
+    set(0, c, 0);
+    set(1, -std::cos(lam) * s, -std::sin(lam) * s);
+    set(2, std::cos(phi) * s, std::sin(phi) * s);
+    set(3, std::cos(phi + lam) * c, std::sin(phi + lam) * c);
+}
+
 }  // namespace
 
-int stage_operand(qsim *s, const void *data, size_t bytes, unsigned char **dev) {
+int ring_reserve(qsim *s, size_t bytes, unsigned char **dev) {
     const size_t need = (bytes + 255) & ~(size_t)255;
     if (need > kWsRingBytes) return set_err(s, QSIM_EINVAL, "block operand too large");
+    if (s->ring_cursor + need > kWsRingBytes) {
+        // the passes that read the ring's pieces must have run
+        cudaError_t e = cudaStreamSynchronize(s->stream);
+        if (e != cudaSuccess) return cuda_err(s, e, "stream synchronize");
+        s->ring_cursor = 0;
+    }
+    *dev = (unsigned char *)s->ws + kWsRing + s->ring_cursor;
+    s->ring_cursor += need;
+    return QSIM_OK;
+}
+
+int stage_to(qsim *s, unsigned char *dev, const void *data, size_t bytes) {
+    const size_t need = (bytes + 255) & ~(size_t)255;
+    if (need > kStageBytes) return set_err(s, QSIM_EINVAL, "record too large");
     if (!s->stage_host) {
-        if (cudaMallocHost((void **)&s->stage_host, kWsRingBytes) != cudaSuccess) {
+        if (cudaMallocHost((void **)&s->stage_host, kStageBytes) != cudaSuccess) {
             cudaGetLastError();
             s->stage_host = nullptr;
             return set_err(s, QSIM_ENOMEM, "pinned staging buffer");
         }
         s->stage_cursor = 0;
     }
-    if (s->stage_cursor + need > kWsRingBytes) {
+    cudaError_t e;
+    if (s->stage_cursor + need > kStageBytes) {
         // every earlier copy out of the staging buffer must have run
-        cudaError_t e = cudaStreamSynchronize(s->stream);
+        e = cudaStreamSynchronize(s->stream);
         if (e != cudaSuccess) return cuda_err(s, e, "stream synchronize");
         s->stage_cursor = 0;
     }
     std::memcpy(s->stage_host + s->stage_cursor, data, bytes);
-    unsigned char *d = (unsigned char *)s->ws + kWsRing + s->stage_cursor;
-    cudaError_t e = cudaMemcpyAsync(d, s->stage_host + s->stage_cursor, bytes, cudaMemcpyHostToDevice, s->stream);
+    e = cudaMemcpyAsync(dev, s->stage_host + s->stage_cursor, bytes, cudaMemcpyHostToDevice, s->stream);
     if (e != cudaSuccess) return cuda_err(s, e, "operand copy");
     s->stage_cursor += need;
-    *dev = d;
     return QSIM_OK;
+}
+
+int stage_operand(qsim *s, const void *data, size_t bytes, unsigned char **dev) {
+    const int rc = ring_reserve(s, bytes, dev);
+    return rc ? rc : stage_to(s, *dev, data, bytes);
 }
 
 int check_device_errors(qsim *s) {
@@ -466,30 +598,28 @@ int sim_apply(qsim *s, const double *matrix, const int *targets, int t, const in
     if (!s) return QSIM_EINVAL;
     if (!matrix || !targets || t < 1 || t > 5 || c < 0 || (c > 0 && !controls))
         return set_err(s, QSIM_EINVAL, "bad gate arguments");
-    if (t + c > s->n) return set_err(s, QSIM_ERANGE, "more qubits than the register has");
-    GateRec g;
-    int rc = validate_qubits(s, targets, t, controls, c, &g.tmask, &g.cmask);
-    if (rc) return rc;
-    const int D = 1 << t;
-    for (int i = 0; i < 2 * D * D; ++i)
-        if (!is_finite(matrix[i])) return set_err(s, QSIM_ENONFINITE, "non-finite matrix entry");
-    g.t = t;
-    for (int j = 0; j < t; ++j) g.targets[j] = targets[j];
-    g.controls.assign(controls, controls + c);
-    g.m.resize((size_t)D * D);
-    for (int i = 0; i < D * D; ++i) g.m[i] = cd(matrix[2 * i], matrix[2 * i + 1]);
-    g.kind = classify(g);
-    g.unitary = is_unitary(g);
-    g.perm = perm_map(g, g.pmap);
-    g.diag = true;
-    for (int r = 0; r < D && g.diag; ++r)
-        for (int c = 0; c < D; ++c)
-            if (r != c && g.m[(size_t)r * D + c] != 0.0) {
-                g.diag = false;
-                break;
-            }
-    s->queue.push_back(std::move(g));
-    s->stats.gates++;
+    return queue_gate(s, matrix, targets, t, controls, c);
+}
+
+int sim_apply_gates(qsim *s, int count, const int *kinds, const int *nt, const int *nc, const int *targets,
+                    const int *controls, const double *params, int *queued) {
+    if (queued) *queued = 0;
+    if (!s) return QSIM_EINVAL;
+    if (count < 0 || (count > 0 && (!kinds || !nt || !nc || !targets)))
+        return set_err(s, QSIM_EINVAL, "bad gate arguments");
+    s->queue.reserve(s->queue.size() + (size_t)count);
+    for (int i = 0; i < count; ++i) {
+        double m[32];
+        const int t = kinds[i] == QSIM_G_SWAP ? 2 : 1, np = named_params(kinds[i]);
+        if (np < 0 || nt[i] != t || nc[i] < 0 || (nc[i] > 0 && !controls) || (np > 0 && !params))
+            return set_err(s, QSIM_EINVAL, "bad gate arguments");
+        named_matrix(kinds[i], params, m);
+        if (const int rc = queue_gate(s, m, targets, t, controls, nc[i])) return rc;
+        targets += t;
+        if (nc[i]) controls += nc[i];
+        if (np) params += np;
+        if (queued) *queued = i + 1;
+    }
     return QSIM_OK;
 }
 

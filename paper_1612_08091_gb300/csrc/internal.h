@@ -55,6 +55,7 @@ struct PlanItem {
     int ngates = 0;
     std::vector<int> members;  // queue indices of the gates it executes, in order
     double host_ms = 0;     // host time spent building its matrix (profiling)
+    unsigned char *operand = nullptr;  // tensor-core block: its operand image in the device ring
 };
 
 // The learned cost model used by the planner (host inference).
@@ -100,8 +101,9 @@ struct qsim {
     double norm_target = 1.0;
     uint64_t tc_passes = 0;
     int tc_prev_grid = 0;
-    unsigned char *stage_host = nullptr;  // pinned staging for block operands
-    size_t stage_cursor = 0;
+    unsigned char *stage_host = nullptr;  // pinned staging for records
+    size_t stage_cursor = 0;              // in the staging buffer
+    size_t ring_cursor = 0;               // in the device ring
     // profiling: events around each launch, harvested on demand
     bool profiling = false;
     std::vector<cudaEvent_t> ev_pool;
@@ -144,6 +146,7 @@ constexpr size_t kWsNormBytes = 48u << 10;  // 2 slots x 2 sums x up to kMaxTcGr
 constexpr int kMaxTcGrid = 1024;            // largest grid of a block pass
 constexpr size_t kWsRing = kWsNorm + kWsNormBytes;      // block operand ring
 constexpr size_t kWsRingBytes = 16u << 20;
+constexpr size_t kStageBytes = 2u << 20;                // pinned staging of the records copied to the ring
 constexpr size_t kWsTotal = kWsRing + kWsRingBytes;
 constexpr int kMaxReduceBlocks = 2048;                  // largest reduction grid (partials fit in 1 MiB)
 // Grid of the reduction kernels: four CTAs per SM.
@@ -177,19 +180,27 @@ bool butterfly2(const cd *u);
 int launch_block_diag(qsim *s, uint64_t dmask, const cd *d);
 int launch_set_basis(qsim *s, uint64_t basis);
 
-// Copy a block operand record into the device ring (via pinned staging) on
-// the handle's stream; *dev receives its device address (api.cpp).
+// A piece of the device ring (256-byte aligned).  When the ring is full the
+// stream is waited for and it starts again: pieces stay valid for the work
+// issued before the next full turn.
+int ring_reserve(qsim *s, size_t bytes, unsigned char **dev);
+// Copy host data to a piece of the ring on the handle's stream (through the
+// pinned staging buffer, so the caller's data is free on return).
+int stage_to(qsim *s, unsigned char *dev, const void *data, size_t bytes);
+// Both: a record in the device ring; *dev receives its address (api.cpp).
 int stage_operand(qsim *s, const void *data, size_t bytes, unsigned char **dev);
 // Read and clear the device error flags (synchronises the stream).
 int check_device_errors(qsim *s);
 
-// Fused 4- or 5-qubit tensor-core block (tmem_block_kernel.cu; a 4-qubit
-// block is embedded in a 5-qubit one).  Returns QSIM_ENOTSUP when the
-// block cannot run on the tensor-core kernel (caller falls back).
-int launch_block_tc(qsim *s, const int *qubits, int k, const cd *m);
-// 5- or 6-qubit block with the state operand in tensor memory (complex64,
-// tensor cores, n >= k + 7); QSIM_ENOTSUP otherwise
-int launch_block_tmem(qsim *s, const int *qubits, int k, const cd *m);
+// Tensor-core blocks (tmem_block_kernel.cu): 6 qubits with n >= 13, 4 or 5
+// with n >= 12 (a 4-qubit block runs as a 5-qubit one), complex64.
+// The block's qubits as the kernel takes them (ascending, 5 or 6) in q and
+// their number; 0 where the item does not run on the tensor cores.
+int tmem_block_qubits(const qsim *s, const PlanItem &it, int *q);
+// Build the operand images of `count` such items of the queue, in one launch.
+int build_operands(qsim *s, PlanItem *const *items, int count);
+// Launch one whose image is built; QSIM_ENOTSUP where it does not run there.
+int launch_block_tmem(qsim *s, const PlanItem &it);
 
 // Reductions and measurement (reduce_kernels.cu) ----------------------------
 int run_probs_all(qsim *s, double *p1, double *norm2);

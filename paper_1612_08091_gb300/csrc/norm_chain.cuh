@@ -18,6 +18,7 @@
 
 #include <cmath>
 
+#include "common.cuh"
 #include "internal.h"
 
 namespace qsim_chain {
@@ -31,17 +32,22 @@ struct ChainArgs {
     int prev_grid;
 };
 
-// The output scale of this pass (every CTA's thread 0 computes the same
-// value: fixed summation order); CTA 0 also writes the record.
+// The output scale of this pass, formed by one warp (every CTA computes the
+// same value: fixed summation order; one lane adding up to 2 x 1024 doubles
+// by itself took several microseconds, longer than a pass over a register
+// inside L2); CTA 0 also writes the record.
 __device__ inline float chain_scale(const ChainArgs &c) {
+    const int lane = threadIdx.x & 31;
     float sc = 1.0f;
     double T = c.target;
     if (c.norm_prev) {
         double a = 0.0, b = 0.0;
-        for (int i = 0; i < c.prev_grid; ++i) {
+        for (int i = lane; i < c.prev_grid; i += 32) {
             a += c.norm_prev[i];
             b += c.norm_prev[kMaxTcGrid + i];
         }
+        a = qsim_dev::warp_sum(a);
+        b = qsim_dev::warp_sum(b);
         const double sp = c.rec_prev[0], tp = c.rec_prev[1];
         T = tp > 0.0 ? tp : a;
         if (T > 0.0 && a > 0.0 && b > 0.0 && sp > 0.0 && a < 1e300 && b < 1e300 && T < 1e300) {
@@ -51,7 +57,7 @@ __device__ inline float chain_scale(const ChainArgs &c) {
             if (s2 > 0.25 && s2 < 4.0) sc = (float)sqrt(s2);
         }
     }
-    if (blockIdx.x == 0 && c.rec_out) {
+    if (blockIdx.x == 0 && lane == 0 && c.rec_out) {
         c.rec_out[0] = (double)sc;
         c.rec_out[1] = T;
     }

@@ -146,7 +146,10 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) k_product(const ProdAr
             if ((e >> j) & 1u) a |= 1ull << A.vspec.pos[j];
         return a;
     };
-    if (tid == 0) s_scale = qsim_chain::chain_scale(A.chain);  // and the record
+    if (warp == 0) {
+        const float sc = qsim_chain::chain_scale(A.chain);  // and the record
+        if (lane == 0) s_scale = sc;
+    }
     __syncthreads();
     const float out_scale = s_scale * A.cs;  // every output, before its sign
     const uint64_t off_lo = addr((uint32_t)tid);          // tile bits 0..7 of this thread (stores)

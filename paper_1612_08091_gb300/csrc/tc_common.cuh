@@ -180,7 +180,7 @@ __device__ __forceinline__ void split_pair(float re, float im, uint32_t &hw, uin
 // Host side: round-to-nearest-even bf16 of a float (finite inputs), and the
 // bf16 value back as a double; the operand records split the gate matrix
 // with these in FP64 (R1 = bf16(R), R2 = bf16(R - R1), ...).
-inline uint16_t f32_to_bf16_bits(float f) {
+__host__ __device__ inline uint16_t f32_to_bf16_bits(float f) {
     uint32_t u;
     std::memcpy(&u, &f, 4);
     const uint32_t round = 0x7FFFu + ((u >> 16) & 1u);

@@ -159,11 +159,14 @@ __global__ void __launch_bounds__(kTmThreads, TmShape<K>::kCtasPerSm) k_block_tm
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        // output scale from the previous pass's sums, and record
-        *s_scale = qsim_chain::chain_scale(args.chain);
+        bulk_load(B, args.rec, args.rec_bytes, &bars[0]);
     }
-    __syncthreads();
-    if (tid == 0) bulk_load(B, args.rec, args.rec_bytes, &bars[0]);
+    if (warp == 1) {
+        // output scale from the previous pass's sums, and record
+        const float sc = qsim_chain::chain_scale(args.chain);
+        if ((tid & 31) == 0) *s_scale = sc;
+    }
+    __syncwarp();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(Sh::kCols)
@@ -176,13 +179,9 @@ __global__ void __launch_bounds__(kTmThreads, TmShape<K>::kCtasPerSm) k_block_tm
     const uint32_t tmem = *tmem_slot;
     const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);  // this warp's 32 TMEM lanes
 
-    bool failed = !mbar_wait(&bars[0], 0);
-    if (failed) atomicOr(args.err, 1u);
-    const bool abort0 = __syncthreads_or(failed) != 0;
-
     double nrm_in = 0.0, nrm_out = 0.0;
     const float scale = *s_scale;
-    if (!abort0) {
+    {
         uint64_t coff = 0;  // address bits of this thread's tile column
 #pragma unroll
         for (int j = 0; j < 7; ++j)
@@ -282,7 +281,10 @@ __global__ void __launch_bounds__(kTmThreads, TmShape<K>::kCtasPerSm) k_block_tm
         uint64_t t = blockIdx.x;
         int it = 0;
         bool stop = false;
-        if (t < args.ntiles) load_tile(t);
+        if (t < args.ntiles) load_tile(t);  // in flight while the operand arrives
+        bool failed = !mbar_wait(&bars[0], 0);
+        if (failed) atomicOr(args.err, 1u);
+        if (__syncthreads_or(failed)) t = args.ntiles;  // no tile is processed
         for (; t < args.ntiles; t += gridDim.x, ++it) {
             if (it >= 1) {
                 // MMA(it-1) done: the A columns are free and D holds the
@@ -399,33 +401,148 @@ __global__ void __launch_bounds__(kTmThreads, TmShape<K>::kCtasPerSm) k_block_tm
 // row * 128 with its 16-byte chunks XOR-swizzled by row & 7.  Output j is
 // block row orow(j) and input j' block row irow(j'): the identity, or for
 // the quad fragments of W = 16 (see k_block_tmem) orow(16G + 4h + k) =
-// 16G + 4k + h and irow(16G + 8h + 2k + e) = 16G + 4k + 2h + e.
-int quad_out_row(int j) { return (j & ~15) | ((j & 3) << 2) | ((j >> 2) & 3); }
-int quad_in_row(int j) { return (j & ~15) | (((j >> 1) & 3) << 2) | (((j >> 3) & 1) << 1) | (j & 1); }
+// 16G + 4k + h and irow(16G + 8h + 2k + e) = 16G + 4k + 2h + e.  Here the
+// inverse of both: block row r is output quad_out(r) and input quad_in(r).
+__device__ __forceinline__ int quad_out(int r) { return (r & ~15) | ((r & 3) << 2) | ((r >> 2) & 3); }
+__device__ __forceinline__ int quad_in(int r) {
+    return (r & ~15) | (((r >> 1) & 1) << 3) | (((r >> 2) & 3) << 1) | (r & 1);
+}
 
-void build_operand(const cd *U, int K, int nsplit, bool quad, std::vector<unsigned char> &rec) {
-    const int D = 1 << K, N = 2 * D, half = N * 128, part = (N / 64) * half;
-    rec.assign((size_t)nsplit * part, 0);
-    for (int row = 0; row < N; ++row)
-        for (int k = 0; k < N; ++k) {
-            const int ro = quad ? quad_out_row(row >> 1) : row >> 1;
-            const int ri = quad ? quad_in_row(k >> 1) : k >> 1;
-            const cd u = U[ro * D + ri];
-            const int a = row & 1, b = k & 1;
-            double rem = a == 0 ? (b == 0 ? u.real() : -u.imag()) : (b == 0 ? u.imag() : u.real());
-            const int kb = (k & 63) * 2;
-            const size_t off =
-                (size_t)(k >> 6) * half + (size_t)row * 128 + ((((kb >> 4) ^ (row & 7)) << 4)) + (kb & 15);
-            for (int sp = 0; sp < nsplit; ++sp) {
-                const uint16_t h = f32_to_bf16_bits((float)rem);
-                rem -= bf16_bits_to_double(h);
-                std::memcpy(&rec[(size_t)sp * part + off], &h, 2);
+// Building the images on the device.  U is the ordered product of the
+// block's gates; column c of U is the gates applied to the basis vector
+// e_c, so the columns are independent and a warp (a CTA of its own) takes
+// one: 2^K amplitudes in shared memory in FP64, two or one per lane, each
+// lane forming its outputs' 2^t-term sums.  Then it splits its column into
+// bf16 parts and writes them at their swizzled places.  One launch builds
+// the images of many blocks (blockIdx.y).  On the host the same took 200 us
+// per 6-qubit block (the product of some 28 gates and 16,384 elements
+// split), longer than a pass over a register of 26 qubits or fewer.  Here a
+// launch is bound by the FP64 units' latency and rate (8 FMAs per output,
+// gate and column, two a cycle on an SM): 29 us for one block of 36 gates,
+// 35 us for eight blocks (20-qubit circuit of 21 blocks: 7.66 -> 0.62 ms with
+// the gates queued in one call).
+struct BlockGate {      // one gate of a block, in block-local bits
+    uint32_t cmask;     // controls
+    uint32_t tmask;     // targets
+    uint16_t type;      // 0 dense, 1 diagonal, 2 X
+    uint16_t t;         // targets
+    uint8_t tpos[8];    // target j <-> block bit tpos[j]
+    uint32_t off;       // its matrix (dense: 4^t, diagonal: 2^t entries), bytes from the record's start
+    uint32_t pad[2];
+};
+static_assert(sizeof(cd) == 16 && sizeof(BlockGate) == 32, "records are made of 16-byte units");
+struct BlockJob {       // one block
+    unsigned char *out; // operand image
+    const unsigned char *rec;
+    uint32_t rec_bytes;
+    uint16_t K, quad;
+    uint16_t nsplit, init;  // init: the record is U itself (row-major), no gates
+    uint32_t ngates;
+};
+constexpr int kJobStage = 6144;  // bytes of a record kept in shared memory
+
+__global__ void __launch_bounds__(32) k_build_operand(const BlockJob *__restrict__ jobs) {
+    __shared__ double2 x[64];
+    __shared__ __align__(16) unsigned char stage[kJobStage];
+    const BlockJob J = jobs[blockIdx.y];
+    const int D = 1 << J.K, c = blockIdx.x, lane = threadIdx.x;
+    if (c >= D) return;
+    const unsigned char *rec = J.rec;
+    if (J.rec_bytes <= (uint32_t)kJobStage && !J.init) {
+        const int units = (int)J.rec_bytes / 16;
+#pragma unroll 4
+        for (int i = lane; i < units; i += 32) ((float4 *)stage)[i] = ((const float4 *)J.rec)[i];
+        rec = stage;
+    }
+    const int per = D >> 5;  // outputs per lane: 2 or 1
+    for (int u = 0; u < per; ++u) {
+        const int i = lane + 32 * u;
+        x[i] = J.init ? ((const double2 *)J.rec)[i * D + c] : make_double2(i == c ? 1.0 : 0.0, 0.0);
+    }
+    __syncwarp();
+    for (uint32_t g = 0; g < J.ngates; ++g) {
+        const BlockGate G = ((const BlockGate *)rec)[g];
+        const double2 *m = (const double2 *)(rec + G.off);
+        if (G.t == 1) {
+            // a pair per lane, in place
+            const int b = G.tpos[0], i0 = ((lane >> b) << (b + 1)) | (lane & ((1 << b) - 1)), i1 = i0 | (1 << b);
+            if (lane < D / 2 && ((uint32_t)i0 & G.cmask) == G.cmask) {
+                const double2 v0 = x[i0], v1 = x[i1];
+                double2 y0 = v1, y1 = v0;
+                if (G.type == 0) {
+                    const double2 a = m[0], e = m[1], f = m[2], h = m[3];
+                    y0.x = fma(a.x, v0.x, -a.y * v0.y) + fma(e.x, v1.x, -e.y * v1.y);
+                    y0.y = fma(a.x, v0.y, a.y * v0.x) + fma(e.x, v1.y, e.y * v1.x);
+                    y1.x = fma(f.x, v0.x, -f.y * v0.y) + fma(h.x, v1.x, -h.y * v1.y);
+                    y1.y = fma(f.x, v0.y, f.y * v0.x) + fma(h.x, v1.y, h.y * v1.x);
+                } else if (G.type == 1) {
+                    const double2 a = m[0], h = m[1];
+                    y0 = make_double2(fma(a.x, v0.x, -a.y * v0.y), fma(a.x, v0.y, a.y * v0.x));
+                    y1 = make_double2(fma(h.x, v1.x, -h.y * v1.y), fma(h.x, v1.y, h.y * v1.x));
+                }
+                x[i0] = y0;
+                x[i1] = y1;
+            }
+            __syncwarp();
+            continue;
+        }
+        double2 y[2];
+        for (int u = 0; u < per; ++u) {
+            const int i = lane + 32 * u;
+            y[u] = x[i];
+            if (((uint32_t)i & G.cmask) != G.cmask) continue;
+            int r = 0;
+            for (int j = 0; j < G.t; ++j) r |= ((i >> G.tpos[j]) & 1) << j;
+            if (G.type == 1) {
+                const double2 z = m[r], v = y[u];
+                y[u] = make_double2(fma(z.x, v.x, -z.y * v.y), fma(z.x, v.y, z.y * v.x));
+                continue;
+            }
+            const int base = i & ~(int)G.tmask, T = 1 << G.t;
+            y[u] = make_double2(0.0, 0.0);
+            for (int k = 0; k < T; ++k) {
+                int s = base;
+                for (int j = 0; j < G.t; ++j) s |= ((k >> j) & 1) << G.tpos[j];
+                const double2 w = m[r * T + k], v = x[s];
+                y[u].x += fma(w.x, v.x, -w.y * v.y);
+                y[u].y += fma(w.x, v.y, w.y * v.x);
             }
         }
+        __syncwarp();
+        for (int u = 0; u < per; ++u) x[lane + 32 * u] = y[u];
+        __syncwarp();
+    }
+    // column c of U is input j' = 2^-1 k: elements k = 2j', 2j'+1 of rows 2j, 2j+1
+    const int N = 2 * D, half = N * 128, part = (N / 64) * half;
+    const int k = 2 * (J.quad ? quad_in(c) : c), kb = (k & 63) * 2;
+    for (int u = 0; u < per; ++u) {
+        const int i = lane + 32 * u;
+        const double2 z = x[i];
+        const int j = J.quad ? quad_out(i) : i;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const int row = 2 * j + a;
+            double r0 = a ? z.y : z.x, r1 = a ? z.x : -z.y;
+            unsigned char *dst =
+                J.out + (size_t)(k >> 6) * half + (size_t)row * 128 + ((((kb >> 4) ^ (row & 7)) << 4)) + (kb & 15);
+            for (int sp = 0; sp < J.nsplit; ++sp) {
+                const uint32_t h0 = f32_to_bf16_bits((float)r0), h1 = f32_to_bf16_bits((float)r1);
+                r0 -= (double)__uint_as_float(h0 << 16);
+                r1 -= (double)__uint_as_float(h1 << 16);
+                *(uint32_t *)(dst + (size_t)sp * part) = h0 | (h1 << 16);
+            }
+        }
+    }
+}
+
+// amplitudes per global access (see k_block_tmem)
+int access_width(const int *q) {
+    const bool low4 = q[0] == 0 && q[1] == 1 && q[2] == 2 && q[3] == 3;
+    return low4 ? 16 : (q[0] == 0 && q[1] == 1) ? 4 : (q[0] == 0 ? 2 : 1);
 }
 
 template <int K>
-int launch_tmem(qsim *s, const int *qubits, const cd *m) {
+int launch_tmem(qsim *s, const int *qubits, const unsigned char *dev_rec) {
     using Sh = TmShape<K>;
     const int n = s->n;
     const int nsplit = s->tc_terms == 5 ? 3 : 2;
@@ -450,16 +567,8 @@ int launch_tmem(qsim *s, const int *qubits, const cd *m) {
     // W = 16: tile columns 32w + q + 8i lie qoff[i] from 32w + q
     for (int i = 0; i < 4; ++i)
         a.qoff[i] = ((i & 1) ? 1ull << a.fpos[3] : 0ull) + ((i & 2) ? 1ull << a.fpos[4] : 0ull);
-    // amplitudes per global access (see k_block_tmem)
-    const bool low4 = qubits[0] == 0 && qubits[1] == 1 && qubits[2] == 2 && qubits[3] == 3;
-    const int W = low4 ? 16 : (qubits[0] == 0 && qubits[1] == 1) ? 4 : (qubits[0] == 0 ? 2 : 1);
+    const int W = access_width(qubits);
     const int wi = W == 16 ? 3 : W == 4 ? 2 : W - 1;
-
-    std::vector<unsigned char> rec;
-    build_operand(m, K, nsplit, W == 16, rec);
-    unsigned char *dev_rec = nullptr;
-    int rc = stage_operand(s, rec.data(), rec.size(), &dev_rec);
-    if (rc) return rc;
 
     auto kernel = W == 16 ? k_block_tmem<K, 16>
                           : W == 4 ? k_block_tmem<K, 4> : (W == 2 ? k_block_tmem<K, 2> : k_block_tmem<K, 1>);
@@ -497,7 +606,7 @@ int launch_tmem(qsim *s, const int *qubits, const cd *m) {
     }
     a.psi = (float2 *)s->state;
     a.rec = dev_rec;
-    a.rec_bytes = (uint32_t)rec.size();
+    a.rec_bytes = (uint32_t)(nsplit * Sh::kBPart);
     a.nsplit = nsplit;
     a.ntiles = 1ull << (n - Sh::kTileBits);
     a.err = (unsigned int *)((char *)s->ws + kWsErr);
@@ -511,50 +620,122 @@ int launch_tmem(qsim *s, const int *qubits, const cd *m) {
     return cuda_err(s, cudaGetLastError(), "tmem block launch");
 }
 
-// Embed a k-qubit block (k < 5) into the 5-qubit block on its qubits and the
-// lowest qubits outside them (identity on the added ones), so that it runs
-// on the 5-qubit kernel.  q5 receives the 5 qubits in ascending order.
-void pad_to_five(int n, const int *q, int k, const cd *m, int *q5, std::vector<cd> &m5) {
-    uint64_t S = 0;
-    for (int j = 0; j < k; ++j) S |= 1ull << q[j];
-    uint64_t S5 = S;
-    for (int b = 0; b < n && __builtin_popcountll(S5) < 5; ++b) S5 |= 1ull << b;
-    int kk = 0;
-    for (int b = 0; b < n; ++b)
-        if ((S5 >> b) & 1ull) q5[kk++] = b;
-    int pos[5] = {0, 0, 0, 0, 0};  // position in q5 of block qubit j
-    for (int j = 0; j < k; ++j)
-        for (int i = 0; i < 5; ++i)
-            if (q5[i] == q[j]) pos[j] = i;
-    uint32_t added = 0;  // positions (in q5) of the added qubits
-    for (int i = 0; i < 5; ++i)
-        if (!((S >> q5[i]) & 1ull)) added |= 1u << i;
-    const int D = 1 << k;
-    m5.assign(32 * 32, cd(0.0, 0.0));
-    for (int r = 0; r < 32; ++r)
-        for (int c = 0; c < 32; ++c) {
-            if ((r & added) != (c & added)) continue;
-            int ro = 0, co = 0;
-            for (int j = 0; j < k; ++j) {
-                ro |= ((r >> pos[j]) & 1) << j;
-                co |= ((c >> pos[j]) & 1) << j;
-            }
-            m5[r * 32 + c] = m[ro * D + co];
+// A block's record: its gates in block-local bits and their matrices, or,
+// where that would be longer than U itself, U (block_matrix).
+void block_record(const std::vector<GateRec> &q, const PlanItem &it, const int *S, int K, std::vector<unsigned char> &rec,
+                  BlockJob &job) {
+    const size_t start = rec.size(), D = (size_t)1 << K;
+    size_t bytes = sizeof(BlockGate) * it.members.size();
+    for (int gi : it.members) {
+        const GateRec &g = q[gi];
+        const size_t T = (size_t)1 << g.t;
+        bytes += g.kind == GK_X ? 0 : sizeof(cd) * (g.diag ? T : T * T);
+    }
+    if (bytes > sizeof(cd) * D * D) {
+        PlanItem whole = it;
+        whole.k = K;
+        for (int j = 0; j < K; ++j) whole.qubits[j] = S[j];
+        block_matrix(q, whole);
+        rec.resize(start + sizeof(cd) * D * D);
+        std::memcpy(&rec[start], whole.m.data(), sizeof(cd) * D * D);
+        job.init = 1;
+        job.ngates = 0;
+        job.rec_bytes = (uint32_t)(sizeof(cd) * D * D);
+        return;
+    }
+    rec.resize(start + bytes);
+    BlockGate *gates = (BlockGate *)&rec[start];
+    size_t off = sizeof(BlockGate) * it.members.size();
+    for (size_t i = 0; i < it.members.size(); ++i) {
+        const GateRec &g = q[it.members[i]];
+        BlockGate &b = gates[i];
+        b = BlockGate{};
+        auto bit = [&](int qubit) {
+            int j = 0;
+            while (S[j] != qubit) ++j;
+            return j;
+        };
+        for (int c : g.controls) b.cmask |= 1u << bit(c);
+        for (int j = 0; j < g.t; ++j) {
+            b.tpos[j] = (uint8_t)bit(g.targets[j]);
+            b.tmask |= 1u << b.tpos[j];
         }
+        b.t = (uint16_t)g.t;
+        b.type = g.kind == GK_X ? 2 : g.diag ? 1 : 0;
+        b.off = (uint32_t)off;
+        const int T = 1 << g.t;
+        cd *m = (cd *)&rec[start + off];
+        if (b.type == 0) {
+            std::memcpy((void *)m, g.m.data(), sizeof(cd) * T * T);
+            off += sizeof(cd) * T * T;
+        } else if (b.type == 1) {
+            for (int r = 0; r < T; ++r) m[r] = g.m[(size_t)r * T + r];
+            off += sizeof(cd) * T;
+        }
+    }
+    job.init = 0;
+    job.ngates = (uint32_t)it.members.size();
+    job.rec_bytes = (uint32_t)bytes;
 }
 
 }  // namespace
 
-int launch_block_tmem(qsim *s, const int *qubits, int k, const cd *m) {
-    if (s->prec != QSIM_C64 || !s->tc_enabled || (k != 5 && k != 6) || s->n < k + 7) return QSIM_ENOTSUP;
-    return k == 6 ? launch_tmem<6>(s, qubits, m) : launch_tmem<5>(s, qubits, m);
+int tmem_block_qubits(const qsim *s, const PlanItem &it, int *q) {
+    if (!it.fused || it.diag_block || it.prod_block || it.perm_block || s->prec != QSIM_C64 || !s->tc_enabled) return 0;
+    if (it.k < 4 || it.k > 6 || s->n < (it.k == 6 ? 13 : 12)) return 0;
+    uint64_t S = 0;
+    for (int j = 0; j < it.k; ++j) S |= 1ull << it.qubits[j];
+    // a 4-qubit block runs as the 5-qubit block on its qubits and the lowest
+    // other one
+    for (int b = 0; b < s->n && __builtin_popcountll(S) < 5; ++b) S |= 1ull << b;
+    int K = 0;
+    for (int b = 0; b < s->n; ++b)
+        if ((S >> b) & 1ull) q[K++] = b;
+    return K;
 }
 
-int launch_block_tc(qsim *s, const int *qubits, int k, const cd *m) {
-    if (s->prec != QSIM_C64 || !s->tc_enabled || k < 4 || k > 5 || s->n < 12) return QSIM_ENOTSUP;
-    if (k == 5) return launch_tmem<5>(s, qubits, m);
-    int q5[5];
-    std::vector<cd> m5;
-    pad_to_five(s->n, qubits, k, m, q5, m5);
-    return launch_tmem<5>(s, q5, m5.data());
+int build_operands(qsim *s, PlanItem *const *items, int count) {
+    if (count < 1) return QSIM_OK;
+    const uint32_t nsplit = s->tc_terms == 5 ? 3 : 2;
+    // the jobs, then the records; offsets turn into addresses once the place
+    // in the device ring is known
+    std::vector<unsigned char> rec(sizeof(BlockJob) * count);
+    std::vector<size_t> at(count), image(count);
+    size_t images = 0;
+    int kmax = 5;
+    for (int i = 0; i < count; ++i) {
+        int q[6];
+        const int K = tmem_block_qubits(s, *items[i], q);
+        BlockJob job{};
+        job.K = (uint16_t)K;
+        job.nsplit = (uint16_t)nsplit;
+        job.quad = access_width(q) == 16;
+        at[i] = rec.size();
+        block_record(s->queue, *items[i], q, K, rec, job);
+        std::memcpy(&rec[sizeof(BlockJob) * i], &job, sizeof(job));
+        image[i] = images;
+        images += (size_t)nsplit * (K == 6 ? TmShape<6>::kBPart : TmShape<5>::kBPart);
+        if (K > kmax) kmax = K;
+    }
+    unsigned char *out = nullptr, *dev = nullptr;
+    int rc = ring_reserve(s, images + rec.size() + 512, &out);  // both in one piece of the ring
+    if (rc) return rc;
+    dev = out + ((images + 255) & ~(size_t)255);
+    for (int i = 0; i < count; ++i) {
+        BlockJob *job = (BlockJob *)&rec[sizeof(BlockJob) * i];
+        job->out = out + image[i];
+        job->rec = dev + at[i];
+        items[i]->operand = job->out;
+    }
+    if ((rc = stage_to(s, dev, rec.data(), rec.size()))) return rc;
+    k_build_operand<<<dim3(1u << kmax, (unsigned)count), 32, 0, s->stream>>>((const BlockJob *)dev);
+    s->stats.launches++;
+    return cuda_err(s, cudaGetLastError(), "block operand launch");
+}
+
+int launch_block_tmem(qsim *s, const PlanItem &it) {
+    int q[6];
+    const int K = tmem_block_qubits(s, it, q);
+    if (K == 0 || !it.operand) return QSIM_ENOTSUP;
+    return K == 6 ? launch_tmem<6>(s, q, it.operand) : launch_tmem<5>(s, q, it.operand);
 }
