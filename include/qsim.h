@@ -68,7 +68,8 @@ enum qsim_precision {
 };
 
 enum qsim_fusion {
-    QSIM_FUSE_NONE = 0,   /* one launch per gate ("plain") */
+    QSIM_FUSE_NONE = 0,   /* gate by gate ("plain"): one launch per gate; registers of up to 13
+                             (complex64: 16) qubits run the gates of a flush in one launch */
     QSIM_FUSE_GREEDY = 1, /* greedy grouping into blocks of <= kmax qubits */
     QSIM_FUSE_MLP = 2     /* block boundaries chosen by the learned cost model */
 };

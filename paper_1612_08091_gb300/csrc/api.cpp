@@ -292,7 +292,16 @@ int flush(qsim *s) {
         plan_mlp(q, s->n, s->prec, s->tc_enabled, s->c128_df, s->perm_blocks, block_kmax(s), s->cost, ch);
         s->last_plan_predicted_ms = ch.predicted_ms;
     }
-    if (s->fusion == QSIM_FUSE_NONE || (s->fusion == QSIM_FUSE_MLP && s->cost.loaded() && ch.kmax == 1)) {
+    if (small_queue_ok(s)) {
+        size_t done = 0;
+        rc = launch_small_queue(s, &done);
+        for (size_t i = 0; i < done; ++i) {
+            if (!q[i].unitary) norm_anchor(s, -1.0);
+            s->stats.passes++;
+            s->stats.amp_updates += std::ldexp(1.0, s->n - (int)q[i].controls.size());
+            s->stats.alg_bytes += gate_bytes(s, q[i]);
+        }
+    } else if (s->fusion == QSIM_FUSE_NONE || (s->fusion == QSIM_FUSE_MLP && s->cost.loaded() && ch.kmax == 1)) {
         std::vector<PlanItem> plan;
         plan_none(q, s->n, plan);
         rc = execute_plan(s, plan);

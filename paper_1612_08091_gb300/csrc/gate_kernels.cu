@@ -30,29 +30,37 @@ template <typename Amp, int K> struct MatK { Amp m[(1 << K) * (1 << K)]; uint64_
 // block * 256 kGroups + u * 256 + thread (u < kGroups), and issues all their
 // loads before any arithmetic, so that 4 to 8 amplitudes per thread are in
 // flight (one group per thread left too few bytes in flight for HBM).
-constexpr int kGroups = 4;
-constexpr int kPhaseGroups = 8;  // the phase kernel loads one amplitude per group
+// A register whose groups would not fill the SMs that way takes one group a
+// thread in blocks of 64 (kGroups and kPhaseGroups are then 1): at 12 qubits
+// complex128 two CTAs did all the FP64 work, 8 us a dense gate against
+// 3.5 us.
+constexpr int kWide = 4, kWidePhase = 8;  // the phase kernel loads one amplitude per group
+constexpr int kNarrowThreads = 64;
 
 inline unsigned blocks_for(uint64_t work, int threads) {
     return (unsigned)((work + (uint64_t)threads - 1) / (uint64_t)threads);
 }
+// fewer than two wide blocks per SM
+inline bool narrow(const qsim *s, uint64_t ngroups, int wide) {
+    return ngroups < (uint64_t)s->sms * 2 * 256 * (uint64_t)wide;
+}
 
-template <typename Amp>
+template <typename Amp, int kGroups>
 __global__ void __launch_bounds__(256) k_dense1(Amp *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                 uint64_t cmask, uint64_t tbit, const Mat1<Amp> M) {
-    const uint64_t g0 = blockIdx.x * (uint64_t)(256 * kGroups) + threadIdx.x;
+    const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kGroups) + threadIdx.x;
     uint64_t i0[kGroups];
     Amp a[kGroups], b[kGroups];
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
-            i0[u] = insert_zeros(g0 + u * 256, ins) | cmask;
+        if (g0 + u * blockDim.x < ngroups) {
+            i0[u] = insert_zeros(g0 + u * blockDim.x, ins) | cmask;
             a[u] = psi[i0[u]];
             b[u] = psi[i0[u] | tbit];
         }
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
+        if (g0 + u * blockDim.x < ngroups) {
             Amp na = cmul(M.m[0], a[u]);
             na = cfma(M.m[1], b[u], na);
             Amp nb = cmul(M.m[2], a[u]);
@@ -81,60 +89,60 @@ __global__ void __launch_bounds__(128) k_denseK(Amp *__restrict__ psi, uint64_t 
     }
 }
 
-template <typename Amp>
+template <typename Amp, int kPhaseGroups>
 __global__ void __launch_bounds__(256) k_phase(Amp *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                uint64_t mask, Amp z) {
-    const uint64_t g0 = blockIdx.x * (uint64_t)(256 * kPhaseGroups) + threadIdx.x;
+    const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kPhaseGroups) + threadIdx.x;
     uint64_t i[kPhaseGroups];
     Amp v[kPhaseGroups];
 #pragma unroll
     for (int u = 0; u < kPhaseGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
-            i[u] = insert_zeros(g0 + u * 256, ins) | mask;
+        if (g0 + u * blockDim.x < ngroups) {
+            i[u] = insert_zeros(g0 + u * blockDim.x, ins) | mask;
             v[u] = psi[i[u]];
         }
 #pragma unroll
     for (int u = 0; u < kPhaseGroups; ++u)
-        if (g0 + u * 256 < ngroups) psi[i[u]] = cmul(z, v[u]);
+        if (g0 + u * blockDim.x < ngroups) psi[i[u]] = cmul(z, v[u]);
 }
 
-template <typename Amp>
+template <typename Amp, int kGroups>
 __global__ void __launch_bounds__(256) k_diag1(Amp *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                uint64_t cmask, uint64_t tbit, Amp d0, Amp d1) {
-    const uint64_t g0 = blockIdx.x * (uint64_t)(256 * kGroups) + threadIdx.x;
+    const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kGroups) + threadIdx.x;
     uint64_t i0[kGroups];
     Amp a[kGroups], b[kGroups];
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
-            i0[u] = insert_zeros(g0 + u * 256, ins) | cmask;
+        if (g0 + u * blockDim.x < ngroups) {
+            i0[u] = insert_zeros(g0 + u * blockDim.x, ins) | cmask;
             a[u] = psi[i0[u]];
             b[u] = psi[i0[u] | tbit];
         }
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
+        if (g0 + u * blockDim.x < ngroups) {
             psi[i0[u]] = cmul(d0, a[u]);
             psi[i0[u] | tbit] = cmul(d1, b[u]);
         }
 }
 
-template <typename Amp>
+template <typename Amp, int kGroups>
 __global__ void __launch_bounds__(256) k_x(Amp *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                            uint64_t cmask, uint64_t tbit) {
-    const uint64_t g0 = blockIdx.x * (uint64_t)(256 * kGroups) + threadIdx.x;
+    const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kGroups) + threadIdx.x;
     uint64_t i0[kGroups];
     Amp a[kGroups], b[kGroups];
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
-            i0[u] = insert_zeros(g0 + u * 256, ins) | cmask;
+        if (g0 + u * blockDim.x < ngroups) {
+            i0[u] = insert_zeros(g0 + u * blockDim.x, ins) | cmask;
             a[u] = psi[i0[u]];
             b[u] = psi[i0[u] | tbit];
         }
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
+        if (g0 + u * blockDim.x < ngroups) {
             psi[i0[u]] = b[u];
             psi[i0[u] | tbit] = a[u];
         }
@@ -146,61 +154,64 @@ struct MatDF {
     qsim_df::C2 m[4];
 };
 
+template <int kGroups>
 __global__ void __launch_bounds__(256) k_dense1_df(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                    uint64_t cmask, uint64_t tbit, const MatDF M) {
-    const uint64_t g0 = blockIdx.x * (uint64_t)(256 * kGroups) + threadIdx.x;
+    const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kGroups) + threadIdx.x;
     uint64_t i0[kGroups];
     double2 a[kGroups], b[kGroups];
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
-            i0[u] = insert_zeros(g0 + u * 256, ins) | cmask;
+        if (g0 + u * blockDim.x < ngroups) {
+            i0[u] = insert_zeros(g0 + u * blockDim.x, ins) | cmask;
             a[u] = psi[i0[u]];
             b[u] = psi[i0[u] | tbit];
         }
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
+        if (g0 + u * blockDim.x < ngroups) {
             const qsim_df::C2 x = qsim_df::split(a[u]), y = qsim_df::split(b[u]);
             psi[i0[u]] = qsim_df::to_double(qsim_df::cdot2(M.m[0], x, M.m[1], y));
             psi[i0[u] | tbit] = qsim_df::to_double(qsim_df::cdot2(M.m[2], x, M.m[3], y));
         }
 }
 
+template <int kGroups>
 __global__ void __launch_bounds__(256) k_diag1_df(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                   uint64_t cmask, uint64_t tbit, const MatDF M) {
-    const uint64_t g0 = blockIdx.x * (uint64_t)(256 * kGroups) + threadIdx.x;
+    const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kGroups) + threadIdx.x;
     uint64_t i0[kGroups];
     double2 a[kGroups], b[kGroups];
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
-            i0[u] = insert_zeros(g0 + u * 256, ins) | cmask;
+        if (g0 + u * blockDim.x < ngroups) {
+            i0[u] = insert_zeros(g0 + u * blockDim.x, ins) | cmask;
             a[u] = psi[i0[u]];
             b[u] = psi[i0[u] | tbit];
         }
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
+        if (g0 + u * blockDim.x < ngroups) {
             psi[i0[u]] = qsim_df::to_double(qsim_df::cmul(M.m[0], qsim_df::split(a[u])));
             psi[i0[u] | tbit] = qsim_df::to_double(qsim_df::cmul(M.m[3], qsim_df::split(b[u])));
         }
 }
 
+template <int kPhaseGroups>
 __global__ void __launch_bounds__(256) k_phase_df(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                   uint64_t mask, const MatDF M) {
-    const uint64_t g0 = blockIdx.x * (uint64_t)(256 * kPhaseGroups) + threadIdx.x;
+    const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kPhaseGroups) + threadIdx.x;
     uint64_t i[kPhaseGroups];
     double2 v[kPhaseGroups];
 #pragma unroll
     for (int u = 0; u < kPhaseGroups; ++u)
-        if (g0 + u * 256 < ngroups) {
-            i[u] = insert_zeros(g0 + u * 256, ins) | mask;
+        if (g0 + u * blockDim.x < ngroups) {
+            i[u] = insert_zeros(g0 + u * blockDim.x, ins) | mask;
             v[u] = psi[i[u]];
         }
 #pragma unroll
     for (int u = 0; u < kPhaseGroups; ++u)
-        if (g0 + u * 256 < ngroups) psi[i[u]] = qsim_df::to_double(qsim_df::cmul(M.m[3], qsim_df::split(v[u])));
+        if (g0 + u * blockDim.x < ngroups) psi[i[u]] = qsim_df::to_double(qsim_df::cmul(M.m[3], qsim_df::split(v[u])));
 }
 
 // complex128 k-qubit dense gate or fused block in double-float arithmetic:
@@ -258,20 +269,29 @@ bool gate_df(qsim *s, const GateRec &g) {
     case GK_DENSE: {
         spec(g.tmask | g.cmask);
         const uint64_t ng = 1ull << (s->n - ins.m);
-        k_dense1_df<<<blocks_for(ng, 256 * kGroups), 256, 0, s->stream>>>(psi, ng, ins, g.cmask, tbit, M);
+        if (narrow(s, ng, kWide))
+            k_dense1_df<1><<<blocks_for(ng, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(psi, ng, ins, g.cmask, tbit, M);
+        else
+            k_dense1_df<kWide><<<blocks_for(ng, 256 * kWide), 256, 0, s->stream>>>(psi, ng, ins, g.cmask, tbit, M);
         return true;
     }
     case GK_DIAG1: {
         spec(g.tmask | g.cmask);
         const uint64_t ng = 1ull << (s->n - ins.m);
-        k_diag1_df<<<blocks_for(ng, 256 * kGroups), 256, 0, s->stream>>>(psi, ng, ins, g.cmask, tbit, M);
+        if (narrow(s, ng, kWide))
+            k_diag1_df<1><<<blocks_for(ng, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(psi, ng, ins, g.cmask, tbit, M);
+        else
+            k_diag1_df<kWide><<<blocks_for(ng, 256 * kWide), 256, 0, s->stream>>>(psi, ng, ins, g.cmask, tbit, M);
         return true;
     }
     case GK_PHASE: {
         const uint64_t mask = g.tmask | g.cmask;
         spec(mask);
         const uint64_t ng = 1ull << (s->n - ins.m);
-        k_phase_df<<<blocks_for(ng, 256 * kPhaseGroups), 256, 0, s->stream>>>(psi, ng, ins, mask, M);
+        if (narrow(s, ng, kWidePhase))
+            k_phase_df<1><<<blocks_for(ng, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(psi, ng, ins, mask, M);
+        else
+            k_phase_df<kWidePhase><<<blocks_for(ng, 256 * kWidePhase), 256, 0, s->stream>>>(psi, ng, ins, mask, M);
         return true;
     }
     default:
@@ -343,20 +363,28 @@ int gate_plain(qsim *s, const GateRec &g) {
         const uint64_t mask = g.tmask | g.cmask;
         const InsertSpec ins = make_spec(mask);
         const uint64_t ngroups = 1ull << (s->n - ins.m);
-        k_phase<Amp><<<blocks_for(ngroups, 256 * kPhaseGroups), 256, 0, s->stream>>>(psi, ngroups, ins, mask, amp<Amp>(g.m[3]));
+        if (narrow(s, ngroups, kWidePhase))
+            k_phase<Amp, 1><<<blocks_for(ngroups, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(psi, ngroups, ins, mask, amp<Amp>(g.m[3]));
+        else
+            k_phase<Amp, kWidePhase><<<blocks_for(ngroups, 256 * kWidePhase), 256, 0, s->stream>>>(psi, ngroups, ins, mask, amp<Amp>(g.m[3]));
         break;
     }
     case GK_DIAG1: {
         const InsertSpec ins = make_spec(g.tmask | g.cmask);
         const uint64_t ngroups = 1ull << (s->n - ins.m);
-        k_diag1<Amp><<<blocks_for(ngroups, 256 * kGroups), 256, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit,
-                                                                        amp<Amp>(g.m[0]), amp<Amp>(g.m[3]));
+        if (narrow(s, ngroups, kWide))
+            k_diag1<Amp, 1><<<blocks_for(ngroups, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit, amp<Amp>(g.m[0]), amp<Amp>(g.m[3]));
+        else
+            k_diag1<Amp, kWide><<<blocks_for(ngroups, 256 * kWide), 256, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit, amp<Amp>(g.m[0]), amp<Amp>(g.m[3]));
         break;
     }
     case GK_X: {
         const InsertSpec ins = make_spec(g.tmask | g.cmask);
         const uint64_t ngroups = 1ull << (s->n - ins.m);
-        k_x<Amp><<<blocks_for(ngroups, 256 * kGroups), 256, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit);
+        if (narrow(s, ngroups, kWide))
+            k_x<Amp, 1><<<blocks_for(ngroups, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit);
+        else
+            k_x<Amp, kWide><<<blocks_for(ngroups, 256 * kWide), 256, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit);
         break;
     }
     default: {
@@ -366,7 +394,10 @@ int gate_plain(qsim *s, const GateRec &g) {
             for (int i = 0; i < 4; ++i) M.m[i] = amp<Amp>(g.m[i]);
             const InsertSpec ins = make_spec(g.tmask | g.cmask);
             const uint64_t ngroups = 1ull << (s->n - ins.m);
-            k_dense1<Amp><<<blocks_for(ngroups, 256 * kGroups), 256, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit, M);
+            if (narrow(s, ngroups, kWide))
+            k_dense1<Amp, 1><<<blocks_for(ngroups, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit, M);
+        else
+            k_dense1<Amp, kWide><<<blocks_for(ngroups, 256 * kWide), 256, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit, M);
             break;
         }
         case 2: return dense_k<Amp, 2>(s, g.targets, g.cmask, g.m.data());

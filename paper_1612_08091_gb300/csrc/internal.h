@@ -160,6 +160,10 @@ int cuda_err(qsim *s, cudaError_t e, const char *where);
 // Launchers (gate_kernels.cu) -----------------------------------------------
 int launch_gate_plain(qsim *s, const GateRec &g);
 int launch_block_dense(qsim *s, const int *qubits, int k, const cd *m);
+// The whole queue on a small register in one launch or a few, gate by gate
+// (small_kernel.cu); *done: gates executed.
+bool small_queue_ok(const qsim *s);
+int launch_small_queue(qsim *s, size_t *done);
 // Emulated classical bijection on a register (perm_kernels.cu).
 // *kind: which kernel ran: 0 tiled, 1 cycle walk through registers, 2 cycle
 // walk through the bulk-copy engine

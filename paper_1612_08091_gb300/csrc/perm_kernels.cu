@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(kPermThreads, sizeof(Amp) == 8 ? 6 : 3) k_perm
     uint64_t *roff = ohi + 64;
     uint32_t *finv = (uint32_t *)(roff + R);
     for (unsigned i = threadIdx.x; i < 128; i += kPermThreads) olo[i] = goff[i];  // olo and ohi
+#pragma unroll 8
     for (unsigned i = threadIdx.x; i < D; i += kPermThreads) finv[i] = gfinv[i];
     for (unsigned i = threadIdx.x; i < R; i += kPermThreads) roff[i] = groff[i];
     __syncthreads();

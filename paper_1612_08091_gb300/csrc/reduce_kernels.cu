@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(kRedThreads) k_chunk_sums(const Amp *__restric
 // Inclusive FP64 scan of |psi_i|^2 over one chunk, starting from `carry`;
 // writes the first index whose running sum exceeds `target` (or ~0 if none)
 // and that amplitude.  One block of 1024 threads; per step thread t owns the
-// run of kSearchRun consecutive amplitudes at off + t * kSearchRun: run sums
+// run of `rl` (at most 32) consecutive amplitudes at off + t * rl: run sums
 // (FP64) are scanned across the block, and the one thread whose run crosses
 // the target scans its own amplitudes.
 struct SearchOut {
@@ -705,7 +705,8 @@ struct SearchOut {
 };
 
 constexpr int kSearchThreads = 1024;
-constexpr int kSearchRun = 32;
+constexpr int kSearchRun = 32;  // runs are shorter where a chunk has fewer than 32 x 1024 amplitudes, so
+                                // that all threads take part (12 qubits: 32 us with runs of 32, 6.4 us with runs of 1)
 
 template <typename Amp>
 __global__ void __launch_bounds__(kSearchThreads) k_chunk_search(const Amp *__restrict__ psi, uint64_t begin,
@@ -720,11 +721,12 @@ __global__ void __launch_bounds__(kSearchThreads) k_chunk_search(const Amp *__re
         s_carry = carry;
     }
     __syncthreads();
-    const uint64_t step = (uint64_t)kSearchThreads * kSearchRun;
+    const int rl = (int)(len / kSearchThreads < 1 ? 1 : len / kSearchThreads > kSearchRun ? kSearchRun : len / kSearchThreads);
+    const uint64_t step = (uint64_t)kSearchThreads * rl;
     for (uint64_t off = 0; off < len; off += step) {
-        const uint64_t r0 = off + (uint64_t)threadIdx.x * kSearchRun;  // this thread's run, relative to begin
+        const uint64_t r0 = off + (uint64_t)threadIdx.x * rl;  // this thread's run, relative to begin
         double run = 0.0;
-        for (int k = 0; k < kSearchRun; ++k)
+        for (int k = 0; k < rl; ++k)
             if (r0 + k < len) run += (double)norm2(psi[begin + r0 + k]);
         // inclusive scan of the run sums over the block
         double w = run;
@@ -751,7 +753,7 @@ __global__ void __launch_bounds__(kSearchThreads) k_chunk_search(const Amp *__re
             // in the order of `run`, so the last one equals it and crosses
             double part = 0.0;
             uint64_t hit = r0;
-            for (int k = 0; k < kSearchRun && r0 + k < len; ++k) {
+            for (int k = 0; k < rl && r0 + k < len; ++k) {
                 part += (double)norm2(psi[begin + r0 + k]);
                 hit = r0 + k;
                 if (before + part > target) break;

@@ -1,0 +1,229 @@
+// small_kernel.cu -- a queue of plain gates on a small register, executed one
+// after the other in one launch.
+//
+// The simulator's per-gate sweep (ProjectQ paper, Sec. 4.3.2) over a register
+// of a few thousand amplitudes is bound by the launch, not by the sweep: at
+// 12 qubits a gate is 64 KB of complex128 amplitudes, and a launch with its
+// gap took 3 to 8 us.  Here a cluster of 16 CTAs holds the register in its
+// shared memory (the top 4 qubits are the CTA's rank) and applies the queued
+// gates in order, each with the arithmetic of its plain kernel
+// (gate_kernels.cu), so the results are the same bits:
+//   - a one-qubit gate on a qubit below the rank bits pairs amplitudes of the
+//     same CTA: in place, one block barrier;
+//   - a gate on a rank qubit, or on several qubits: every CTA forms its own
+//     outputs from the others' amplitudes, read through distributed shared
+//     memory, into its second buffer; one cluster barrier before.  A CTA
+//     writes the buffer that others may still be reading only after the next
+//     such barrier, which they reach when they have read.
+// Registers of up to 8 qubits take one CTA.  complex128 runs up to 13 qubits:
+// a dense gate costs 8 FP64 FMAs an amplitude, 0.5 us for 12 qubits on 16 SMs
+// at two a cycle, so larger registers are better off with all SMs
+// (12 qubits, 350 gates: 0.345 ms, 1.0 us a gate, against 2.46 ms launched one
+// by one); complex64 up to 16.
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+
+#include <cstring>
+#include <vector>
+
+#include "common.cuh"
+#include "internal.h"
+
+using namespace qsim_dev;
+namespace cgrp = cooperative_groups;
+
+namespace {
+
+constexpr int kSmallThreads = 128;
+constexpr int kSmallRankBits = 4;
+constexpr int kSmallOneCta = 8;           // registers of up to this many qubits take one CTA
+constexpr uint32_t kSmallRecord = 40960;  // bytes of gates and matrices per launch
+
+struct SmallGate {
+    uint32_t cmask, tmask;  // controls and targets
+    uint32_t off;           // its matrix (4^t, or the entries a diagonal kind needs), bytes from the record's start
+    uint8_t kind, t;        // GateKind, targets
+    uint8_t tpos[6];        // target j <-> qubit tpos[j]
+    uint32_t pad[3];
+};
+static_assert(sizeof(SmallGate) == 32, "records are made of 16-byte units");
+
+template <typename Amp, int RB>
+__global__ void __launch_bounds__(kSmallThreads) k_small(Amp *__restrict__ psi, int n,
+                                                         const unsigned char *__restrict__ rec, int ngates,
+                                                         uint32_t rec_bytes) {
+    extern __shared__ __align__(16) unsigned char sms[];
+    const int nl = n - RB;               // qubits below the rank bits
+    const uint32_t L = 1u << nl;         // amplitudes of this CTA
+    Amp *buf[2] = {(Amp *)sms, (Amp *)sms + L};
+    unsigned char *r = sms + 2 * sizeof(Amp) * (size_t)L;
+    const uint32_t tid = threadIdx.x, rank = RB ? blockIdx.x : 0u;
+    for (uint32_t i = tid; i < rec_bytes / 16; i += kSmallThreads) ((float4 *)r)[i] = ((const float4 *)rec)[i];
+    Amp *x = buf[0], *other = buf[1];
+    for (uint32_t i = tid; i < L; i += kSmallThreads) x[i] = psi[((uint64_t)rank << nl) | i];
+    __syncthreads();
+    const uint32_t base = rank << nl;    // register index of this CTA's amplitude 0
+    for (int g = 0; g < ngates; ++g) {
+        const SmallGate G = ((const SmallGate *)r)[g];
+        const Amp *m = (const Amp *)(r + G.off);
+        if (G.kind == GK_PHASE) {
+            const uint32_t mask = G.cmask | G.tmask;
+            for (uint32_t i = tid; i < L; i += kSmallThreads)
+                if (((base | i) & mask) == mask) x[i] = cmul(m[0], x[i]);
+            __syncthreads();
+        } else if (G.kind == GK_DIAG1) {
+            for (uint32_t i = tid; i < L; i += kSmallThreads)
+                if (((base | i) & G.cmask) == G.cmask) x[i] = cmul(m[((base | i) & G.tmask) ? 1 : 0], x[i]);
+            __syncthreads();
+        } else if (G.t == 1 && G.tpos[0] < nl) {
+            const int b = G.tpos[0];
+            for (uint32_t p = tid; p < L / 2; p += kSmallThreads) {
+                const uint32_t i0 = ((p >> b) << (b + 1)) | (p & ((1u << b) - 1u)), i1 = i0 | (1u << b);
+                if (((base | i0) & G.cmask) != G.cmask) continue;
+                const Amp v0 = x[i0], v1 = x[i1];
+                if (G.kind == GK_X) {
+                    x[i0] = v1;
+                    x[i1] = v0;
+                } else {
+                    x[i0] = cfma(m[1], v1, cmul(m[0], v0));
+                    x[i1] = cfma(m[3], v1, cmul(m[2], v0));
+                }
+            }
+            __syncthreads();
+        } else {
+            // outputs from amplitudes of any CTA, into the other buffer
+            if (RB)
+                cgrp::this_cluster().sync();
+            else
+                __syncthreads();
+            auto at = [&](uint32_t i) {  // amplitude i of the register
+                const uint32_t owner = i >> nl;
+                const Amp *p = RB && owner != rank ? cgrp::this_cluster().map_shared_rank(x, owner) : x;
+                return p[i & (L - 1u)];
+            };
+            for (uint32_t i = tid; i < L; i += kSmallThreads) {
+                const uint32_t gi = base | i;
+                Amp y = x[i];
+                if ((gi & G.cmask) == G.cmask) {
+                    if (G.kind == GK_X) {
+                        y = at(gi ^ G.tmask);
+                    } else {
+                        const uint32_t rest = gi & ~G.tmask;
+                        const int T = 1 << G.t;
+                        uint32_t row = 0;
+                        for (int j = 0; j < G.t; ++j) row |= ((gi >> G.tpos[j]) & 1u) << j;
+                        y = cmul(m[row * T], at(rest));
+                        for (int k = 1; k < T; ++k) {
+                            uint32_t s = rest;
+                            for (int j = 0; j < G.t; ++j) s |= (uint32_t)((k >> j) & 1) << G.tpos[j];
+                            y = cfma(m[row * T + k], at(s), y);
+                        }
+                    }
+                }
+                other[i] = y;
+            }
+            Amp *swap = x;
+            x = other;
+            other = swap;
+            __syncthreads();
+        }
+    }
+    for (uint32_t i = tid; i < L; i += kSmallThreads) psi[((uint64_t)rank << nl) | i] = x[i];
+    if (RB) cgrp::this_cluster().sync();  // no CTA ends while another reads its amplitudes
+}
+
+inline void put(double2 *d, cd z) { *d = make_double2(z.real(), z.imag()); }
+inline void put(float2 *d, cd z) { *d = make_float2((float)z.real(), (float)z.imag()); }
+
+template <typename Amp, int RB>
+int launch_small(qsim *s, const unsigned char *dev, int ngates, uint32_t rec_bytes) {
+    static bool attr[64] = {false};
+    // at most 2 x 2^9 complex128 or 2 x 2^12 complex64 amplitudes, or those of kSmallOneCta qubits
+    constexpr int kMaxSmem = (int)(2 * (sizeof(Amp) == 16 ? 8192 : 32768) + kSmallRecord);
+    if (s->device < 0 || s->device >= 64) return QSIM_ENOTSUP;
+    if (!attr[s->device]) {
+        cudaError_t e =
+            cudaFuncSetAttribute(k_small<Amp, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        if (e == cudaSuccess && RB)
+            e = cudaFuncSetAttribute(k_small<Amp, RB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return cuda_err(s, e, "small register kernel attribute");
+        attr[s->device] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << RB);
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = 2 * (sizeof(Amp) << (s->n - RB)) + rec_bytes;
+    cfg.stream = s->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1u << RB;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = RB ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_small<Amp, RB>, (Amp *)s->state, s->n, dev, ngates, rec_bytes);
+    s->stats.launches++;
+    if (e != cudaSuccess) cudaGetLastError();
+    return cuda_err(s, e, "small register launch");
+}
+
+template <typename Amp>
+int small_queue(qsim *s, size_t *done) {
+    const std::vector<GateRec> &q = s->queue;
+    std::vector<unsigned char> mats;
+    std::vector<SmallGate> gates;
+    for (size_t i = 0; i < q.size();) {
+        gates.clear();
+        mats.clear();
+        for (; i < q.size(); ++i) {
+            const GateRec &g = q[i];
+            const size_t T = (size_t)1 << g.t;
+            const size_t count = g.kind == GK_X ? 0 : g.kind == GK_PHASE ? 1 : g.kind == GK_DIAG1 ? 2 : T * T;
+            const size_t mb = (count * sizeof(Amp) + 15) & ~(size_t)15;
+            if (sizeof(SmallGate) * (gates.size() + 1) + mats.size() + mb > kSmallRecord) break;
+            SmallGate r{};
+            r.cmask = (uint32_t)g.cmask;
+            r.tmask = (uint32_t)g.tmask;
+            r.off = (uint32_t)mats.size();
+            r.kind = (uint8_t)g.kind;
+            r.t = (uint8_t)g.t;
+            for (int j = 0; j < g.t; ++j) r.tpos[j] = (uint8_t)g.targets[j];
+            gates.push_back(r);
+            mats.resize(mats.size() + mb);
+            Amp *d = (Amp *)(mats.data() + r.off);
+            if (g.kind == GK_PHASE) {
+                put(d, g.m[3]);
+            } else if (g.kind == GK_DIAG1) {
+                put(d, g.m[0]);
+                put(d + 1, g.m[3]);
+            } else {
+                for (size_t e = 0; e < count; ++e) put(d + e, g.m[e]);
+            }
+        }
+        const size_t head = sizeof(SmallGate) * gates.size();
+        for (SmallGate &g : gates) g.off += (uint32_t)head;
+        std::vector<unsigned char> rec(head + mats.size());
+        std::memcpy(rec.data(), gates.data(), head);
+        std::memcpy(rec.data() + head, mats.data(), mats.size());
+        unsigned char *dev = nullptr;
+        int rc = stage_operand(s, rec.data(), rec.size(), &dev);
+        if (rc) return rc;
+        rc = s->n <= kSmallOneCta ? launch_small<Amp, 0>(s, dev, (int)gates.size(), (uint32_t)rec.size())
+                                  : launch_small<Amp, kSmallRankBits>(s, dev, (int)gates.size(), (uint32_t)rec.size());
+        if (rc) return rc;
+        *done = i;
+    }
+    return QSIM_OK;
+}
+
+}  // namespace
+
+bool small_queue_ok(const qsim *s) {
+    // fewer than 3 gates: as many launches cost less than the record's copy
+    return s->fusion == QSIM_FUSE_NONE && !s->profiling && !s->c128_df && s->queue.size() >= 3 &&
+           s->n <= (s->prec == QSIM_C128 ? 13 : 16);
+}
+
+int launch_small_queue(qsim *s, size_t *done) {
+    *done = 0;
+    return s->prec == QSIM_C128 ? small_queue<double2>(s, done) : small_queue<float2>(s, done);
+}

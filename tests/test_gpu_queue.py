@@ -32,6 +32,8 @@ def mixed_ops(n, count, seed, wires=None):
         k = kinds[i % len(kinds)]
         t = 2 if k == "SWAP" else int(r.integers(1, 4)) if k == "MAT" else 1
         q = [int(v) for v in r.permutation(wires)[:t + int(r.integers(0, 3))]]
+        if len(q) < t:
+            continue
         npar = {"RX": 1, "RY": 1, "RZ": 1, "R": 1, "U3": 3}.get(k, 0)
         params = tuple(float(v) for v in r.uniform(-7, 7, npar))
         if k == "MAT":
