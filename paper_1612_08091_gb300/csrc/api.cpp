@@ -147,10 +147,11 @@ int block_kmax(const qsim *s) {
     return s->kmax;
 }
 
-// Launch one planned item.  With profiling: events around it; in mode 2
+// Launch one planned item, or a run of diagonal blocks as one pass (it and
+// the `more` after it).  With profiling: events around it; in mode 2
 // also its features and its host time (building the block matrix, the
 // operand record, staging and launching), for the cost model.
-int execute_item(qsim *s, PlanItem &it) {
+int execute_item(qsim *s, PlanItem &it, PlanItem *more = nullptr, int nmore = 0) {
     const auto h0 = std::chrono::steady_clock::now();
     const double built_ms = it.host_ms;  // before this call
     int rc;
@@ -174,6 +175,8 @@ int execute_item(qsim *s, PlanItem &it) {
     // a non-unitary gate changes the norm: no correction across it
     bool unitary = true;
     for (int gi : it.members) unitary = unitary && s->queue[gi].unitary;
+    for (int i = 0; i < nmore; ++i)
+        for (int gi : more[i].members) unitary = unitary && s->queue[gi].unitary;
     if (!unitary) norm_anchor(s, -1.0);
     if (s->profiling) {
         if (s->pending.size() >= 4096 && (rc = harvest(s))) return rc;
@@ -188,8 +191,10 @@ int execute_item(qsim *s, PlanItem &it) {
         cls = gate_class(g);
     } else if (it.diag_block) {
         cls = KC_BLOCK_DIAG;
-        if (it.dtab.empty()) block_matrix(s->queue, it);
-        rc = launch_block_diag(s, it.dmask, it.dtab.data());
+        PlanItem *run[kMaxDiagRun] = {&it};
+        for (int i = 0; i < nmore; ++i) run[1 + i] = more + i;
+        rc = it.operand ? QSIM_OK : build_diag_tables(s, run, 1 + nmore);
+        if (!rc) rc = launch_block_diag(s, run, 1 + nmore);
         bytes = 2.0 * (double)amp_bytes(s) * std::ldexp(1.0, s->n);
     } else if (it.prod_block) {
         int npasses = 0;
@@ -237,6 +242,7 @@ int execute_item(qsim *s, PlanItem &it) {
     }
     s->stats.passes++;
     s->stats.amp_updates += it.amp_updates;
+    for (int i = 0; i < nmore; ++i) s->stats.amp_updates += more[i].amp_updates;
     return QSIM_OK;
 }
 
@@ -246,41 +252,65 @@ int execute_plan(qsim *s, std::vector<PlanItem> &plan) {
     return QSIM_OK;
 }
 
-// Runs the items of a plan as they come, the operand images of up to
-// kMaxGroup tensor-core blocks built in one launch: the first block at once,
-// then 2, 4, ... so that the device has work while the host plans on.  With
-// profiling on each block's image is built on its own, inside its events.
+// Runs the items of a plan as they come.  The device-built images (operands
+// of tensor-core blocks, tables of diagonal blocks) of a group of items are
+// built in one launch each: of the first item at once, then of 2, 4, ... so
+// that the device has work while the host plans on.  Diagonal blocks that
+// follow one another run as one pass, and a group does not end between them.
+// With profiling on the images are built on their own, inside their events;
+// where launches are recorded item by item, nothing is merged.
 struct GroupRunner {
-    // records of a group fit the staging buffer (at most 64 KB each), and its
-    // images and the records of its other items (at most kMaxHeld of 64 KB)
-    // a fraction of the ring, so that none is overwritten before its pass
-    static constexpr int kMaxGroup = 16, kMaxHeld = 64;
+    static constexpr int kMaxGroup = 16, kMaxHeld = 32;
     qsim *s;
     std::vector<PlanItem> held;
-    int blocks = 0, group = 1;
-    int add(PlanItem &it) {
+    int built = 0, group = 1, run_len = 0;  // run_len: diagonal blocks at the end of `held`
+    bool image(const PlanItem &it) const {
         int q[6];
-        const bool tc = tmem_block_qubits(s, it, q) != 0;
-        if ((!tc && held.empty()) || s->profiling) return execute_item(s, it);
+        return it.fused && (it.diag_block || tmem_block_qubits(s, it, q) != 0);
+    }
+    int add(PlanItem &it) {
+        if (s->record_items) return execute_item(s, it);
+        const bool diag = it.fused && it.diag_block, joins = diag && run_len > 0 && run_len < diag_run_limit(s);
+        if ((built >= group || held.size() >= (size_t)kMaxHeld) && !joins)
+            if (const int rc = run()) return rc;
+        const bool img = image(it);
+        if (!img && held.empty()) return execute_item(s, it);
+        run_len = diag ? (joins ? run_len + 1 : 1) : 0;
+        built += img;
         held.push_back(std::move(it));
-        blocks += tc;
-        return blocks >= group || held.size() >= (size_t)kMaxHeld ? run() : QSIM_OK;
+        return QSIM_OK;
     }
     int run() {
-        std::vector<PlanItem *> tc;
-        int q[6];
-        for (PlanItem &it : held)
-            if (tmem_block_qubits(s, it, q)) tc.push_back(&it);
-        if (const int rc = build_operands(s, tc.data(), (int)tc.size())) return rc;
-        const int rc = execute_plan(s, held);
+        int rc = QSIM_OK;
+        if (!s->profiling) {
+            std::vector<PlanItem *> tc, dg;
+            for (PlanItem &it : held)
+                if (image(it)) (it.diag_block ? dg : tc).push_back(&it);
+            rc = build_operands(s, tc.data(), (int)tc.size());
+            if (!rc) rc = build_diag_tables(s, dg.data(), (int)dg.size());
+        }
+        for (size_t i = 0; i < held.size() && !rc;) {
+            size_t j = i + 1;
+            if (held[i].fused && held[i].diag_block)
+                while (j < held.size() && j - i < (size_t)diag_run_limit(s) && held[j].fused && held[j].diag_block) ++j;
+            rc = execute_item(s, held[i], held.data() + i + 1, (int)(j - i - 1));
+            i = j;
+        }
         held.clear();
-        blocks = 0;
+        built = run_len = 0;
         group = std::min(2 * group, kMaxGroup);
         return rc;
     }
 };
-static_assert(GroupRunner::kMaxGroup * (64u << 10) < kStageBytes &&
-                  GroupRunner::kMaxGroup * (160u << 10) + 2 * GroupRunner::kMaxHeld * (64u << 10) < kWsRingBytes,
+// A group's records fit the staging buffer; its images and records and the
+// records of its other items (64 KB at most each) stay in the ring until its
+// passes are issued, also where the ring starts again in between: the group
+// may be longer than kMaxGroup by a run of diagonal blocks
+constexpr size_t kGroupDense = (GroupRunner::kMaxGroup + 1) * (size_t)(160u << 10),
+                 kGroupDiag = (GroupRunner::kMaxHeld + kMaxDiagRun) * ((64u << 10) + kDiagRecordBytes),
+                 kGroupOther = GroupRunner::kMaxHeld * (size_t)(64u << 10);
+static_assert((GroupRunner::kMaxHeld + kMaxDiagRun) * (kDiagRecordBytes + 64) <= kStageBytes &&
+                  2 * (kGroupDiag + kGroupOther) + kGroupDense < kWsRingBytes,
               "a group's records and images stay valid until its passes are issued");
 
 int flush(qsim *s) {

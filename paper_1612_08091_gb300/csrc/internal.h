@@ -55,7 +55,8 @@ struct PlanItem {
     int ngates = 0;
     std::vector<int> members;  // queue indices of the gates it executes, in order
     double host_ms = 0;     // host time spent building its matrix (profiling)
-    unsigned char *operand = nullptr;  // tensor-core block: its operand image in the device ring
+    unsigned char *operand = nullptr;  // its image in the device ring: a tensor-core block's operand, a
+                                       // diagonal block's table
 };
 
 // The learned cost model used by the planner (host inference).
@@ -180,8 +181,14 @@ int product_pass_count(uint64_t qmask);
 // = -s01 s10 (products of H and X), to 1e-12 relative: the matrices a
 // product pass takes (planner.cpp)
 bool butterfly2(const cd *u);
-// Diagonal block: psi_i *= d[bits of i on dmask] (diag_kernels.cu).
-int launch_block_diag(qsim *s, uint64_t dmask, const cd *d);
+// Diagonal blocks (diag_kernels.cu): psi_i *= d[bits of i on dmask].  Build
+// the tables of `count` of them in one launch; apply a run of them (at most
+// diag_run_limit) whose tables are built in one pass.
+constexpr int kMaxDiagRun = 4;
+constexpr size_t kDiagRecordBytes = 48u << 10;  // longest record of a table's gates
+int diag_run_limit(const qsim *s);
+int build_diag_tables(qsim *s, PlanItem *const *items, int count);
+int launch_block_diag(qsim *s, PlanItem *const *items, int count);
 int launch_set_basis(qsim *s, uint64_t basis);
 
 // A piece of the device ring (256-byte aligned).  When the ring is full the
