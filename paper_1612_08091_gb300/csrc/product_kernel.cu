@@ -21,24 +21,24 @@
 // than the issue rate allows at HBM speed; those layers stay with the
 // tensor-core blocks.)
 //
-// A tile is 32 KB of shared memory, double-buffered: the next tile arrives
-// by 16-byte cp.async copies (two amplitudes, bypassing L1) while this one
-// is processed (64 KB per CTA, three CTAs per SM).  256 threads hold 16
-// amplitudes each in three layouts (tile index e, bits 0..11):
-//   A  e = i | tid << 4:                              registers = tile bits 0..3
-//   B  e = (tid & 15) | i << 4 | (tid >> 4) << 8:     registers = tile bits 4..7
-//   C  e = tid | i << 8:                              registers = tile bits 8..11
-// The copies (e = 2 tid + i << 9, 16 bytes each) and the stores (layout C)
-// put the lanes on the lowest tile bits (address bits 0..3 and more:
-// 128-byte runs at least).  Element e sits at shared position
-// e ^ ((e >> 4) & 7) << 1: bits 1..3 XOR bits 4..6, bit 0 kept, so an
-// amplitude pair stays one aligned 16-byte slot; the 16-byte copies and
-// layout-A accesses meet 8 different slots per quarter-warp and the 8-byte
-// accesses of layouts B and C 16 different bank pairs per half-warp.  (A
-// padded layout, rows of 16 with a pitch of 17, needs no address
-// arithmetic per access but measured 5 % slower.)  The global addresses of
-// a thread's copies and stores step through the register bits in Gray-code
-// order, one 64-bit add each.
+// A tile is 32 KB of shared memory.  256 threads hold 16 amplitudes each in
+// three layouts (tile index e, bits 0..11), so that every butterfly finds
+// both amplitudes in one thread's registers:
+//   1  registers = tile bits 0, 1, 10, 11, thread = bits 2..9: loaded from
+//      global memory as whole 32-byte sectors, 1 KB per warp access;
+//   2  registers = tile bits 2..5, read and written back in place;
+//   3  registers = tile bits 6..9, thread = bits 0..5, 10, 11: stored, the
+//      lanes on consecutive amplitudes.
+// A tile crosses shared memory four times; four CTAs per SM cover one
+// another's loads and barriers (three a tile).  Element e sits at position
+// p = e ^ (bits 6..8 of e) << 2, then bit 1 XOR bit 4 of p: the 16-byte
+// writes of eight lanes meet eight different slots, the 8-byte accesses of a
+// warp 32 different places.  The global addresses of a thread's accesses step
+// through the register bits in Gray-code order, one 64-bit add each.
+// Per 28-qubit pass: 0.778 ms (5.52 TB/s, 82 % of HBM) against 0.805 ms with
+// tiles copied in asynchronously ahead (double-buffered, 24 instead of 32
+// warps per SM, six crossings of shared memory).  With 64 amplitudes a thread and two layouts (two crossings, 12 warps
+// per SM) a pass took 1.18 ms: too few warps to cover the latencies.
 //
 // Norm control.  A product pass is one step of the same norm chain as the
 // tensor-core block passes (norm_chain.cuh): its inputs' and outputs' sums
@@ -62,11 +62,10 @@ namespace {
 constexpr int kPBits = 12;                           // tile bits
 constexpr int kPThreads = 256;
 constexpr int kPPer = (1 << kPBits) / kPThreads;     // amplitudes per thread: 16
-constexpr int kPRegBits = 4;                         // log2(kPPer)
-constexpr int kPCtasPerSm = 3;
+constexpr int kPCtasPerSm = 4;
 constexpr int kPMinRun = 4;                          // runs of at least 2^4 amplitudes (128 B)
-constexpr int kPTile = 1 << kPBits;                  // amplitudes per tile buffer
-constexpr int kPSmem = 2 * kPTile * 8;               // two tile buffers (64 KB)
+constexpr int kPTile = 1 << kPBits;                  // amplitudes per tile
+constexpr int kPSmem = kPTile * 8;                   // 32 KB
 
 struct ProdArgs {
     float2 *psi;
@@ -78,12 +77,17 @@ struct ProdArgs {
     uint32_t gmask;           // tile bits that carry a gate
     uint32_t fmask;           // F: tile bits whose s10 differs from s00
     float p[kPBits];          // p = s00 s01 of tile bit j
+    uint64_t step[kPBits];    // address bit of tile bit j
+    uint32_t flip[kPBits];    // the sign bit where F holds tile bit j
     float cs;                 // C sigma
     qsim_chain::ChainArgs chain;  // norm control (norm_chain.cuh)
 };
 
-// shared-memory position of tile element e
-__device__ __forceinline__ uint32_t swz(uint32_t e) { return e ^ (((e >> 4) & 7u) << 1); }
+// shared-memory position of tile element e (linear over GF(2))
+__host__ __device__ constexpr uint32_t swz(uint32_t e) {
+    const uint32_t p = e ^ (((e >> 6) & 7u) << 2);
+    return p ^ (((p >> 4) & 1u) << 1);
+}
 
 // Gray code of step k and the bit it changes from step k - 1
 __host__ __device__ constexpr int gray(int k) { return k ^ (k >> 1); }
@@ -109,41 +113,32 @@ __device__ __forceinline__ void bfly(float2 &v0, float2 &v1, float p) {
     v1 = make_float2(fmaf(-p, b.x, a.x), fmaf(-p, b.y, a.y));
 }
 
-// Butterflies of tile bits base + r (register bit r of the layout), for the
-// r in `bits` (a 4-bit mask)
-__device__ __forceinline__ void stage(float2 (&v)[kPPer], const ProdArgs &A, int base, uint32_t bits) {
+// Butterfly of register bit r (a tile bit's p)
+template <int R>
+__device__ __forceinline__ void stage(float2 (&v)[kPPer], float p) {
 #pragma unroll
-    for (int r = 0; r < kPRegBits; ++r) {
-        if (!((bits >> r) & 1u)) continue;
-        const float p = A.p[base + r];
-#pragma unroll
-        for (int i = 0; i < kPPer; ++i)
-            if (!((i >> r) & 1)) bfly(v[i], v[i | (1 << r)], p);
-    }
+    for (int i = 0; i < kPPer; ++i)
+        if (!((i >> R) & 1)) bfly(v[i], v[i | (1 << R)], p);
 }
 
-// 16-byte asynchronous copy global -> shared (no register staging, not
-// cached in L1)
-__device__ __forceinline__ void cp_async16(void *sdst, const void *gsrc) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(sdst)),
-                 "l"(gsrc)
-                 : "memory");
+// whole-sector load: four adjacent amplitudes (32-byte aligned)
+__device__ __forceinline__ void ld_sector(const float2 *p, float2 &a, float2 &b, float2 &c, float2 &d) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(b.x), "=f"(b.y), "=f"(c.x), "=f"(c.y), "=f"(d.x), "=f"(d.y)
+                 : "l"(p));
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// all of this thread's copies complete
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) k_product(const ProdArgs A) {
-    extern __shared__ __align__(16) float2 smd[];  // two tiles of 2^12 amplitudes (positions swz(e))
+    extern __shared__ __align__(16) float2 x[];  // a tile of 2^12 amplitudes (positions swz(e))
     __shared__ float s_scale;
     __shared__ double s_red[kPThreads / 32][2];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // address bits of tile index e
     auto addr = [&](uint32_t e) {
         uint64_t a = 0;
 #pragma unroll
         for (int j = 0; j < kPBits; ++j)
-            if ((e >> j) & 1u) a |= 1ull << A.vspec.pos[j];
+            if ((e >> j) & 1u) a |= A.step[j];
         return a;
     };
     if (warp == 0) {
@@ -152,104 +147,77 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) k_product(const ProdAr
     }
     __syncthreads();
     const float out_scale = s_scale * A.cs;  // every output, before its sign
-    const uint64_t off_lo = addr((uint32_t)tid);          // tile bits 0..7 of this thread (stores)
-    const uint64_t off_cp = addr((uint32_t)tid << 1);     // tile bits 1..8 of this thread's copies
-    const uint32_t gA = A.gmask & 15u, gB = (A.gmask >> 4) & 15u, gC = (A.gmask >> 8) & 15u;
-    // sign of output i (layout C, e = tid | i << 8) in bit i
-    uint32_t sgn = 0;
-    {
-        const uint32_t f_tid = (uint32_t)__popc((uint32_t)tid & A.fmask) & 1u, f_hi = A.fmask >> 8;
-#pragma unroll
-        for (int i = 0; i < kPPer; ++i) sgn |= ((f_tid ^ (uint32_t)__popc((uint32_t)i & f_hi)) & 1u) << i;
-    }
-    // address bits of tile bits 8..11 (the register index of the copies and
-    // of layout C)
-    uint64_t hb[kPRegBits];
-#pragma unroll
-    for (int r = 0; r < kPRegBits; ++r) hb[r] = 1ull << A.vspec.pos[8 + r];
-    // tile bits 9..11: the register index of the copies
-    uint64_t cb[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) cb[r] = 1ull << A.vspec.pos[9 + r];
-    // layouts A (e = i | tid << 4) and B; C and the copies: e = tid | i << 8
-    const uint32_t eA = (uint32_t)tid << 4, eB = ((uint32_t)tid & 15u) | (((uint32_t)tid >> 4) << 8);
-    // copies of the tile at `base`: elements e, e + 1 with e = 2 tid + k << 9,
-    // k in Gray order
-    auto copy_in = [&](uint64_t base, int buf) {
-        const float2 *p = A.psi + base + off_cp;
-        float2 *d = smd + buf * kPTile;
-#pragma unroll
-        for (int k = 0; k < kPPer / 2; ++k) {
-            const int g = gray(k), b = gray_bit(k);
-            if (b >= 0) p = (gray(k - 1) >> b) & 1 ? p - cb[b] : p + cb[b];
-            cp_async16(d + swz(((uint32_t)tid << 1) | ((uint32_t)g << 9)), p);
-        }
-    };
+    // this thread's tile bits in the three layouts
+    const uint32_t e1 = tid << 2, e2 = (tid & 3u) | ((tid >> 2) << 6), e3 = (tid & 63u) | ((tid >> 6) << 10);
+    const uint64_t off1 = addr(e1), off3 = addr(e3);
+    // the sign of this thread's first output; the others follow bit by bit
+    const float f_tid = (__popc(e3 & A.fmask) & 1) ? -out_scale : out_scale;
+    const uint32_t w1 = swz(e1), r2 = swz(e2), r3 = swz(e3);
     double nin = 0.0, nout = 0.0;
-    uint64_t t = blockIdx.x;
-    uint64_t base = t < A.ntiles ? tile_base(t, A) : 0;
-    if (t < A.ntiles) copy_in(base, 0);
-    cp_async_commit();
-    for (int it = 0; t < A.ntiles; t += gridDim.x, ++it) {
-        cp_async_wait_all();
-        // every thread's copies of tile t have landed, and every thread is
-        // done with iteration it - 1, whose buffer the next copies refill
-        __syncthreads();
-        const uint64_t tn = t + gridDim.x;
-        const uint64_t base_n = tn < A.ntiles ? tile_base(tn, A) : 0;
-        if (tn < A.ntiles) copy_in(base_n, (it + 1) & 1);  // in flight during this tile's stages
-        cp_async_commit();
-        float2 *x = smd + (it & 1) * kPTile;
-        float2 v[kPPer];
-        // layout A: input sums, butterflies of tile bits 0..3
+    for (uint64_t t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
+        const uint64_t base = tile_base(t, A);
+        float2 v[kPPer];  // layout 1: register i = tile bits 0, 1 | bits 10, 11 << 2
         {
+            const float2 *p = A.psi + base + off1;
 #pragma unroll
-            for (int j = 0; j < kPPer / 2; ++j) {
-                const float4 w = *(const float4 *)(x + swz(eA | 2u * (uint32_t)j));
-                v[2 * j] = make_float2(w.x, w.y);
-                v[2 * j + 1] = make_float2(w.z, w.w);
+            for (int k = 0; k < 4; ++k) {
+                const int g = gray(k), b = gray_bit(k);
+                if (b >= 0) p = (gray(k - 1) >> b) & 1 ? p - A.step[10 + b] : p + A.step[10 + b];
+                ld_sector(p, v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
             }
+        }
+        {
             float q[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int i = 0; i < kPPer; ++i) q[i & 3] = fmaf(v[i].x, v[i].x, fmaf(v[i].y, v[i].y, q[i & 3]));
             nin += (double)((q[0] + q[1]) + (q[2] + q[3]));
-            if (gA) {
-                stage(v, A, 0, gA);
+        }
+        if (A.gmask & 1u) stage<0>(v, A.p[0]);
+        if (A.gmask & 2u) stage<1>(v, A.p[1]);
+        if (A.gmask & 0x400u) stage<2>(v, A.p[10]);
+        if (A.gmask & 0x800u) stage<3>(v, A.p[11]);
+        __syncthreads();  // the previous tile has been read
 #pragma unroll
-                for (int j = 0; j < kPPer / 2; ++j)
-                    *(float4 *)(x + swz(eA | 2u * (uint32_t)j)) =
-                        make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 a = v[4 * g + 2 * h], b = v[4 * g + 2 * h + 1];
+                *(float4 *)(x + (w1 ^ swz(((uint32_t)g << 10) | (2u * h)))) = make_float4(a.x, a.y, b.x, b.y);
             }
+        __syncthreads();
+        if (A.gmask & 0x3Cu) {
+#pragma unroll
+            for (int i = 0; i < kPPer; ++i) v[i] = x[r2 ^ swz((uint32_t)i << 2)];
+            if (A.gmask & 4u) stage<0>(v, A.p[2]);
+            if (A.gmask & 8u) stage<1>(v, A.p[3]);
+            if (A.gmask & 0x10u) stage<2>(v, A.p[4]);
+            if (A.gmask & 0x20u) stage<3>(v, A.p[5]);
+#pragma unroll
+            for (int i = 0; i < kPPer; ++i) x[r2 ^ swz((uint32_t)i << 2)] = v[i];
             __syncthreads();
         }
-        if (gB) {
-            // layout B: butterflies of tile bits 4..7
 #pragma unroll
-            for (int i = 0; i < kPPer; ++i) v[i] = x[swz(eB | ((uint32_t)i << 4))];
-            stage(v, A, 4, gB);
-#pragma unroll
-            for (int i = 0; i < kPPer; ++i) x[swz(eB | ((uint32_t)i << 4))] = v[i];
-            __syncthreads();
-        }
-        // layout C: butterflies of tile bits 8..11, the output factors,
-        // output sums, stores
-#pragma unroll
-        for (int i = 0; i < kPPer; ++i) v[i] = x[swz((uint32_t)tid | ((uint32_t)i << 8))];
-        stage(v, A, 8, gC);
+        for (int i = 0; i < kPPer; ++i) v[i] = x[r3 ^ swz((uint32_t)i << 6)];
+        if (A.gmask & 0x40u) stage<0>(v, A.p[6]);
+        if (A.gmask & 0x80u) stage<1>(v, A.p[7]);
+        if (A.gmask & 0x100u) stage<2>(v, A.p[8]);
+        if (A.gmask & 0x200u) stage<3>(v, A.p[9]);
         {
             float q[4] = {0.f, 0.f, 0.f, 0.f};
-            float2 *p = A.psi + base + off_lo;
+            float2 *p = A.psi + base + off3;
+            float f = f_tid;
 #pragma unroll
             for (int k = 0; k < kPPer; ++k) {
                 const int i = gray(k), b = gray_bit(k);
-                if (b >= 0) p = (gray(k - 1) >> b) & 1 ? p - hb[b] : p + hb[b];
+                if (b >= 0) {
+                    p = (gray(k - 1) >> b) & 1 ? p - A.step[6 + b] : p + A.step[6 + b];
+                    f = __uint_as_float(__float_as_uint(f) ^ A.flip[6 + b]);
+                }
                 q[k & 3] = fmaf(v[i].x, v[i].x, fmaf(v[i].y, v[i].y, q[k & 3]));
-                const float f = ((sgn >> i) & 1u) ? -out_scale : out_scale;
                 *p = make_float2(v[i].x * f, v[i].y * f);
             }
             nout += (double)((q[0] + q[1]) + (q[2] + q[3]));
         }
-        base = base_n;
     }
     // per-CTA sums, fixed order; the outputs' sum before the chain's scale
     nin = warp_sum(nin);
@@ -293,6 +261,8 @@ int launch_pass(qsim *s, const int *qubits, const cd *const *mats, int m) {
                     C *= std::abs(u[0]);
                     sigma *= s00;
                 }
+            a.step[k] = 1ull << b;
+            a.flip[k] = (a.fmask >> k) & 1u ? 0x80000000u : 0u;
             a.vspec.pos[k++] = b;
         }
     a.cs = (float)(C * sigma);
