@@ -14,9 +14,11 @@
 // subspace (Z, S, T, R(phi), CZ, multi-controlled Z), a diagonal one-qubit
 // gate (RZ), and the X permutation (X, CNOT, Toffoli).
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "df128.cuh"
+#include "fx128.cuh"
 #include "internal.h"
 
 using namespace qsim_dev;
@@ -35,6 +37,7 @@ template <typename Amp, int K> struct MatK { Amp m[(1 << K) * (1 << K)]; uint64_
 // complex128 two CTAs did all the FP64 work, 8 us a dense gate against
 // 3.5 us.
 constexpr int kWide = 4, kWidePhase = 8;  // the phase kernel loads one amplitude per group
+constexpr int kWideFx = 2;                 // k_dense1_fx: 4 groups leave too few warps, 1 too few loads in flight
 constexpr int kNarrowThreads = 64;
 
 inline unsigned blocks_for(uint64_t work, int threads) {
@@ -68,6 +71,41 @@ __global__ void __launch_bounds__(256) k_dense1(Amp *__restrict__ psi, uint64_t 
             psi[i0[u]] = na;
             psi[i0[u] | tbit] = nb;
         }
+}
+
+// complex128 one-qubit dense gate in shared-exponent integers (fx128.cuh): 26
+// qubits 0.43 ms (5.0 TB/s, 74 % of HBM) against 1.03 ms in FP64 arithmetic;
+// bound by the integer multiply-add pipe (78 % busy).
+template <int kGroups>
+__global__ void __launch_bounds__(256) k_dense1_fx(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
+                                                   uint64_t cmask, uint64_t tbit, const qsim_fx::MatFx M) {
+    const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kGroups) + threadIdx.x;
+    // the groups' first indices: a zero bit inserted at p turns i into
+    // i + (i & -2^p), two operations (the integer units are the bottleneck)
+    uint64_t i0[kGroups];
+#pragma unroll
+    for (int u = 0; u < kGroups; ++u) i0[u] = g0 + u * blockDim.x;
+    for (int j = 0; j < ins.m; ++j) {
+        const uint64_t high = ~0ull << ins.pos[j];
+#pragma unroll
+        for (int u = 0; u < kGroups; ++u) i0[u] += i0[u] & high;
+    }
+    double2 a[kGroups], b[kGroups];
+#pragma unroll
+    for (int u = 0; u < kGroups; ++u)
+        if (g0 + u * blockDim.x < ngroups) {
+            i0[u] |= cmask;
+            a[u] = psi[i0[u]];
+            b[u] = psi[i0[u] | tbit];
+        }
+#pragma unroll
+    for (int u = 0; u < kGroups; ++u) {
+        if (g0 + u * blockDim.x >= ngroups) continue;
+        double2 na, nb;
+        qsim_fx::dense1(M, a[u], b[u], na, nb);
+        psi[i0[u]] = na;
+        psi[i0[u] | tbit] = nb;
+    }
 }
 
 template <typename Amp, int K>
@@ -390,10 +428,22 @@ int gate_plain(qsim *s, const GateRec &g) {
     default: {
         switch (g.t) {
         case 1: {
-            Mat1<Amp> M;
-            for (int i = 0; i < 4; ++i) M.m[i] = amp<Amp>(g.m[i]);
             const InsertSpec ins = make_spec(g.tmask | g.cmask);
             const uint64_t ngroups = 1ull << (s->n - ins.m);
+            if constexpr (sizeof(Amp) == 16) {
+                qsim_fx::MatFx F;
+                if (qsim_fx::make_fx(g.m.data(), F)) {
+                    if (narrow(s, ngroups, kWideFx))
+                        k_dense1_fx<1><<<blocks_for(ngroups, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(
+                            psi, ngroups, ins, g.cmask, tbit, F);
+                    else
+                        k_dense1_fx<kWideFx><<<blocks_for(ngroups, 256 * kWideFx), 256, 0, s->stream>>>(
+                            psi, ngroups, ins, g.cmask, tbit, F);
+                    break;
+                }
+            }
+            Mat1<Amp> M;
+            for (int i = 0; i < 4; ++i) M.m[i] = amp<Amp>(g.m[i]);
             if (narrow(s, ngroups, kWide))
             k_dense1<Amp, 1><<<blocks_for(ngroups, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(psi, ngroups, ins, g.cmask, tbit, M);
         else

@@ -18,8 +18,8 @@
 // Registers of up to 8 qubits take one CTA.  complex128 runs up to 13 qubits:
 // a dense gate costs 8 FP64 FMAs an amplitude, 0.5 us for 12 qubits on 16 SMs
 // at two a cycle, so larger registers are better off with all SMs
-// (12 qubits, 350 gates: 0.345 ms, 1.0 us a gate, against 2.46 ms launched one
-// by one); complex64 up to 16.
+// (12 qubits, 350 gates: 0.33 ms against 2.46 ms launched one by one);
+// complex64 up to 16.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fx128.cuh"
 #include "internal.h"
 
 using namespace qsim_dev;
@@ -37,14 +38,15 @@ namespace {
 constexpr int kSmallThreads = 128;
 constexpr int kSmallRankBits = 4;
 constexpr int kSmallOneCta = 8;           // registers of up to this many qubits take one CTA
-constexpr uint32_t kSmallRecord = 40960;  // bytes of gates and matrices per launch
+constexpr uint32_t kSmallRecord = 81920;  // bytes of gates and matrices per launch
 
 struct SmallGate {
     uint32_t cmask, tmask;  // controls and targets
     uint32_t off;           // its matrix (4^t, or the entries a diagonal kind needs), bytes from the record's start
     uint8_t kind, t;        // GateKind, targets
     uint8_t tpos[6];        // target j <-> qubit tpos[j]
-    uint32_t pad[3];
+    uint32_t fx;            // its matrix is a qsim_fx::MatFx
+    uint32_t pad[2];
 };
 static_assert(sizeof(SmallGate) == 32, "records are made of 16-byte units");
 
@@ -84,7 +86,15 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(Amp *__restrict__ psi, 
                 if (G.kind == GK_X) {
                     x[i0] = v1;
                     x[i1] = v0;
-                } else {
+                    continue;
+                }
+                if constexpr (sizeof(Amp) == 16) {
+                    if (G.fx) {
+                        qsim_fx::dense1(*(const qsim_fx::MatFx *)m, v0, v1, x[i0], x[i1]);
+                        continue;
+                    }
+                }
+                {
                     x[i0] = cfma(m[1], v1, cmul(m[0], v0));
                     x[i1] = cfma(m[3], v1, cmul(m[2], v0));
                 }
@@ -107,6 +117,10 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(Amp *__restrict__ psi, 
                 if ((gi & G.cmask) == G.cmask) {
                     if (G.kind == GK_X) {
                         y = at(gi ^ G.tmask);
+                    } else if (sizeof(Amp) == 16 && G.fx) {
+                        if constexpr (sizeof(Amp) == 16)
+                            y = qsim_fx::dense1_row(*(const qsim_fx::MatFx *)m, (gi & G.tmask) ? 1 : 0,
+                                                    at(gi & ~G.tmask), at(gi | G.tmask));
                     } else {
                         const uint32_t rest = gi & ~G.tmask;
                         const int T = 1 << G.t;
@@ -178,7 +192,10 @@ int small_queue(qsim *s, size_t *done) {
             const GateRec &g = q[i];
             const size_t T = (size_t)1 << g.t;
             const size_t count = g.kind == GK_X ? 0 : g.kind == GK_PHASE ? 1 : g.kind == GK_DIAG1 ? 2 : T * T;
-            const size_t mb = (count * sizeof(Amp) + 15) & ~(size_t)15;
+            qsim_fx::MatFx fx;
+            const bool use_fx =
+                sizeof(Amp) == 16 && g.t == 1 && g.kind == GK_DENSE && qsim_fx::make_fx(g.m.data(), fx);
+            const size_t mb = ((use_fx ? sizeof(fx) : count * sizeof(Amp)) + 15) & ~(size_t)15;
             if (sizeof(SmallGate) * (gates.size() + 1) + mats.size() + mb > kSmallRecord) break;
             SmallGate r{};
             r.cmask = (uint32_t)g.cmask;
@@ -190,7 +207,10 @@ int small_queue(qsim *s, size_t *done) {
             gates.push_back(r);
             mats.resize(mats.size() + mb);
             Amp *d = (Amp *)(mats.data() + r.off);
-            if (g.kind == GK_PHASE) {
+            if (use_fx) {
+                gates.back().fx = 1;
+                std::memcpy((void *)d, &fx, sizeof(fx));
+            } else if (g.kind == GK_PHASE) {
                 put(d, g.m[3]);
             } else if (g.kind == GK_DIAG1) {
                 put(d, g.m[0]);
