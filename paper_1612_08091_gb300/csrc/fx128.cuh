@@ -75,10 +75,21 @@ __device__ __forceinline__ Fx to_fx(double x, int E) {
 struct Acc {
     long long a, b;
 };
+// s + a b.  Written out: from (long long)a * b with a factor it knows not to
+// be negative the compiler makes several mixed-sign instructions (3.5 in
+// place of one in a block gate).
+__device__ __forceinline__ long long mad_wide(int a, int b, long long s) {
+#ifdef __CUDA_ARCH__
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(a), "r"(b));
+    return s;
+#else
+    return s + (long long)a * b;
+#endif
+}
 __device__ __forceinline__ void mac(Acc &s, Fx m, Fx x) {
-    s.a += (long long)m.hi * x.hi;
-    s.b += (long long)m.hi * x.lo;
-    s.b += (long long)m.lo * x.hi;
+    s.a = mad_wide(m.hi, x.hi, s.a);
+    s.b = mad_wide(m.hi, x.lo, s.b);
+    s.b = mad_wide(m.lo, x.hi, s.b);
 }
 
 // The sum as a double: units of 2^(E - 1081 - S); eadd = (E - 1025 - S) 2^20.
@@ -87,6 +98,42 @@ __device__ __forceinline__ void mac(Acc &s, Fx m, Fx x) {
 // took twice the whole gate's other integer work.
 __device__ __forceinline__ double to_double(const Acc &s, int eadd) {
     const double d = (double)(s.a + (s.b >> 28));  // units of 2^56; |.| <= 2^62 + 2^34
+    const int h = __double2hiint(d);
+    return __hiloint2double(h ? h + eadd : 0, __double2loint(d));
+}
+
+// ---------------------------------------------------------------------------
+// gates on several qubits: 51 bits, the cross sums in FP32
+// ---------------------------------------------------------------------------
+// For the handles that allow double-float accuracy.  v = x 2^(1073 - E) = hi
+// 2^25 + lo with 26 bits and a sign in hi; a matrix element w = m 2^S in the
+// same form (lo rounded to nearest, -2^24..2^24), scaled so that its largest
+// row sum of |re| + |im| is below 2^52.  The sum of hi hi' is exact in 64 bits
+// (one multiply-add a product, four cycles of a pipe that plain FP32 does not
+// need); the cross terms, 2^-25 of it, go to an FP32 sum, which is off by some
+// 2^-24 of that.  Error of a result: some 2^-48 of the group's largest
+// amplitude.
+struct FxF {  // an amplitude's component
+    int hi;
+    float fhi, flo;  // hi rounded, lo exact
+};
+__device__ __forceinline__ FxF to_fxf(double x, int E) {
+    const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+    const uint32_t sg = (uint32_t)((int)h >> 31);
+    const unsigned long long m =
+        ((unsigned long long)(((h & 0xFFFFFu) | 0x100000u) ^ sg) << 32) | (unsigned long long)(l ^ sg);
+    const long long v = shr_s64((long long)m, (uint32_t)(E + 2 - (int)((h >> 20) & 0x7FFu)));
+    FxF r;
+    r.hi = (int)(v >> 25);
+    r.fhi = (float)r.hi;
+    r.flo = (float)((uint32_t)v & 0x1FFFFFFu);
+    return r;
+}
+// a 2^50 + c 2^25 as a double: units of 2^(E - 1073 - S); eadd = (E - 1023 - S)
+// 2^20.  |c| < 2^55.2: sum |w.hi| < 2^27 times lo < 2^25, and up to 32 terms
+// of |w.lo| <= 2^24 times |hi| <= 2^26.
+__device__ __forceinline__ double to_double_f(long long a, float c, int eadd) {
+    const double d = (double)(a + (long long)__float2int_rn(c * 0x1p-25f));
     const int h = __double2hiint(d);
     return __hiloint2double(h ? h + eadd : 0, __double2loint(d));
 }

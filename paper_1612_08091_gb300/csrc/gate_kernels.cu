@@ -15,6 +15,7 @@
 // gate (RZ), and the X permutation (X, CNOT, Toffoli).
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "common.cuh"
 #include "df128.cuh"
@@ -252,7 +253,93 @@ __global__ void __launch_bounds__(256) k_phase_df(double2 *__restrict__ psi, uin
         if (g0 + u * blockDim.x < ngroups) psi[i[u]] = qsim_df::to_double(qsim_df::cmul(M.m[3], qsim_df::split(v[u])));
 }
 
-// complex128 k-qubit dense gate or fused block in double-float arithmetic:
+// complex128 k-qubit dense gate or fused block where the handle allows
+// double-float accuracy, in shared-exponent integers and FP32 (fx128.cuh): a
+// thread takes a group's 2^k amplitudes; a complex product is 4 integer
+// multiply-adds and 8 FP32 ones, on two halves of the FMA pipe, where pairs of
+// FP32 took 48 operations; one FP64 conversion per result.  26 qubits, 4-qubit
+// blocks: 0.80 ms a pass (2.69 TB/s) against 1.59 ms, bound by issue (69 %) and
+// the integer multiply-adds (60 % of their pipe); a 27-pass circuit ends 6.0e-14
+// from 64 bits, with pairs 6.2e-14.  (With the cross sums in integers too, 9
+// multiply-adds a product: 1.4e-15, but 1.09 ms a pass.)
+template <int K> struct MatKFx {
+    // each element's re and im (hi, hi rounded, lo) for 16- and 8-byte loads
+    int4 a[(1 << K) * (1 << K)];    // re hi, im hi, and both as floats
+    float2 b[(1 << K) * (1 << K)];  // re lo, im lo
+    uint64_t off[1 << K];
+    int shift;                    // -1023 - S
+    double unit;                  // 2^-S
+};
+
+template <int K>
+__global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
+                                                   uint64_t cmask, const MatKFx<K> M) {
+    using namespace qsim_fx;
+    constexpr int D = 1 << K;
+    const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (g >= ngroups) return;
+    double2 *const p = psi + (insert_zeros(g, ins) | cmask);
+    double2 v[D];
+    uint32_t top = 0;
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+        v[r] = p[M.off[r]];
+        top = max(top, mag(v[r]));
+    }
+    const int E = (int)(top >> 20);
+    if (!fx_range(E)) {
+        bool zero = top == 0;
+#pragma unroll
+        for (int r = 0; r < D; ++r) zero = zero && v[r].x == 0.0 && v[r].y == 0.0;
+        if (zero) return;
+        // amplitudes near the ends of the range: FP64
+#pragma unroll 1
+        for (int r = 0; r < D; ++r) {
+            double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+                const int4 w = M.a[r * D + c];
+                const float2 l = M.b[r * D + c];
+                acc = cfma(make_double2((w.x * 0x1p25 + l.x) * M.unit, (w.y * 0x1p25 + l.y) * M.unit), v[c], acc);
+            }
+            p[M.off[r]] = acc;
+        }
+        return;
+    }
+    FxF xr[D], xi[D];
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+        xr[r] = to_fxf(v[r].x, E);
+        xi[r] = to_fxf(v[r].y, E);
+    }
+    const int eadd = (E + M.shift) << 20;
+#pragma unroll 2
+    for (int r = 0; r < D; ++r) {
+        long long rr = 0, ii = 0, ri = 0;  // sums of mr xr, mi xi, mr xi + mi xr
+        float cr = 0.f, ci = 0.f;          // cross sums of the two results
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            const int4 w = M.a[r * D + c];
+            const float2 l = M.b[r * D + c];
+            const float frh = __int_as_float(w.z), fih = __int_as_float(w.w);
+            rr = mad_wide(w.x, xr[c].hi, rr);
+            ii = mad_wide(w.y, xi[c].hi, ii);
+            ri = mad_wide(w.x, xi[c].hi, ri);
+            ri = mad_wide(w.y, xr[c].hi, ri);
+            cr = fmaf(frh, xr[c].flo, cr);
+            cr = fmaf(l.x, xr[c].fhi, cr);
+            cr = fmaf(-fih, xi[c].flo, cr);
+            cr = fmaf(-l.y, xi[c].fhi, cr);
+            ci = fmaf(frh, xi[c].flo, ci);
+            ci = fmaf(l.x, xi[c].fhi, ci);
+            ci = fmaf(fih, xr[c].flo, ci);
+            ci = fmaf(l.y, xr[c].fhi, ci);
+        }
+        p[M.off[r]] = make_double2(to_double_f(rr - ii, cr, eadd), to_double_f(ri, ci, eadd));
+    }
+}
+
+// complex128 5-qubit dense gate or fused block in double-float arithmetic:
 // the group's 2^k amplitudes split into FP32 pairs, each output the sum of
 // 2^k exact-product complex MACs with two-sum additions, rounded once to
 // double.  About 40 FP32 operations per MAC instead of 4 FP64 FMAs (FP64
@@ -370,10 +457,7 @@ int dense_k_df(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
 }
 
 template <typename Amp, int K>
-int dense_k(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
-    if constexpr (sizeof(Amp) == 16) {
-        if (s->c128_df) return dense_k_df<K>(s, targets, cmask, m);
-    }
+int dense_k_plain(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
     constexpr int D = 1 << K;
     MatK<Amp, K> M;
     uint64_t tmask = 0;
@@ -390,6 +474,65 @@ int dense_k(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
     k_denseK<Amp, K><<<blocks_for(ngroups, 128), 128, 0, s->stream>>>((Amp *)s->state, ngroups, ins, cmask, M);
     s->stats.launches++;
     return cuda_err(s, cudaGetLastError(), "dense gate launch");
+}
+
+template <int K>
+int dense_k_fx(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
+    constexpr int D = 1 << K;
+    MatKFx<K> M;
+    uint64_t tmask = 0;
+    for (int j = 0; j < K; ++j) tmask |= 1ull << targets[j];
+    for (int r = 0; r < D; ++r) {
+        uint64_t o = 0;
+        for (int j = 0; j < K; ++j)
+            if ((r >> j) & 1) o |= 1ull << targets[j];
+        M.off[r] = o;
+    }
+    double rows = 0.0;  // largest sum of |re| + |im| of a row
+    for (int r = 0; r < D; ++r) {
+        double t = 0.0;
+        for (int c = 0; c < D; ++c) t += std::abs(m[r * D + c].real()) + std::abs(m[r * D + c].imag());
+        rows = std::max(rows, t);
+    }
+    // a zero or an extreme matrix: FP64
+    if (!(rows > 0x1p-64) || !(rows < 0x1p64)) return dense_k_plain<double2, K>(s, targets, cmask, m);
+    int x;
+    std::frexp(rows, &x);  // rows < 2^x
+    const int S = 52 - x;
+    for (int i = 0; i < D * D; ++i) {
+        auto part = [&](double v, int &hi, float &fhi, float &flo) {
+            const long long w = std::llrint(std::ldexp(v, S));
+            hi = (int)((w + (1ll << 24)) >> 25);
+            fhi = (float)hi;
+            flo = (float)(w - ((long long)hi << 25));
+        };
+        float fr, fi;
+        part(m[i].real(), M.a[i].x, fr, M.b[i].x);
+        part(m[i].imag(), M.a[i].y, fi, M.b[i].y);
+        std::memcpy(&M.a[i].z, &fr, 4);
+        std::memcpy(&M.a[i].w, &fi, 4);
+    }
+    M.shift = -1023 - S;
+    M.unit = std::ldexp(1.0, -S);
+    const InsertSpec ins = make_spec(tmask | cmask);
+    const uint64_t ngroups = 1ull << (s->n - ins.m);
+    k_denseK_fx<K><<<blocks_for(ngroups, 128), 128, 0, s->stream>>>((double2 *)s->state, ngroups, ins, cmask, M);
+    s->stats.launches++;
+    return cuda_err(s, cudaGetLastError(), "integer dense gate launch");
+}
+
+template <typename Amp, int K>
+int dense_k(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
+    if constexpr (sizeof(Amp) == 16) {
+        // integers up to 4 qubits; the 32 amplitudes of a 5-qubit group in FP32
+        // pairs, whose plans the narrower blocks beat either way (27 qubits,
+        // depth 10: 56 ms with 4-qubit blocks, 69 ms with integer 5-qubit ones)
+        if (s->c128_df) {
+            if constexpr (K <= 4) return dense_k_fx<K>(s, targets, cmask, m);
+            return dense_k_df<K>(s, targets, cmask, m);
+        }
+    }
+    return dense_k_plain<Amp, K>(s, targets, cmask, m);
 }
 
 template <typename Amp>
