@@ -182,7 +182,7 @@ int sim_flush(qsim *s);
  * amplitude of register value x moves to register value f(x).  Flushes the
  * queue, then runs at once (one pass over the touched groups; fixed points
  * of f are not touched when the register and controls lie above the lowest
- * 4 KB of amplitudes and f's cycles give at least one task per SM). */
+ * 64 bytes of amplitudes and f's cycles give at least one task per SM). */
 int sim_apply_permutation(qsim *s, const uint64_t *perm, const int *qubits, int m, const int *controls, int c);
 
 /* P(qubit = 1) = sum of |psi_i|^2 over indices with bit q set, accumulated

@@ -26,16 +26,19 @@
 // 6..11 of the value), the run offsets and f^-1 come from a device record
 // and are copied to shared memory once per CTA.  m <= 12.
 //
-// Where the register and the controls lie above the 9 lowest qubits (8 for
-// complex128: 4 KB of contiguous amplitudes), the permutation
+// Where the register and the controls leave the 3 lowest qubits free (2 for
+// complex128: pieces of 64 contiguous bytes), the permutation
 // instead follows the cycles of f: for a cycle e_0 -> e_1 -> ... -> e_{L-1}
-// -> e_0 and a slice of 4 KB at the same place in every register value's
-// block, the data rotate one step along the cycle in place,
+// -> e_0 and a slice of 4 KB of the amplitudes that share a register value
+// (the free qubits' lowest bits), the data rotate one step along the cycle in
+// place,
 //   new[e_{i+1}] = old[e_i],
 // walked from e_{L-1} down to e_0 with the loads of the next eight elements
-// in flight (a load of e_j always precedes the store to e_j).  Every access
-// of a CTA is 4 KB contiguous, fixed points of f are not touched, and the
-// work is (cycle, slice) tasks, longest cycles first.  Above the lowest 16 KB
+// in flight (a load of e_j always precedes the store to e_j).  Fixed points
+// of f are not touched, and the work is (cycle, slice) tasks, longest cycles
+// first.  (A tile of a 12-qubit register above qubit 2 has room for runs of 32
+// bytes only, 128 KB for one CTA per SM: 1.55 ms on 28 qubits against 0.86 ms,
+// 5.0 TB/s, for the walk.)  Above the lowest 16 KB
 // the same walk runs through the bulk-copy engine (k_permute_cycles_bulk).
 #include <cuda_runtime.h>
 
@@ -146,8 +149,11 @@ __global__ void __launch_bounds__(kCycThreads) k_permute_cycles(float4 *__restri
             loaded = cyc;
         }
         const uint64_t *e = s_e;
-        // this thread's 16 bytes of the slice at register value 0
-        float4 *p = psi16 + (((insert_zeros(sl << (8 + amp_shift), ins) >> amp_shift) | cmask16) + threadIdx.x);
+        // this thread's 16 bytes of the slice at register value 0: 256
+        // consecutive units of the free qubits, contiguous memory below the
+        // lowest register or control qubit
+        float4 *p =
+            psi16 + ((insert_zeros(((sl << 8) | threadIdx.x) << amp_shift, ins) >> amp_shift) | cmask16);
         const float4 first = p[e[L - 1]];
         float4 r[kCycDepth];  // r[j] holds old[e_{L-2-j}], then the element kCycDepth further down
 #pragma unroll
@@ -270,18 +276,20 @@ __global__ void __launch_bounds__(32) k_permute_cycles_bulk(unsigned char *__res
     }
 }
 
-// The cycle walk when the register and the controls leave the lowest 4 KB
-// of amplitudes contiguous and there are enough tasks to fill the GPU;
+// The cycle walk when the register and the controls leave the lowest 64
+// bytes of amplitudes contiguous and there are enough tasks to fill the GPU;
 // returns QSIM_ENOTSUP otherwise (the tiled kernel then runs).
 template <typename Amp>
 int permute_cycles(qsim *s, const uint64_t *perm, const int *qubits, int m, uint64_t qmask, uint64_t cmask,
                    bool *bulk) {
     *bulk = false;
     const int amp_shift = sizeof(Amp) == 8 ? 1 : 0;  // amplitudes per 16 bytes: 2 or 1
-    const int slice_bits = 8 + amp_shift;  // 4 KB slices: 512 c64 or 256 c128 amplitudes
+    const int slice_bits = 8 + amp_shift;  // slices of 4 KB: 512 c64 or 256 c128 amplitudes
     const int bulk_bits = slice_bits + 2;  // 16 KB slices for the bulk-copy walk
     const uint64_t fixed = qmask | cmask;
-    if ((fixed & ((1ull << slice_bits) - 1ull)) != 0) return QSIM_ENOTSUP;
+    const int nfree = s->n - m - __builtin_popcountll(cmask);
+    // a thread's 16 bytes, and pieces of at least 64 bytes, contiguous
+    if ((fixed & ((1ull << (2 + amp_shift)) - 1ull)) != 0 || nfree < slice_bits) return QSIM_ENOTSUP;
     const int D = 1 << m;
     // the cycles of f, longest first
     std::vector<std::vector<uint32_t>> cycles;
@@ -298,7 +306,6 @@ int permute_cycles(qsim *s, const uint64_t *perm, const int *qubits, int m, uint
         cycles.push_back(std::move(cy));
     }
     if (cycles.empty()) return QSIM_OK;  // f is the identity
-    const int nfree = s->n - m - __builtin_popcountll(cmask);
     const uint64_t nslices = 1ull << (nfree - slice_bits);
     if ((uint64_t)cycles.size() * nslices < (uint64_t)s->sms) return QSIM_ENOTSUP;
     // the bulk-copy walk: 16 KB slices, at least two tasks per SM
