@@ -12,25 +12,15 @@
 // ladder is one permutation: applied in order it maps |b> to |b'> with
 // b'_k = b_0 ^ ... ^ b_k, i.e. psi'[y] = psi[y ^ (y << 1) mod 2^n].
 //
-// One persistent launch: every CTA takes circuit ids from an atomic counter
-// (largest circuits first) until the batch is done; there is no waiting on
-// other CTAs.  A circuit of n <= m qubits (m = 12..14, tuned) lives in the
-// CTA's shared memory; a larger one lives in a per-CTA pair of global
-// buffers and is processed in chunks of 2^g amplitudes (g = 12):
-//   pair pass: the ladder permutation of the previous layer maps the
-//     destination chunks hi and hi ^ (2^h - 1) (h = n - g) onto the same two
-//     source chunks S, S ^ 1 with S = hi ^ (hi << 1): an element at offset o
-//     of source chunk S ^ p lands in chunk hi if parity(o) == p, else in its
-//     partner, at the offset whose bit k is the XOR of bits 0..k of o.  Both
-//     source chunks are copied whole into shared memory and stay in source
-//     order there (logical qubit k pairs the elements p and p ^ (3 << k)),
-//     get the gates on qubits 0..g-1, and are written back whole, each
-//     destination element read from its source position;
-//   high pass: tiles made of runs of 2^(g-h) amplitudes times the h top
-//     qubits get the gates on the top qubits, in place.
-// The energy is read after one more pair pass that applies the last layer's
-// permutation.  Amplitudes are complex64 in FP32 arithmetic; energies
-// accumulate per thread in FP32 over a few terms and in FP64 beyond.
+// Two persistent launches: every CTA takes circuit ids from an atomic counter
+// (largest circuits first) until its part of the batch is done; there is no
+// waiting on other CTAs.  A circuit of n <= m qubits (m = 12..14, tuned) lives
+// in the CTA's shared memory (k_vqe_batch); a larger one lives in a per-CTA
+// global buffer and is processed in tiles of 2^13 amplitudes by window passes
+// (k_vqe_window; vqe_window.cuh says which gates a pass applies).  The energy's
+// X terms on the qubits above 12 are read in the last pass, the rest in one
+// more read of the state.  Amplitudes are complex64 in FP32 arithmetic;
+// energies accumulate per thread in FP32 over a few terms and in FP64 beyond.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -44,10 +34,10 @@
 
 #include "../../include/qsim.h"
 #include "common.cuh"
-#include "tc_common.cuh"
+#include "vqe_window.cuh"
 
 using namespace qsim_dev;
-using namespace qsim_tc;
+using namespace qsim_vqe;
 
 namespace {
 
@@ -65,7 +55,7 @@ struct VqeArgs {
     unsigned int *err;      // error flag (a bounded wait gave up)
     int begin, end;   // its circuits: order[begin..end)
     int m;            // qubits held in shared memory
-    float2 *gbuf;     // per-CTA global buffers (two of gstride amplitudes each)
+    float2 *gbuf;     // per-CTA global buffers of gstride amplitudes
     size_t gstride;
     double h;
 };
@@ -239,142 +229,45 @@ __device__ void build_phase_table(float2 *t, int kb, const float2 *ph, float2 ex
     }
 }
 
-// GLOBAL = false: circuits of n <= m qubits, each held in one CTA's shared
-// memory.  GLOBAL = true: larger circuits in per-CTA global buffers, two
-// CTAs per SM so that one CTA's loads, arithmetic and stores overlap the
-// other's (measured faster than one CTA of 512 threads per SM with
-// double-buffered copies: 44.9 against 41.0 ms for the 4096-circuit batch).
-// The global-memory kernel's chunk size (2^12 amplitudes; a pair of chunks
-// is 64 KB of shared memory) and block size.
-constexpr int kGlobalThreads = 128;
-constexpr int kGlobalCtas = 3;  // resident CTAs per SM the register budget is sized for
-constexpr int kGlobalBits = 12;
-
-// Position in a pair buffer (source order, after a ladder permutation) of
-// logical element e: bits 0..g-1 are gl = (e ^ e << 1) mod 2^g, bit g is
-// parity(gl) ^ (e >> g).  The map is linear over GF(2), so for the store's
-// elements e = tid ^ (j << 8) it is pair_perm(tid) ^ pair_perm(j << 8), the
-// second term a compile-time constant.
-__host__ __device__ constexpr unsigned pair_perm(unsigned e) {
-    const unsigned gl = (e ^ (e << 1)) & ((1u << kGlobalBits) - 1u);
-    unsigned par = 0;
-    for (int b = 0; b < kGlobalBits; ++b) par ^= (gl >> b) & 1u;
-    return ((par ^ (e >> kGlobalBits)) << kGlobalBits) | gl;
+// A qubit's part of a layer (see Rot): t, the phase p_q, its factor
+// s c' e^{-i (+-phi) / 2} of the layer's global factor, and its flip.
+struct QubitLayer {
+    float t;
+    float2 ph, f;
+    unsigned flip;
+};
+__device__ __forceinline__ QubitLayer qubit_layer(double theta, double phi) {
+    constexpr double kPi = 3.14159265358979323846;
+    const double hth = remainder(0.5 * theta, 2.0 * kPi);  // theta/2 (RY has period 4 pi)
+    const double j = rint(hth * (2.0 / kPi));               // -2..2
+    const int ji = (int)j;
+    float sh, ch, sp, cp, s2, c2;
+    sincosf((float)(hth - j * (0.5 * kPi)), &sh, &ch);
+    sincosf((float)remainder(phi, 2.0 * kPi), &sp, &cp);
+    sincosf((float)(0.5 * remainder(phi, 4.0 * kPi)), &s2, &c2);
+    QubitLayer r;
+    r.flip = (unsigned)ji & 1u;
+    const float sc = ((ji >> 1) & 1) ? -ch : ch;  // (-1)^floor(j/2) c'
+    r.t = sh / ch;
+    r.ph = r.flip ? make_float2(-cp, sp) : make_float2(cp, sp);
+    r.f = make_float2(sc * c2, r.flip ? sc * s2 : -sc * s2);
+    return r;
 }
 
-// Order of the pair pass's 12 rotations, taken four at a time, one of the
-// qubits 0..2 in each group (qubits 0..3 decide the shared-memory bank of
-// an 8-byte element; see pair_group for how the groups avoid conflicts).
-__constant__ int kPairOrder[12] = {0, 4, 5, 6, 1, 7, 8, 9, 2, 3, 10, 11};
-
-// One group of the pair pass with compile-time qubits Q0 < Q1 < Q2 < Q3 (a
-// group of kPairOrder): the 2^13-element pair buffer x holds 512 groups of
-// 16 elements, base (zeros at the pivots P0 < P1 < P2 < P3) XOR any subset
-// of the masks Mj = (PERM ? 3 : 1) << Qj; rotation j uses r[j].t.  PERM: the
-// buffer is in source order after a ladder permutation, where logical qubit
-// k pairs the elements p and p ^ (3 << k); either of those two bits can be
-// the pivot (Pj = Qj or Qj + 1; the masks restricted to the pivots must be
-// invertible); the element whose logical bit k is 0 is the one whose bits
-// 0..k have even parity, which for rotation j is the base's parity, so the
-// rotation is applied with t -> -t where that parity is odd.
-//
-// Banks.  In each access all lanes use the same subset of masks, so the 16
-// lanes of a half-warp (8-byte elements) hit 16 banks only if their bases
-// differ in all of bits 0..3.  A pivot there is 0 in every base; instead,
-// lanes whose group-index bit (4 - c + i) is set (c = number of pivots
-// below 4) start from base ^ M of the i-th such rotation: the same 16
-// elements in another order, which flips that pivot's bank bit, and that
-// rotation's pair is met with its two elements swapped (t -> -t in those
-// lanes).  The other rotations are unaffected: a mask changes the parity of
-// bits 0..q of no other rotation's base.
-template <bool PERM, int Q0, int Q1, int Q2, int Q3, int P0, int P1, int P2, int P3>
-__device__ __forceinline__ void pair_group(float2 *x, const Rot *r) {
-    static_assert(Q0 < Q1 && Q1 < Q2 && Q2 < Q3, "qubits in ascending order");
-    static_assert(P0 < P1 && P1 < P2 && P2 < P3, "pivots in ascending order");
-    constexpr unsigned W = PERM ? 3u : 1u;
-    constexpr unsigned M0 = W << Q0, M1 = W << Q1, M2 = W << Q2, M3 = W << Q3;
-    static_assert(((M0 >> P0) & 1u) && ((M1 >> P1) & 1u) && ((M2 >> P2) & 1u) && ((M3 >> P3) & 1u),
-                  "each pivot is a bit of its own mask");
-    // restricted to the pivots the masks form a triangular matrix
-    static_assert(!((M0 >> P1) & 1u) && !((M0 >> P2) & 1u) && !((M0 >> P3) & 1u) && !((M1 >> P2) & 1u) &&
-                      !((M1 >> P3) & 1u) && !((M2 >> P3) & 1u) ||
-                  (!((M1 >> P0) & 1u) && !((M2 >> P0) & 1u) && !((M3 >> P0) & 1u) && !((M2 >> P1) & 1u) &&
-                   !((M3 >> P1) & 1u) && !((M3 >> P2) & 1u)),
-                  "masks restricted to the pivots must be invertible");
-    constexpr int c = (P0 < 4) + (P1 < 4) + (P2 < 4) + (P3 < 4);  // pivots in the bank bits
-    static_assert(c <= 2 && (P0 < 4 || c == 0) && (P1 < 4 || c <= 1) && P2 >= 4 && P3 >= 4,
-                  "bank pivots come first");
-    const float t0 = r[0].t, t1 = r[1].t, t2 = r[2].t, t3 = r[3].t;
-    for (unsigned gi = threadIdx.x; gi < (1u << (kGlobalBits + 1 - 4)); gi += (unsigned)kGlobalThreads) {
-        unsigned base = gi;
-        base = ((base >> P0) << (P0 + 1)) | (base & ((1u << P0) - 1u));
-        base = ((base >> P1) << (P1 + 1)) | (base & ((1u << P1) - 1u));
-        base = ((base >> P2) << (P2 + 1)) | (base & ((1u << P2) - 1u));
-        base = ((base >> P3) << (P3 + 1)) | (base & ((1u << P3) - 1u));
-        // lane-dependent start of the bank-pivot rotations (see above)
-        const bool sw0 = c >= 1 && ((gi >> (4 - c)) & 1u);
-        const bool sw1 = c >= 2 && ((gi >> (5 - c)) & 1u);
-        const unsigned start = base ^ (sw0 ? M0 : 0u) ^ (sw1 ? M1 : 0u);
-        float2 v[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            v[k] = x[start ^ ((k & 1) ? M0 : 0u) ^ ((k & 2) ? M1 : 0u) ^ ((k & 4) ? M2 : 0u) ^ ((k & 8) ? M3 : 0u)];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int q = j == 0 ? Q0 : j == 1 ? Q1 : j == 2 ? Q2 : Q3;
-            float t = j == 0 ? t0 : j == 1 ? t1 : j == 2 ? t2 : t3;
-            if (PERM && (__popc(base & ((2u << q) - 1u)) & 1)) t = -t;
-            if ((j == 0 && sw0) || (j == 1 && sw1)) t = -t;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                if ((k >> j) & 1) continue;
-                const int k1 = k | (1 << j);
-                const float2 a = v[k], b = v[k1];
-                v[k] = make_float2(fmaf(-t, b.x, a.x), fmaf(-t, b.y, a.y));
-                v[k1] = make_float2(fmaf(t, a.x, b.x), fmaf(t, a.y, b.y));
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            x[start ^ ((k & 1) ? M0 : 0u) ^ ((k & 2) ? M1 : 0u) ^ ((k & 4) ? M2 : 0u) ^ ((k & 8) ? M3 : 0u)] = v[k];
-    }
-    __syncthreads();
-}
-
-// The pair pass's 12 rotations (r in kPairOrder) on a pair buffer.  Group
-// {2, 3, 10, 11} takes qubit 3's pivot at bit 4 when PERM allows it, so that
-// it has one pivot in the bank bits, like the other two groups.
-template <bool PERM>
-__device__ __forceinline__ void pair_gates(float2 *x, const Rot *r) {
-    pair_group<PERM, 0, 4, 5, 6, 0, 4, 5, 6>(x, r);
-    pair_group<PERM, 1, 7, 8, 9, 1, 7, 8, 9>(x, r + 4);
-    pair_group<PERM, 2, 3, 10, 11, 2, (PERM ? 4 : 3), 10, 11>(x, r + 8);
-}
-
-template <int T, bool GLOBAL>
-__global__ void __launch_bounds__(T, GLOBAL ? kGlobalCtas : 1) k_vqe_batch(const VqeArgs A) {
+// Circuits of n <= m qubits, each held in one CTA's shared memory.
+template <int T>
+__global__ void __launch_bounds__(T, 1) k_vqe_batch(const VqeArgs A) {
     constexpr int kRegAmps = RegAmps<T>::value;
     extern __shared__ float2 sm[];
     __shared__ int s_idx;
     __shared__ double s_red[32];
     __shared__ Rot s_rot[32];       // this layer's RY per qubit
-    __shared__ Rot s_rotp[32];      // the pair pass's rotations, in kPairOrder
     __shared__ float2 s_ph[32];     // e^{i phi_q}
     __shared__ unsigned s_mask[32]; // XOR mask of each rotation in the current pass
     __shared__ float2 s_tlo[128];   // phases of index bits 0..6 (times the global factor)
     __shared__ float2 s_thi[128];   // phases of the next bits of a chunk or register
     __shared__ float2 s_gph;        // the layer's global factor: prod_q s_q c'_q times e^{-i Phi'/2}
     __shared__ unsigned s_flip;     // the layer's flip mask F
-    __shared__ __align__(8) uint64_t s_bar[1];  // bulk-copy completion (global-memory path)
-    __shared__ uint32_t s_phase;
-    if (threadIdx.x == 0) {
-        if (GLOBAL) {
-            mbar_init(s_bar, 1);
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            s_phase = 0;
-        }
-    }
-    __syncthreads();
     // the layer's rotations t_q, per-qubit phases p_q, flip mask and global
     // factor (warp 0; n <= 32)
     auto layer_setup = [&](const double *al, int n) {
@@ -383,21 +276,11 @@ __global__ void __launch_bounds__(T, GLOBAL ? kGlobalCtas : 1) k_vqe_batch(const
             unsigned flip = 0;
             float2 f = make_float2(1.f, 0.f);
             if (q < (unsigned)n) {
-                constexpr double kPi = 3.14159265358979323846;
-                const double hth = remainder(0.5 * al[q], 2.0 * kPi);  // theta/2 (RY has period 4 pi)
-                const double j = rint(hth * (2.0 / kPi));                // -2..2
-                const int ji = (int)j;
-                float sh, ch;
-                sincosf((float)(hth - j * (0.5 * kPi)), &sh, &ch);
-                flip = (unsigned)ji & 1u;
-                const float sc = ((ji >> 1) & 1) ? -ch : ch;  // (-1)^floor(j/2) c'
-                const double phi = al[n + q];
-                float sp, cp, s2, c2;
-                sincosf((float)remainder(phi, 2.0 * kPi), &sp, &cp);
-                sincosf((float)(0.5 * remainder(phi, 4.0 * kPi)), &s2, &c2);
-                s_rot[q] = Rot{sh / ch};
-                s_ph[q] = flip ? make_float2(-cp, sp) : make_float2(cp, sp);
-                f = make_float2(sc * c2, flip ? sc * s2 : -sc * s2);
+                const QubitLayer r = qubit_layer(al[q], al[n + q]);
+                s_rot[q] = Rot{r.t};
+                s_ph[q] = r.ph;
+                flip = r.flip;
+                f = r.f;
             }
             const unsigned fl = __ballot_sync(0xffffffffu, flip);
 #pragma unroll
@@ -421,7 +304,7 @@ __global__ void __launch_bounds__(T, GLOBAL ? kGlobalCtas : 1) k_vqe_batch(const
         const double *ang = A.angles + A.aoff[c];
         const unsigned N = 1u << n;
         double zz = 0.0, xx = 0.0;
-        if constexpr (!GLOBAL) {
+        {
             // --- shared-memory resident circuit -------------------------------
             for (unsigned i = threadIdx.x; i < N; i += T) sm[i] = make_float2(i == 0 ? 1.f : 0.f, 0.f);
             __syncthreads();
@@ -455,210 +338,323 @@ __global__ void __launch_bounds__(T, GLOBAL ? kGlobalCtas : 1) k_vqe_batch(const
             }
             zz = (double)zz_chunk(sm, n, 0ull, n);
             for (int q = 0; q < n; ++q) xx += (double)x_chunk(sm, n, q);
-        } else {
-            // --- global-memory circuit, chunks of 2^g ----------------------------
-            // Data arrive by bulk copies completing on an mbarrier (no
-            // register staging): a pair pass copies the two source chunks
-            // whole and works on them in source order, where logical qubit
-            // k < g pairs the elements p and p ^ (3 << k); the store reads
-            // each destination element at its source position.  Every wait
-            // is bounded; on time-out the CTA raises the error flag and
-            // stops.
-            constexpr int g = kGlobalBits;
-            // the top-qubit pass takes tiles of the whole pair buffer, 2^(g+1)
-            // amplitudes: 2^h runs of 2^lowrun (h >= 1, lowrun >= 1 for n <= 2g)
-            const int h = n - g, lowrun = g + 1 - h;
-            float2 *src = A.gbuf + (size_t)blockIdx.x * 2 * A.gstride;
-            float2 *dst = src + A.gstride;
-            const unsigned G = 1u << g, nchunks = 1u << h, hmask = nchunks - 1u, gmask = G - 1u;
-            const unsigned run_bytes = 8u << lowrun;  // a high-pass tile is 2^h runs of 2^lowrun amplitudes
-            const unsigned ntiles = nchunks / 2, GT = 2u * G;
-            float2 *const s_ttop = sm + ((size_t)2 << g);  // phases of the top h qubits, after the pair buffer
-            for (unsigned i = threadIdx.x; i < N; i += T) src[i] = make_float2(i == 0 ? 1.f : 0.f, 0.f);
-            __syncthreads();
-            bool permuted = false;  // src holds the state before a pending ladder permutation
-            bool failed = false;
-            // wait for the current copy phase; the result is uniform over the CTA
-            auto wait_copies = [&]() {
-                bool ok = mbar_wait(s_bar, s_phase);
-                if (!ok) ok = mbar_wait(s_bar, s_phase);  // give copies in flight a second bound
-                __syncthreads();
-                if (threadIdx.x == 0) s_phase ^= 1u;
-                if (__syncthreads_or(!ok)) {
-                    if (threadIdx.x == 0) atomicOr(A.err, 1u);
-                    return false;
-                }
-                return true;
-            };
-            // chunks pr and pr ^ hmask (through the pending permutation: the
-            // source chunks S and S ^ 1, S = pr ^ (pr << 1)) into sm[0..2G)
-            // every thread orders its generic stores to global memory and its
-            // shared-memory accesses before the bulk copies that follow
-            auto before_copies = [&]() {
-                fence_proxy_async_global();
-                fence_proxy_async_smem();
-                __syncthreads();
-            };
-            // the two source chunks of destination pair pr
-            auto pair_chunks = [&](unsigned pr, unsigned &ca, unsigned &cb) {
-                const unsigned S = permuted ? ((pr ^ (pr << 1)) & hmask) : pr;
-                ca = S;
-                cb = permuted ? S ^ 1u : pr ^ hmask;
-            };
-            // (Bringing the next pair's or tile's data into L2 once a copy
-            // had landed, with cp.async.bulk.prefetch.L2, measured 4 %
-            // slower: 6.5 % more DRAM reads.)
-            auto load_pair = [&](const float2 *from, unsigned pr) {
-                unsigned ca, cb;
-                pair_chunks(pr, ca, cb);
-                before_copies();
-                if (threadIdx.x == 0) {
-                    mbar_expect_tx(s_bar, 16u * G);
-                    bulk_copy(sm, from + ((size_t)ca << g), 8u * G, s_bar);
-                    bulk_copy(sm + G, from + ((size_t)cb << g), 8u * G, s_bar);
-                }
-                return wait_copies();
-            };
-            // physical position in the pair buffer of logical element e
-            // (e < G: chunk pr, else chunk pr ^ hmask; offset e & gmask)
-            auto pair_pos = [&](unsigned e) {
-                if (!permuted) return e;
-                const unsigned gl = ((e ^ (e << 1)) & gmask);
-                return ((((unsigned)__popc(gl) & 1u) ^ (e >> g)) << g) | gl;
-            };
-            // Destination chunks pr (logical elements e < G) and pr ^ hmask,
-            // written whole: this thread's elements are e = tid + j T, each
-            // read at pair_pos(e ^ flo) (linear: a per-thread part and a
-            // compile-time part); phased: the layer's phases of qubits
-            // 0..g-1 and flips (flo), the low seven phase bits constant per
-            // thread.
-            auto store_pair = [&](float2 *to, unsigned pr, bool phased, unsigned flo) {
-                static_assert(T == kGlobalThreads && T >= 128 && (2 << g) % T == 0,
-                              "store_pair: the thread index holds bits 0..6 of the element");
-                const unsigned tf = threadIdx.x ^ flo;
-                const unsigned pt = permuted ? pair_perm(tf) : tf;
-                float2 *dst0 = to + ((size_t)pr << g) + threadIdx.x;
-                float2 *dst1 = to + ((size_t)(pr ^ hmask) << g) + threadIdx.x;
-                const float2 tlo = s_tlo[tf & 127u];
-                const unsigned thi0 = (tf >> 7) & 31u;
-#pragma unroll
-                for (int j = 0; j < (2 << g) / T; ++j) {
-                    const unsigned cj = (unsigned)j * (unsigned)T;  // e = tid | j T
-                    float2 v = sm[pt ^ (permuted ? pair_perm(cj) : cj)];
-                    if (phased) v = cmul(v, cmul(tlo, s_thi[thi0 ^ ((cj >> 7) & 31u)]));
-                    ((j < G / T) ? dst0 : dst1)[cj & gmask] = v;
-                }
-                __syncthreads();
-            };
-            auto tile_index = [&](unsigned t, unsigned e) {
-                const unsigned lo = e & ((1u << lowrun) - 1u), top = e >> lowrun;
-                return lo | (t << lowrun) | (top << g);
-            };
-            // tile t: run `top` (2^lowrun amplitudes at t << lowrun | top << g)
-            // to sm[top << lowrun]
-            auto load_tile = [&](const float2 *from, unsigned t) {
-                if (run_bytes < 16) {  // runs below the bulk-copy granule: plain loads
-                    for (unsigned e = threadIdx.x; e < GT; e += T) sm[e] = from[tile_index(t, e)];
-                    __syncthreads();
-                    return true;
-                }
-                before_copies();
-                if (threadIdx.x == 0) mbar_expect_tx(s_bar, 8u * GT);
-                __syncthreads();
-                for (unsigned top = threadIdx.x; top < nchunks; top += T) {
-                    bulk_copy(sm + (top << lowrun), from + ((size_t)t << lowrun) + ((size_t)top << g), run_bytes,
-                              s_bar);
-                }
-                return wait_copies();
-            };
-            for (int l = 0; l < L && !failed; ++l) {
-                const double *al = ang + 2 * l * n;
-                layer_setup(al, n);
-                build_phase_table(s_tlo, 7, s_ph, s_gph);
-                build_phase_table(s_thi, g - 7, s_ph + 7, make_float2(1.f, 0.f));
-                build_phase_table(s_ttop, h, s_ph + g, make_float2(1.f, 0.f));
-                // the pair pass's rotations in kPairOrder; the top-qubit
-                // pass's masks (tile bits lowrun..g)
-                if (threadIdx.x < (unsigned)g) s_rotp[threadIdx.x] = s_rot[kPairOrder[threadIdx.x]];
-                if (threadIdx.x < (unsigned)h) s_mask[g + threadIdx.x] = 1u << (lowrun + threadIdx.x);
-                __syncthreads();
-                // pair pass: src (through the pending permutation) -> dst, RY
-                // on qubits 0..g-1 over both chunks at once, their RZ phases
-                // on the way out
-                for (unsigned pr = 0; pr < nchunks / 2 && !failed; ++pr) {
-                    if (!load_pair(src, pr)) {
-                        failed = true;
-                        break;
-                    }
-                    if (permuted)
-                        pair_gates<true>(sm, s_rotp);
-                    else
-                        pair_gates<false>(sm, s_rotp);
-                    store_pair(dst, pr, true, s_flip & gmask);
-                }
-                // high pass on dst, in place: RY on the top qubits, then
-                // their RZ phases on the way out
-                for (unsigned t = 0; t < ntiles && !failed; ++t) {
-                    if (!load_tile(dst, t)) {
-                        failed = true;
-                        break;
-                    }
-                    gates_blocked(sm, g + 1, s_mask + g, s_rot + g, h);
-                    const unsigned fhi = s_flip >> g;  // flips of the top qubits
-                    for (unsigned e = threadIdx.x; e < GT; e += T) {
-                        const unsigned ef = e ^ (fhi << lowrun);
-                        dst[tile_index(t, e)] = cmul(sm[ef], s_ttop[ef >> lowrun]);
-                    }
-                    __syncthreads();
-                }
-                float2 *tmp = src;
-                src = dst;
-                dst = tmp;
-                permuted = true;  // this layer's CNOT ladder is still to be applied
-            }
-            // the last permutation, with the ZZ terms and the X terms of
-            // qubits 0..g-1 read on the way; then the top qubits' X terms
-            float zf = 0.f, xf = 0.f;
-            for (unsigned pr = 0; pr < nchunks / 2 && !failed; ++pr) {
-                if (!load_pair(src, pr)) {
-                    failed = true;
-                    break;
-                }
-                const unsigned hb = pr ^ hmask;
-                for (unsigned e = threadIdx.x; e < 2 * G; e += T) {
-                    const unsigned long long gi = ((unsigned long long)(e < G ? pr : hb) << g) | (e & gmask);
-                    const float w = norm2(sm[pair_pos(e)]);
-                    zf += w * (float)((n - 1) - 2 * __popcll((gi ^ (gi >> 1)) & ((1ull << (n - 1)) - 1ull)));
-                }
-                for (int q = 0; q < g; ++q) {
-                    // logical pairs (e, e ^ 2^q) are the buffer pairs (p, p ^ (3 << q))
-                    // (single bits if no layer ran: the buffer is in logical order);
-                    // Re(conj(a) b) does not depend on which of the two is which
-                    const unsigned msk = (permuted ? 3u : 1u) << q, low = (1u << q) - 1u;
-                    for (unsigned u = threadIdx.x; u < G; u += T) {
-                        const unsigned p0 = ((u & ~low) << 1) | (u & low);
-                        const float2 a = sm[p0], b = sm[p0 ^ msk];
-                        xf += 2.f * (a.x * b.x + a.y * b.y);
-                    }
-                }
-                store_pair(dst, pr, false, 0u);
-            }
-            for (unsigned t = 0; t < ntiles && !failed; ++t) {
-                if (!load_tile(dst, t)) {
-                    failed = true;
-                    break;
-                }
-                for (int q = g; q < n; ++q) xf += x_chunk(sm, g + 1, lowrun + (q - g));
-                __syncthreads();
-            }
-            zz = (double)zf;
-            xx = (double)xf;
-            if (failed) break;  // the error flag is set; this CTA stops
         }
         const double zzs = block_sum_d(zz, s_red);
         const double xxs = block_sum_d(xx, s_red);
         if (threadIdx.x == 0) A.energies[c] = -zzs - A.h * xxs;
         __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// larger circuits: window passes over a state in global memory
+// ---------------------------------------------------------------------------
+// A CTA of 256 threads takes a circuit.  Per pass it works out the gates
+// (thread 0), their rotations and phase tables and the groups (a thread each),
+// then for every tile: asynchronous 16-byte copies in (zeros where the state
+// is still zero), the steps, and 16-byte stores in logical order.  A step's
+// rotations go five at a time on 32 amplitudes in registers, one start of the
+// group per thread, the lanes on different banks (vqe_window.cuh); the last
+// group of a step multiplies in the step's RZ phases, one factor per amplitude
+// from two tables.  Two CTAs per SM.
+// (Before: a pair pass and a top-qubit pass over the whole state per layer:
+// the 3009 circuits of 13..20 qubits of the 4096-circuit batch MEASURED_V0;
+// now MEASURED_V1.)
+constexpr int kWinThreads = 256;
+constexpr int kWinCtas = 2;
+constexpr int kTile = 1 << kTileBits;
+static_assert(kWinThreads == 1 << (kTileBits - kGroupBits), "one start of a group per thread");
+
+struct WinShared {
+    Progress prog;
+    Pass pass;
+    Map map[kMaxSteps];      // before each step
+    Map end;                 // after the last
+    Group group[kMaxGroups];
+    float t[kMaxGroups][kGroupBits];
+    float ts[kMaxSteps][kTileBits];
+    float2 ph[kMaxSteps][kTileBits], f[kMaxSteps][kTileBits];
+    unsigned flip[kMaxSteps];
+    float2 tlo[kMaxSteps][128], thi[kMaxSteps][64];
+    Group xgroup[3];         // X terms
+    int nx;
+};
+
+// One group on the tile: each thread's 32 amplitudes, position start ^ sums of
+// the masks, logical index y ^ the corresponding bits.
+template <class F>
+__device__ __forceinline__ void with_group(float2 *x, const Group &G, bool store, F f) {
+    const unsigned sy = G.lane[threadIdx.x & 31] ^ G.hi[threadIdx.x >> 5];
+    unsigned m[kGroupBits];
+#pragma unroll
+    for (int j = 0; j < kGroupBits; ++j) m[j] = G.m[j];
+    float2 v[1 << kGroupBits];
+    unsigned p = sy & 0xFFFFu;
+#pragma unroll
+    for (int k = 0; k < (1 << kGroupBits); ++k) {
+        const int g = k ^ (k >> 1);
+        if (k) {
+            const int b = (k & 1) ? 0 : (k & 2) ? 1 : (k & 4) ? 2 : (k & 8) ? 3 : 4;
+            p ^= m[b];
+        }
+        v[g] = x[p];
+    }
+    f(v, sy >> 16);
+    if (!store) return;
+    p = sy & 0xFFFFu;
+#pragma unroll
+    for (int k = 0; k < (1 << kGroupBits); ++k) {
+        const int g = k ^ (k >> 1);
+        if (k) {
+            const int b = (k & 1) ? 0 : (k & 2) ? 1 : (k & 4) ? 2 : (k & 8) ? 3 : 4;
+            p ^= m[b];
+        }
+        x[p] = v[g];
+    }
+}
+
+// The groups of X terms on the tile bits of `bits`, under the map a (threads 0..2).
+__device__ __forceinline__ void x_groups(WinShared &S, const Map &a, unsigned bits) {
+    const int c = __popc(bits), ng = (c + kGroupBits - 1) / kGroupBits;
+    if (threadIdx.x == 0) S.nx = ng;
+    if ((int)threadIdx.x < ng) {
+        int q[kGroupBits], k = 0, i = 0;
+        for (int t = 0; t < kTileBits; ++t)
+            if ((bits >> t) & 1u) {
+                if (i % ng == (int)threadIdx.x) q[k++] = t;
+                ++i;
+            }
+        make_group(a, q, k, S.xgroup[threadIdx.x]);
+    }
+    __syncthreads();
+}
+// sum over the groups' X terms of 2 Re(conj(a) b) over the pairs
+__device__ __forceinline__ float x_terms(float2 *x, const WinShared &S) {
+    float acc = 0.f;
+    for (int g = 0; g < S.nx; ++g) {
+        const int cnt = S.xgroup[g].cnt;
+        with_group(x, S.xgroup[g], false, [&](float2(&v)[32], unsigned) {
+#pragma unroll
+            for (int j = 0; j < kGroupBits; ++j) {
+                if (j >= cnt) continue;
+                float s = 0.f;
+#pragma unroll
+                for (int k = 0; k < 32; ++k)
+                    if (!((k >> j) & 1)) s = fmaf(v[k].x, v[k | (1 << j)].x, fmaf(v[k].y, v[k | (1 << j)].y, s));
+                acc = fmaf(2.f, s, acc);
+            }
+        });
+    }
+    return acc;
+}
+
+__global__ void __launch_bounds__(kWinThreads, kWinCtas) k_vqe_window(const VqeArgs A) {
+    extern __shared__ __align__(16) float2 x[];  // the tile
+    __shared__ WinShared S;
+    __shared__ int s_idx;
+    __shared__ double s_red[32];
+    const unsigned tid = threadIdx.x;
+    float2 *const buf = A.gbuf + (size_t)blockIdx.x * A.gstride;
+    // address of unit u (amplitudes 2u, 2u + 1 of the tile) of tile t
+    auto tile_fixed = [](unsigned t, int w) {
+        return ((t & ((1u << (w - kRunBits)) - 1u)) << kRunBits) | ((t >> (w - kRunBits)) << (w + kWindow));
+    };
+    auto unit_addr = [](unsigned u, int w) { return ((u & 1u) << 1) | ((u >> 1) << w); };
+    constexpr unsigned kUnits = kTile / 2 / kWinThreads;  // 16 per thread
+    auto load = [&](unsigned fixed, int w, int nz) {
+#pragma unroll 4
+        for (unsigned i = 0; i < kUnits; ++i) {
+            const unsigned u = tid + i * kWinThreads, at = fixed | unit_addr(u, w);
+            if (at >> nz)
+                *(float4 *)(x + 2 * u) = make_float4(0.f, 0.f, 0.f, 0.f);
+            else
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                 (uint32_t)__cvta_generic_to_shared(x + 2 * u)),
+                             "l"(buf + at)
+                             : "memory");
+        }
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+    };
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) s_idx = A.begin + (int)atomicAdd(A.counter, 1u);
+        __syncthreads();
+        const int idx = s_idx;
+        if (idx >= A.end) break;
+        const int c = A.order[idx];
+        const int n = A.nq[c], L = A.nl[c];
+        const double *ang = A.angles + A.aoff[c];
+        if (L == 0) {  // |0...0>
+            if (tid == 0) A.energies[c] = -(double)(n - 1);
+            continue;
+        }
+        if (tid == 0) {
+            progress_start(S.prog, n, L);
+            buf[0] = make_float2(1.f, 0.f);
+            buf[1] = make_float2(0.f, 0.f);
+        }
+        int nz = 1;  // the state is zero from index 2^nz on
+        double xx = 0.0, zz = 0.0;
+        for (bool last = false; !last;) {
+            __syncthreads();
+            if (tid == 0) make_pass(S.prog, window_start(S.prog), S.pass);
+            __syncthreads();
+            const int w = S.pass.w, ns = S.pass.nsteps;
+            last = lowest_ready(S.prog) >= n;
+            if (ns == 0 && S.pass.cn0 == 0) {  // cannot happen: every window holds a ready gate
+                if (tid == 0) atomicOr(A.err, 1u);
+                break;
+            }
+            // rotations of every step
+            if (tid < kMaxSteps) S.flip[tid] = 0;
+            __syncthreads();
+            for (int i = tid; i < ns * kTileBits; i += kWinThreads) {
+                const int st = i / kTileBits, t = i - st * kTileBits;
+                if (!((S.pass.step[st].rot >> t) & 1u)) continue;
+                const int q = t < kRunBits ? t : w + t - kRunBits, l = S.pass.step[st].layer[t];
+                const QubitLayer r = qubit_layer(ang[2 * l * n + q], ang[2 * l * n + n + q]);
+                S.ts[st][t] = r.t;
+                S.ph[st][t] = r.ph;
+                S.f[st][t] = r.f;
+                if (r.flip) atomicOr(&S.flip[st], 1u << t);
+            }
+            __syncthreads();
+            if (tid == 0) {
+                Map M;
+                map_identity(M);
+                auto sweep = [&](unsigned cn) {
+                    for (int t = 0; t + 1 < kTileBits; ++t)
+                        if ((cn >> t) & 1u) map_cnot(M, t, t + 1);
+                };
+                sweep(S.pass.cn0);
+                for (int st = 0; st < ns; ++st) {
+                    S.map[st] = M;
+                    M.f ^= S.flip[st];
+                    sweep(S.pass.step[st].cn);
+                }
+                S.end = M;
+            }
+            // phase tables: index bits 0..6 (times the step's factor) and 7..12
+            for (int i = tid; i < ns * 192; i += kWinThreads) {
+                const int st = i / 192, e = i - st * 192;
+                const unsigned rot = S.pass.step[st].rot;
+                float2 z = make_float2(1.f, 0.f);
+                if (e < 128) {
+                    for (int t = 0; t < kTileBits; ++t)
+                        if ((rot >> t) & 1u) z = cmul(z, S.f[st][t]);
+                    for (int t = 0; t < 7; ++t)
+                        if (((rot & (unsigned)e) >> t) & 1u) z = cmul(z, S.ph[st][t]);
+                    S.tlo[st][e] = z;
+                } else {
+                    for (int t = 7; t < kTileBits; ++t)
+                        if ((rot >> t) & ((unsigned)(e - 128) >> (t - 7)) & 1u) z = cmul(z, S.ph[st][t]);
+                    S.thi[st][e - 128] = z;
+                }
+            }
+            __syncthreads();
+            if (tid < kMaxGroups) {
+                for (int st = 0; st < ns; ++st) {
+                    const Step &P = S.pass.step[st];
+                    if ((int)tid < P.g0 || (int)tid >= P.g1) continue;
+                    const int ng = P.g1 - P.g0, g = (int)tid - P.g0;
+                    int q[kGroupBits], k = 0, i = 0;
+                    for (int t = 0; t < kTileBits; ++t)
+                        if ((P.rot >> t) & 1u) {
+                            if (i % ng == g) {
+                                S.t[tid][k] = S.ts[st][t];
+                                q[k++] = t;
+                            }
+                            ++i;
+                        }
+                    make_group(S.map[st], q, k, S.group[tid]);
+                }
+            }
+            __syncthreads();
+            // the X terms on qubits 13 and above: the last window holds them
+            unsigned xbits = 0;
+            if (last)
+                for (int t = kRunBits; t < kTileBits; ++t)
+                    if (w + t - kRunBits >= kTileBits && w + t - kRunBits < n) xbits |= 1u << t;
+            if (xbits) x_groups(S, S.end, xbits);
+            const int reach = w + kWindow < n ? w + kWindow : n;
+            const int nz_out = reach > nz ? reach : nz;
+            // where this thread's stores find their amplitudes
+            const unsigned p_tid = map_position(S.end, 2 * tid), p_one = S.end.inv[0];
+            const unsigned tiles = 1u << (nz_out - kTileBits);
+            for (unsigned t = 0; t < tiles; ++t) {
+                const unsigned fixed = tile_fixed(t, w);
+                load(fixed, w, nz);
+                for (int st = 0; st < ns; ++st) {
+                    const int g1 = S.pass.step[st].g1;
+                    for (int g = S.pass.step[st].g0; g < g1; ++g) {
+                        const Group &G = S.group[g];
+                        const bool phases = g == g1 - 1;
+                        with_group(x, G, true, [&](float2(&v)[32], unsigned y) {
+                            const int cnt = G.cnt;
+#pragma unroll
+                            for (int j = 0; j < kGroupBits; ++j) {
+                                if (j >= cnt) continue;
+                                float r = S.t[g][j];
+                                if ((y >> G.q[j]) & 1u) r = -r;
+#pragma unroll
+                                for (int k = 0; k < 32; ++k) {
+                                    if ((k >> j) & 1) continue;
+                                    const float2 a = v[k], b = v[k | (1 << j)];
+                                    v[k] = make_float2(fmaf(-r, b.x, a.x), fmaf(-r, b.y, a.y));
+                                    v[k | (1 << j)] = make_float2(fmaf(r, a.x, b.x), fmaf(r, a.y, b.y));
+                                }
+                            }
+                            if (phases) {
+#pragma unroll
+                                for (int k = 0; k < 32; ++k) {
+                                    const int gk = k ^ (k >> 1);
+                                    if (k) {
+                                        const int b = (k & 1) ? 0 : (k & 2) ? 1 : (k & 4) ? 2 : (k & 8) ? 3 : 4;
+                                        y ^= 1u << G.q[b];
+                                    }
+                                    v[gk] = cmul(v[gk], cmul(S.tlo[st][y & 127u], S.thi[st][y >> 7]));
+                                }
+                            }
+                        });
+                        __syncthreads();
+                    }
+                }
+                if (xbits) xx += (double)x_terms(x, S);
+#pragma unroll 4
+                for (unsigned i = 0; i < kUnits; ++i) {
+                    // unit tid + 256 i: index bits 9..12 are i's
+                    unsigned p = p_tid;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        if ((i >> b) & 1u) p ^= S.end.inv[9 + b];
+                    const float2 a = x[p], b = x[p ^ p_one];
+                    *(float4 *)(buf + (fixed | unit_addr(tid + i * kWinThreads, w))) = make_float4(a.x, a.y, b.x, b.y);
+                }
+                __syncthreads();
+            }
+            nz = nz_out;
+        }
+        // ZZ of all qubits and X of the 13 lowest
+        if (tid == 0) map_identity(S.end);
+        __syncthreads();
+        x_groups(S, S.end, n < kTileBits ? (1u << n) - 1u : (unsigned)kTile - 1u);
+        const unsigned m1 = (1u << (n - 1)) - 1u;
+        for (unsigned t = 0; t < (1u << (n - kTileBits)); ++t) {
+            load(t << kTileBits, kRunBits, n);
+            float zf = 0.f;
+            for (unsigned i = 0; i < kTile / kWinThreads; ++i) {
+                const unsigned e = tid + i * kWinThreads, gi = (t << kTileBits) | e;
+                zf = fmaf(norm2(x[e]), (float)((n - 1) - 2 * __popc((gi ^ (gi >> 1)) & m1)), zf);
+            }
+            const float xf = x_terms(x, S);
+            zz += (double)zf;
+            xx += (double)xf;
+            __syncthreads();
+        }
+        const double zzs = block_sum_d(zz, s_red);
+        const double xxs = block_sum_d(xx, s_red);
+        if (tid == 0) A.energies[c] = -zzs - A.h * xxs;
     }
 }
 
@@ -705,21 +701,13 @@ int reg_amps(int threads) { return threads == 256 ? RegAmps<256>::value : thread
 
 typedef void (*VqeKernel)(const VqeArgs);
 VqeKernel kernel_for(int threads) {
-    return threads == 256 ? k_vqe_batch<256, false> : threads == 512 ? k_vqe_batch<512, false>
-                                                                     : k_vqe_batch<1024, false>;
+    return threads == 256 ? k_vqe_batch<256> : threads == 512 ? k_vqe_batch<512> : k_vqe_batch<1024>;
 }
 
-// The global-memory kernel: 256 threads, chunks of 2^12 amplitudes (a pair
-// of them is 64 KB of shared memory, followed by the phase table of the top
-// n - 12 qubits, 2 KB for n = 20, 32 KB for n = 24), two CTAs per SM
-// (measured faster than three, which force the registers down to 80 and
-// spill).
-static_assert(kGlobalBits == 12, "kPairOrder lists the 12 chunk qubits");
-constexpr int kMaxBatchQubits = 2 * kGlobalBits;  // n <= 2 g: a tile's runs are whole amplitudes
-size_t global_smem(int nmax) {
-    return ((size_t)16 << kGlobalBits) + ((size_t)8 << std::max(nmax - kGlobalBits, 0));
-}
-static_assert(kGlobalBits % 4 == 0, "pair-pass rotation groups must not need identity padding");
+// the top window and the 13 lowest qubits cover all qubits
+constexpr int kMaxBatchQubits = kTileBits + kWindow;
+static_assert(kMaxBatchQubits == 24 && kMaxBatchQubits <= kMaxQ, "the range the interface states");
+constexpr size_t kWinSmem = (size_t)8 << kTileBits;
 
 // circuits with more than m qubits: a prefix of the order (sorted by size)
 int count_large(const qsim_batch *b, int m) {
@@ -734,12 +722,11 @@ bool config_valid(const qsim_batch *b, int threads, int m) {
 }
 
 int occupancy_global(const qsim_batch *b, int *grid) {
-    VqeKernel k = k_vqe_batch<kGlobalThreads, true>;
-    const size_t smem = global_smem(b->nmax);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    VqeKernel k = k_vqe_window;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWinSmem);
     if (e != cudaSuccess) return QSIM_ECUDA;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kGlobalThreads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWinThreads, kWinSmem);
     if (e != cudaSuccess || per_sm < 1) return QSIM_ENOTSUP;
     *grid = std::min(b->sms * per_sm, b->max_grid);
     return QSIM_OK;
@@ -787,7 +774,7 @@ int launch(qsim_batch *b, int threads, int m, int grid) {
         a.counter = b->d_counter;
         a.begin = 0;
         a.end = large;
-        k_vqe_batch<kGlobalThreads, true><<<ggrid, kGlobalThreads, global_smem(b->nmax), b->stream>>>(a);
+        k_vqe_window<<<ggrid, kWinThreads, kWinSmem, b->stream>>>(a);
         e = cudaGetLastError();
         if (e != cudaSuccess) return berr(b, QSIM_ECUDA, cudaGetErrorString(e));
     }
@@ -852,7 +839,7 @@ int sim_batch_workspace_bytes(int count, const int *nqubits, const int *layers, 
     const size_t max_grid = (size_t)sms * 4;
     const size_t gstride = nmax > 12 ? ((size_t)1 << nmax) : 0;
     size_t s = align256(sizeof(double) * nang) + align256(sizeof(double) * count) + 3 * align256(sizeof(int) * count) +
-               align256(sizeof(long long) * count) + 256 + max_grid * 2 * gstride * sizeof(float2);
+               align256(sizeof(long long) * count) + 256 + max_grid * gstride * sizeof(float2);
     *bytes = s;
     return QSIM_OK;
 }
@@ -990,7 +977,7 @@ int sim_batch_run(qsim_batch *b, const double *angles, double *energies) {
     cudaError_t e = cudaGraphLaunch(b->graph, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return berr(b, QSIM_ECUDA, cudaGetErrorString(e));
-    if (*b->h_flag) return berr(b, QSIM_ETIMEOUT, "a bounded wait for bulk copies gave up; energies not computed");
+    if (*b->h_flag) return berr(b, QSIM_ETIMEOUT, "a device loop gave up; energies not computed");
     std::memcpy(energies, b->h_energies, sizeof(double) * b->count);
     return QSIM_OK;
 }
