@@ -388,8 +388,8 @@ int sim_batch_create(int count, const int *nqubits, const int *layers, double h,
  * layer, n RY angles (qubit 0..n-1) then n RZ angles; energies (host):
  * count doubles.  The first call captures the graph (angles H2D, queue and
  * error-flag reset, the two persistent kernels, energies and flag D2H);
- * later calls replay it.  QSIM_ETIMEOUT if a bounded device wait gave up
- * (energies then not written). */
+ * later calls replay it.  QSIM_ETIMEOUT if a device loop gave up (energies
+ * then not written). */
 int sim_batch_run(qsim_batch *b, const double *angles, double *energies);
 
 /* Batched sweep (not in the paper).  Time every candidate launch configuration (threads per CTA 256/512/1024,
@@ -401,8 +401,8 @@ int sim_batch_autotune(qsim_batch *b, const double *angles, int reps, int *threa
  * small-circuit kernel by hand
  * (QSIM_EINVAL if it cannot run: 2^m must be <= 32 * threads for 256 and
  * 512 threads, <= 16 * 1024 for 1024); circuits with more than m qubits go
- * to the global-memory kernel (256 threads, two CTAs per SM, 2^12-amplitude
- * chunks). */
+ * to the global-memory kernel (256 threads, two CTAs per SM, tiles of 2^13
+ * amplitudes).  Before a call to this or to sim_batch_autotune: 256, 12. */
 int sim_batch_set_config(qsim_batch *b, int threads, int m);
 
 /* Batched sweep (not in the paper): destroy a batch; the last failure's

@@ -12,9 +12,9 @@
 // ladder is one permutation: applied in order it maps |b> to |b'> with
 // b'_k = b_0 ^ ... ^ b_k, i.e. psi'[y] = psi[y ^ (y << 1) mod 2^n].
 //
-// Two persistent launches: every CTA takes circuit ids from an atomic counter
-// (largest circuits first) until its part of the batch is done; there is no
-// waiting on other CTAs.  A circuit of n <= m qubits (m = 12..14, tuned) lives
+// Two persistent launches: every CTA, or cluster of CTAs, takes circuit ids
+// from an atomic counter (largest circuits first) until its part of the batch
+// is done; no CTA waits for one outside its cluster.  A circuit of n <= m qubits (m = 12..14, tuned) lives
 // in the CTA's shared memory (k_vqe_batch); a larger one lives in a per-CTA
 // global buffer and is processed in tiles of 2^13 amplitudes by window passes
 // (k_vqe_window; vqe_window.cuh says which gates a pass applies).  The energy's
@@ -51,9 +51,10 @@ struct VqeArgs {
     const long long *aoff;
     const double *angles;
     double *energies;
-    unsigned int *counter;  // this launch's queue
+    unsigned int *counter;  // this launch's queue (k_vqe_window: the clusters', then the CTAs')
     unsigned int *err;      // error flag (a bounded wait gave up)
     int begin, end;   // its circuits: order[begin..end)
+    int split;        // k_vqe_window: order[begin..split) by clusters
     int m;            // qubits held in shared memory
     float2 *gbuf;     // per-CTA global buffers of gstride amplitudes
     size_t gstride;
@@ -356,10 +357,17 @@ __global__ void __launch_bounds__(T, 1) k_vqe_batch(const VqeArgs A) {
 // rotations go five at a time on 32 amplitudes in registers, one start of the
 // group per thread, the lanes on different banks (vqe_window.cuh); the last
 // group of a step multiplies in the step's RZ phases, one factor per amplitude
-// from two tables.  Two CTAs per SM.
+// from two tables.  Two CTAs per SM (registers); on a full chip issue slots and
+// shared memory are both half busy, between barriers, DRAM at 2 TB/s.
 // (Before: a pair pass and a top-qubit pass over the whole state per layer:
-// the 3009 circuits of 13..20 qubits of the 4096-circuit batch MEASURED_V0;
-// now MEASURED_V1.)
+// 4096 circuits of 10..20 qubits 26.3 ms, now 16.7.)
+//
+// Where few circuits hold much of the work, a circuit is shared by a cluster
+// (Joint): each CTA works out the passes for itself and takes every csize-th
+// tile, a cluster barrier between passes, the energy's parts added in the order
+// of the ranks.  One CTA per circuit left most of the chip idle at the end (a
+// circuit of 20 qubits and 8 layers alone 7.7 ms; by 8 CTAs 1.33).  When the
+// clusters' circuits are done each CTA goes on alone with the smaller ones.
 constexpr int kWinThreads = 256;
 constexpr int kWinCtas = 2;
 constexpr int kTile = 1 << kTileBits;
@@ -448,13 +456,39 @@ __device__ __forceinline__ float x_terms(float2 *x, const WinShared &S) {
     return acc;
 }
 
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// 64 bits of another CTA's shared memory, where this CTA has `p`
+__device__ __forceinline__ unsigned long long peer_u64(const void *p, unsigned rank) {
+    uint32_t a;
+    unsigned long long v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+
+template <bool Joint>
 __global__ void __launch_bounds__(kWinThreads, kWinCtas) k_vqe_window(const VqeArgs A) {
     extern __shared__ __align__(16) float2 x[];  // the tile
     __shared__ WinShared S;
-    __shared__ int s_idx;
+    __shared__ unsigned long long s_idx;
     __shared__ double s_red[32];
+    __shared__ double s_part[2];  // this CTA's part of a cluster's energy
     const unsigned tid = threadIdx.x;
-    float2 *const buf = A.gbuf + (size_t)blockIdx.x * A.gstride;
+    unsigned rank = 0, csize = 1;  // 0 of 1 too once the clusters' circuits are done
+    if (Joint) {
+        asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(csize));
+    }
+    float2 *buf = A.gbuf + (size_t)(blockIdx.x - rank) * A.gstride;  // a cluster's: its first CTA's
+    // every thread of the circuit's CTAs; what they wrote is visible after it
+    auto sync = [&] {
+        if (Joint && csize > 1)
+            cluster_barrier();
+        else
+            __syncthreads();
+    };
     // address of unit u (amplitudes 2u, 2u + 1 of the tile) of tile t
     auto tile_fixed = [](unsigned t, int w) {
         return ((t & ((1u << (w - kRunBits)) - 1u)) << kRunBits) | ((t >> (w - kRunBits)) << (w + kWindow));
@@ -477,27 +511,37 @@ __global__ void __launch_bounds__(kWinThreads, kWinCtas) k_vqe_window(const VqeA
         __syncthreads();
     };
     for (;;) {
-        __syncthreads();
-        if (tid == 0) s_idx = A.begin + (int)atomicAdd(A.counter, 1u);
-        __syncthreads();
-        const int idx = s_idx;
+        sync();
+        if (tid == 0 && rank == 0)
+            s_idx = Joint && csize > 1 ? A.begin + atomicAdd(A.counter, 1u) : A.split + atomicAdd(A.counter + 1, 1u);
+        sync();
+        const int idx = (int)(Joint && csize > 1 ? peer_u64(&s_idx, 0) : s_idx);
+        if (Joint && csize > 1 && idx >= A.split) {
+            cluster_barrier();  // rank 0's word has been read
+            buf = A.gbuf + (size_t)blockIdx.x * A.gstride;
+            rank = 0;
+            csize = 1;
+            continue;
+        }
         if (idx >= A.end) break;
         const int c = A.order[idx];
         const int n = A.nq[c], L = A.nl[c];
         const double *ang = A.angles + A.aoff[c];
         if (L == 0) {  // |0...0>
-            if (tid == 0) A.energies[c] = -(double)(n - 1);
+            if (tid == 0 && rank == 0) A.energies[c] = -(double)(n - 1);
             continue;
         }
         if (tid == 0) {
             progress_start(S.prog, n, L);
-            buf[0] = make_float2(1.f, 0.f);
-            buf[1] = make_float2(0.f, 0.f);
+            if (rank == 0) {
+                buf[0] = make_float2(1.f, 0.f);
+                buf[1] = make_float2(0.f, 0.f);
+            }
         }
         int nz = 1;  // the state is zero from index 2^nz on
         double xx = 0.0, zz = 0.0;
         for (bool last = false; !last;) {
-            __syncthreads();
+            sync();
             if (tid == 0) make_pass(S.prog, window_start(S.prog), S.pass);
             __syncthreads();
             const int w = S.pass.w, ns = S.pass.nsteps;
@@ -582,7 +626,7 @@ __global__ void __launch_bounds__(kWinThreads, kWinCtas) k_vqe_window(const VqeA
             // where this thread's stores find their amplitudes
             const unsigned p_tid = map_position(S.end, 2 * tid), p_one = S.end.inv[0];
             const unsigned tiles = 1u << (nz_out - kTileBits);
-            for (unsigned t = 0; t < tiles; ++t) {
+            for (unsigned t = rank; t < tiles; t += csize) {
                 const unsigned fixed = tile_fixed(t, w);
                 load(fixed, w, nz);
                 for (int st = 0; st < ns; ++st) {
@@ -637,10 +681,10 @@ __global__ void __launch_bounds__(kWinThreads, kWinCtas) k_vqe_window(const VqeA
         }
         // ZZ of all qubits and X of the 13 lowest
         if (tid == 0) map_identity(S.end);
-        __syncthreads();
+        sync();
         x_groups(S, S.end, n < kTileBits ? (1u << n) - 1u : (unsigned)kTile - 1u);
         const unsigned m1 = (1u << (n - 1)) - 1u;
-        for (unsigned t = 0; t < (1u << (n - kTileBits)); ++t) {
+        for (unsigned t = rank; t < (1u << (n - kTileBits)); t += csize) {
             load(t << kTileBits, kRunBits, n);
             float zf = 0.f;
             for (unsigned i = 0; i < kTile / kWinThreads; ++i) {
@@ -652,9 +696,21 @@ __global__ void __launch_bounds__(kWinThreads, kWinCtas) k_vqe_window(const VqeA
             xx += (double)xf;
             __syncthreads();
         }
-        const double zzs = block_sum_d(zz, s_red);
-        const double xxs = block_sum_d(xx, s_red);
-        if (tid == 0) A.energies[c] = -zzs - A.h * xxs;
+        double zzs = block_sum_d(zz, s_red);
+        double xxs = block_sum_d(xx, s_red);
+        if (Joint && csize > 1) {
+            if (tid == 0) {
+                s_part[0] = zzs;
+                s_part[1] = xxs;
+            }
+            cluster_barrier();
+            if (tid == 0 && rank == 0)
+                for (unsigned r = 1; r < csize; ++r) {
+                    zzs += __longlong_as_double((long long)peer_u64(&s_part[0], r));
+                    xxs += __longlong_as_double((long long)peer_u64(&s_part[1], r));
+                }
+        }
+        if (tid == 0 && rank == 0) A.energies[c] = -zzs - A.h * xxs;
     }
 }
 
@@ -716,14 +772,38 @@ int count_large(const qsim_batch *b, int m) {
     return k;
 }
 
+// CTAs per cluster for the first circuits of the order, *joint of them, when
+// few circuits hold much of the work; 1 when there are enough circuits.  A CTA
+// alone with a circuit ends late if the circuit is more than a CTA's share of
+// the work; of 17 qubits on (16 tiles and more, so that the passes over one
+// tile and their preparation weigh less) sharing pays from half of that on.
+// Milliseconds with 1, 4 and 8 CTAs per circuit, 10..20 qubits: 40 circuits
+// 6.2, 2.1, 1.2; 200: 9.8, 3.9, 2.2; 1024: 14.4, 5.5, 6.3; 4096: 16.7, 19, 20;
+// 13..16 qubits: 1024 circuits 1.2, 1.5, 1.9.
+int cluster_size(const qsim_batch *b, int large, int ctas, int *joint) {
+    auto amps = [&](int k) { return (double)(1u << b->nq[b->order[k]]); };
+    double work = 0.0;
+    for (int k = 0; k < large; ++k) work += amps(k);
+    auto shared = [&](int k) {
+        const int n = b->nq[b->order[k]];
+        return n >= 16 && amps(k) * ctas * (n >= 17 ? 2 : 1) > work;
+    };
+    *joint = 0;
+    while (*joint < large && shared(*joint)) ++*joint;
+    const int cl = amps(0) * ctas > 4.0 * work ? 8 : 4;
+    return *joint > 0 && ctas >= cl ? cl : 1;
+}
+
 bool config_valid(const qsim_batch *b, int threads, int m) {
     (void)b;
     return (1 << m) <= reg_amps(threads) * threads;  // in-place permutation through registers
 }
 
 int occupancy_global(const qsim_batch *b, int *grid) {
-    VqeKernel k = k_vqe_window;
+    VqeKernel k = k_vqe_window<true>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWinSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_vqe_window<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWinSmem);
     if (e != cudaSuccess) return QSIM_ECUDA;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWinThreads, kWinSmem);
@@ -751,8 +831,8 @@ int berr(qsim_batch *b, int code, const std::string &msg) {
 
 int launch(qsim_batch *b, int threads, int m, int grid) {
     const int large = count_large(b, m);
-    // the two queues' counters and the error flag
-    cudaError_t e = cudaMemsetAsync(b->d_counter, 0, 3 * sizeof(unsigned int), b->stream);
+    // the three queues' counters and the error flag
+    cudaError_t e = cudaMemsetAsync(b->d_counter, 0, 4 * sizeof(unsigned int), b->stream);
     if (e != cudaSuccess) return berr(b, QSIM_ECUDA, cudaGetErrorString(e));
     VqeArgs a;
     a.order = b->d_order;
@@ -761,7 +841,7 @@ int launch(qsim_batch *b, int threads, int m, int grid) {
     a.aoff = b->d_aoff;
     a.angles = b->d_angles;
     a.energies = b->d_energies;
-    a.err = b->d_counter + 2;
+    a.err = b->d_counter + 3;
     a.m = m;
     a.gbuf = b->d_gbuf;
     a.gstride = b->gstride;
@@ -774,12 +854,23 @@ int launch(qsim_batch *b, int threads, int m, int grid) {
         a.counter = b->d_counter;
         a.begin = 0;
         a.end = large;
-        k_vqe_window<<<ggrid, kWinThreads, kWinSmem, b->stream>>>(a);
-        e = cudaGetLastError();
+        const int cl = cluster_size(b, large, ggrid, &a.split);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(ggrid / cl * cl);
+        cfg.blockDim = dim3(kWinThreads);
+        cfg.dynamicSmemBytes = kWinSmem;
+        cfg.stream = b->stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = cl;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = cl > 1;
+        e = cudaLaunchKernelEx(&cfg, cl > 1 ? k_vqe_window<true> : k_vqe_window<false>, a);
         if (e != cudaSuccess) return berr(b, QSIM_ECUDA, cudaGetErrorString(e));
     }
     if (large < b->count) {
-        a.counter = b->d_counter + 1;
+        a.counter = b->d_counter + 2;
         a.begin = large;
         a.end = b->count;
         kernel_for(threads)<<<grid, threads, (size_t)8 << m, b->stream>>>(a);
@@ -805,7 +896,7 @@ int build_graph(qsim_batch *b) {
     cudaMemcpyAsync(b->d_angles, b->h_angles, sizeof(double) * b->nangles, cudaMemcpyHostToDevice, b->stream);
     rc = launch(b, b->threads, b->m, grid);
     cudaMemcpyAsync(b->h_energies, b->d_energies, sizeof(double) * b->count, cudaMemcpyDeviceToHost, b->stream);
-    cudaMemcpyAsync(b->h_flag, b->d_counter + 2, sizeof(unsigned int), cudaMemcpyDeviceToHost, b->stream);
+    cudaMemcpyAsync(b->h_flag, b->d_counter + 3, sizeof(unsigned int), cudaMemcpyDeviceToHost, b->stream);
     e = cudaStreamEndCapture(b->stream, &g);
     if (rc) return rc;
     if (e != cudaSuccess) return berr(b, QSIM_ECUDA, cudaGetErrorString(e));
@@ -936,18 +1027,11 @@ int sim_batch_create(int count, const int *nqubits, const int *layers, double h,
         sim_batch_destroy(b);
         return QSIM_ECUDA;
     }
-    // default configuration: the largest valid shared-memory threshold
-    b->threads = 512;
-    b->m = 0;
-    for (int m = 14; m >= 12; --m)
-        if (config_valid(b, 512, m)) {
-            b->m = m;
-            break;
-        }
-    if (!b->m) {
-        sim_batch_destroy(b);
-        return QSIM_ENOTSUP;
-    }
+    // default configuration: window passes from 13 qubits on (4096 circuits of
+    // 13..16 qubits 3.3 ms, with up to 14 qubits in shared memory by 512 threads
+    // 4.1; of 4..12 qubits 1.09 and 1.24; one of 10..20 as long either way)
+    b->threads = 256;
+    b->m = 12;
     *out = b;
     return QSIM_OK;
 }

@@ -45,3 +45,22 @@ def test_windows_against_oracle(qs, oracle_mod, scale):
         # random; the energy's scale is its number of terms
         tol = 2.0 ** -24 * 8 * np.sqrt(max(1, c["n"] * c["L"])) * (2 * c["n"])
         assert abs(e - oracle_energy(oracle_mod, c, h)) <= tol, (c["n"], c["L"])
+
+
+@pytest.mark.parametrize("sizes", [
+    [(17, 3)] * 100 + [(13, 2)] * 40,            # clusters of 4, then CTAs alone
+    [(18, 2)] * 3 + [(14, 0), (15, 4), (9, 2)],  # clusters of 8
+    [(16, 1)] * 330 + [(16, 0)],                 # a CTA per circuit
+])
+def test_shared_circuits_against_alone(qs, sizes):
+    rng = np.random.default_rng(len(sizes))
+    angles = [rng.uniform(-np.pi, np.pi, 2 * n * L) for n, L in sizes]
+    with qs.Batch([n for n, _ in sizes], [L for _, L in sizes], h=0.7) as b:
+        got = b.run(np.concatenate(angles))
+        np.testing.assert_array_equal(got, b.run(np.concatenate(angles)))
+    for i in {0, len(sizes) // 3, len(sizes) // 2, len(sizes) - 2, len(sizes) - 1}:
+        n, L = sizes[i]
+        with qs.Batch([n], [L], h=0.7) as b:
+            alone = b.run(angles[i])[0]
+        # the same FP32 sums per tile, added up in another order in FP64
+        assert abs(got[i] - alone) <= 1e-12 * 2 * n, (i, n, L)
