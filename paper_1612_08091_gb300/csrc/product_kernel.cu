@@ -35,10 +35,12 @@
 // writes of eight lanes meet eight different slots, the 8-byte accesses of a
 // warp 32 different places.  The global addresses of a thread's accesses step
 // through the register bits in Gray-code order, one 64-bit add each.
-// Per 28-qubit pass: 0.778 ms (5.52 TB/s, 82 % of HBM) against 0.805 ms with
+// Per 28-qubit pass: 0.718 ms (5.98 TB/s, 89 % of HBM); 0.778 ms with the
+// passes' qubits in ascending order (launch_product), then 0.805 ms with
 // tiles copied in asynchronously ahead (double-buffered, 24 instead of 32
-// warps per SM, six crossings of shared memory).  With 64 amplitudes a thread and two layouts (two crossings, 12 warps
-// per SM) a pass took 1.18 ms: too few warps to cover the latencies.
+// warps per SM, six crossings of shared memory).  With 64 amplitudes a thread
+// and two layouts (two crossings, 12 warps per SM) a pass took 1.18 ms: too
+// few warps to cover the latencies.
 //
 // Norm control.  A product pass is one step of the same norm chain as the
 // tensor-core block passes (norm_chain.cuh): its inputs' and outputs' sums
@@ -327,6 +329,16 @@ int launch_product(qsim *s, uint64_t qmask, const cd *mats, int *npasses) {
     const int npass_hi = (nhi + per - 1) / per;
     const int last = nhi - (npass_hi - 1) * per;  // qubits of the last high pass
     const bool fold = npass_hi > 0 && (nlo == 0 || lo[nlo - 1] < kPBits - last);
+    // Each pass takes half its qubits from the lowest and half from the highest
+    // left.  A tile of a pass on the 8 highest qubits of 28 has its 256 runs 8 MB
+    // and more apart, each in a page of its own: 0.89 ms, the passes on lower
+    // qubits 0.72.  In halves the pages of a tile are at most 64: the two passes
+    // 1.39 instead of 1.60 ms (every other qubit: 1.43).
+    int of[64];
+    for (int p = 0, a = 0, b = nhi - 1; p < npass_hi; ++p) {
+        const int k = p < npass_hi - 1 ? per : last;
+        for (int i = 0; i < k; ++i) of[i < (k + 1) / 2 ? a++ : b--] = p;
+    }
     int rc = QSIM_OK;
     if (nlo > 0 && !fold) {
         rc = launch_pass(s, lo, mlo, nlo);
@@ -341,10 +353,11 @@ int launch_product(qsim *s, uint64_t qmask, const cd *mats, int *npasses) {
                 q[k] = lo[j];
                 m[k++] = mlo[j];
             }
-        for (int j = p * per; j < nhi && j < (p + 1) * per; ++j) {
-            q[k] = hi[j];
-            m[k++] = mhi[j];
-        }
+        for (int j = 0; j < nhi; ++j)
+            if (of[j] == p) {
+                q[k] = hi[j];
+                m[k++] = mhi[j];
+            }
         rc = launch_pass(s, q, m, k);
         ++*npasses;
     }
