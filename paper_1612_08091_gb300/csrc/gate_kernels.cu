@@ -75,8 +75,9 @@ __global__ void __launch_bounds__(256) k_dense1(Amp *__restrict__ psi, uint64_t 
 }
 
 // complex128 one-qubit dense gate in shared-exponent integers (fx128.cuh): 26
-// qubits 0.36 ms (6.0 TB/s, 89 % of HBM) against 1.03 ms in FP64 arithmetic;
-// bound by issue, about evenly with HBM.
+// qubits 0.43 ms on a full state (5.0 TB/s, 74 % of HBM; 0.31 ms while most
+// groups are zero) against 1.03 ms in FP64 arithmetic; bound by the integer
+// multiply-add pipe.
 template <int kGroups>
 __global__ void __launch_bounds__(256) k_dense1_fx(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                    uint64_t cmask, uint64_t tbit, const qsim_fx::MatFx M) {
