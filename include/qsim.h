@@ -63,7 +63,8 @@ enum qsim_status {
 };
 
 enum qsim_precision {
-    QSIM_C128 = 0, /* complex128 amplitudes, FP64 arithmetic */
+    QSIM_C128 = 0, /* complex128 amplitudes, FP64 arithmetic (one-qubit dense gates in
+                      60-bit integers where these err no more) */
     QSIM_C64 = 1   /* complex64 amplitudes; fused blocks on tensor cores */
 };
 
@@ -96,7 +97,9 @@ typedef struct qsim_opts {
     int c128_double_float;  /* non-zero: complex128 gates (one-qubit dense, diagonal and
                                phase gates, multi-target dense gates) and fused blocks
                                (dense and diagonal) compute in FP32 pairs (about 2^-45
-                               relative error per product) instead of FP64 arithmetic */
+                               relative error per product), or, dense on 2 to 4 qubits,
+                               in integers and FP32 to the same accuracy, instead of
+                               FP64 arithmetic */
     int no_permutation_blocks; /* non-zero: the greedy and learned planners form no
                                permutation blocks (runs of X / CNOT / Toffoli / SWAP
                                executed as one emulated-permutation pass) */

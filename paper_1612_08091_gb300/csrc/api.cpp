@@ -2,8 +2,8 @@
 //
 // Host side only: argument validation, the lazy gate queue, planning and the
 // dispatch of device work onto the handle's stream.  Every arithmetic step
-// on amplitudes runs in the CUDA kernels (gate_kernels.cu,
-// tmem_block_kernel.cu, diag_kernels.cu, perm_kernels.cu,
+// on amplitudes runs in the CUDA kernels (gate_kernels.cu, small_kernel.cu,
+// tmem_block_kernel.cu, diag_kernels.cu, product_kernel.cu, perm_kernels.cu,
 // reduce_kernels.cu).
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>

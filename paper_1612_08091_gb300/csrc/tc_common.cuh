@@ -1,6 +1,5 @@
-// tc_common.cuh -- inline-PTX helpers shared by the tensor-core block
-// kernels (fused_kernel.cu: 5-qubit blocks, tmem_block_kernel.cu: 5- and 6-qubit
-// blocks) and the batched variational kernel (vqe_kernel.cu: bulk copies):
+// tc_common.cuh -- inline-PTX helpers of the tensor-core block kernels
+// (tmem_block_kernel.cu) and the bulk-copy permutations (perm_kernels.cu):
 // mbarriers with bounded waits, bulk copies, tcgen05 fences, shared-memory
 // matrix descriptors, MMA commit, tensor-memory loads and stores, and the
 // bf16 hi/lo split of an amplitude.
@@ -74,11 +73,6 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
     mbar_expect_tx(bar, bytes);
     bulk_copy(dst, src, bytes, bar);
 }
-
-// Order this thread's earlier generic-proxy accesses (to global memory, or
-// to this CTA's shared memory) before its later async-proxy (bulk copy)
-// accesses.
-__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // 64-bit shared-memory matrix descriptor: K-major, 128-byte swizzle, rows of
 // 128 B, 8-row groups 1024 B apart.
