@@ -676,13 +676,16 @@ int sim_mlp_train(qsim_mlp *m, const float *X, const float *T, int n, int epochs
     // rows are whole 16-byte units; the per-layer kernels for other widths
     // (256-sample batches, 64 units: 16.6 us a step against 146 us)
     const bool fused = m->d.H <= kTrainMaxH && m->d.H % 4 == 0;
+    // the copies from host memory are waited for before every return, and the
+    // corrections live as long: the runtime may read them as late as that
+    std::vector<float2> corr;
     if (fused) {
         const size_t smem = train_smem(m->d.H);
         if (cudaFuncSetAttribute(k_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
             cudaGetLastError();
+            cudaStreamSynchronize(m->stream);
             return mlp_err(m, QSIM_ECUDA, "training kernel attribute");
         }
-        std::vector<float2> corr;
         for (long long s0 = 0; s0 < steps; s0 += kTrainSteps) {
             const long long s1 = std::min<long long>(steps, s0 + kTrainSteps);
             if (s0) cudaStreamSynchronize(m->stream);  // `corr` is still being copied from

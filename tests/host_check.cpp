@@ -1,0 +1,54 @@
+// Host-side checks of the library on a fake CUDA runtime (fake_cudart.h),
+// linked with the library's own objects by tests/test_host_cpu.py: what its
+// host code hands to the device, and what it does when a call fails.
+#include "fake_cudart.h"
+
+#include <cstdio>
+#include <vector>
+
+#include "../include/qsim.h"
+
+namespace {
+
+int failures = 0;
+#define CHECK(c)                                                          \
+    do {                                                                  \
+        if (!(c)) {                                                       \
+            std::printf("line %d: %s is false\n", __LINE__, #c);          \
+            ++failures;                                                   \
+        }                                                                 \
+    } while (0)
+
+// sim_mlp_train: what its copies read lives until they have run, also where it
+// returns an error
+void check_training_sources() {
+    const int n = 10;
+    std::vector<float> X(16 * n, 0.5f), T(n, 1.f);
+    qsim_mlp *m = nullptr;
+    CHECK(sim_mlp_create(64, 1, nullptr, &m) == QSIM_OK);
+    float loss = 0.f;
+    fake::freed_sources = 0;
+    CHECK(sim_mlp_train(m, X.data(), T.data(), n, 2, 4, 1e-3f, &loss) == QSIM_OK);
+    CHECK(fake::launched("k_train") == 1);
+    CHECK(sim_mlp_train(m, X.data(), T.data(), n, 500, 1, 1e-3f, &loss) == QSIM_OK);  // 5000 steps: two launches
+    CHECK(fake::launched("k_train") == 3);
+    CHECK(fake::freed_sources == 0);
+    fake::fail_launch = "k_train";
+    CHECK(sim_mlp_train(m, X.data(), T.data(), n, 2, 4, 1e-3f, &loss) == QSIM_ECUDA);
+    fake::fail_launch = nullptr;
+    CHECK(fake::npending == 0 && fake::freed_sources == 0);
+    fake::fail_attribute = 1;
+    CHECK(sim_mlp_train(m, X.data(), T.data(), n, 2, 4, 1e-3f, &loss) == QSIM_ECUDA);
+    fake::fail_attribute = 0;
+    CHECK(fake::npending == 0 && fake::freed_sources == 0);
+    fake::run_copies();
+    sim_mlp_destroy(m);
+}
+
+}  // namespace
+
+int main() {
+    check_training_sources();
+    std::printf(failures ? "%d failures\n" : "ok\n", failures);
+    return failures != 0;
+}
