@@ -46,9 +46,11 @@ struct Fx {  // hi 2^28 + lo, 0 <= lo < 2^28
 // exponent word of a double (sign cleared): its biased exponent is this >> 20
 __device__ __forceinline__ uint32_t mag(double x) { return (uint32_t)__double2hiint(x) & 0x7FFFFFFFu; }
 __device__ __forceinline__ uint32_t mag(double2 z) { return max(mag(z.x), mag(z.y)); }
-// the exponents this arithmetic takes: all intermediate and result exponents
-// are those of normal numbers
+// the exponents this arithmetic takes (amplitudes of 2^-894 to 2^961): with
+// matrices between 2^-64 and kFxMatrixTop all intermediate and result
+// exponents are those of normal numbers (a result is below 2^961 2^59)
 __device__ __forceinline__ bool fx_range(int E) { return E > 128 && E < 0x7C0; }
+constexpr double kFxMatrixLow = 0x1p-64, kFxMatrixTop = 0x1p56;
 
 // arithmetic right shift, by more than 63 too
 __device__ __forceinline__ long long shr_s64(long long v, uint32_t s) {
@@ -200,7 +202,9 @@ inline bool make_fx(const std::complex<double> *m, MatFx &M) {
         low = std::min(low, std::abs(m[e]));
         comp = std::max(comp, std::max(std::abs(m[e].real()), std::abs(m[e].imag())));
     }
-    if (!(low >= std::ldexp(top, -kFxMinLog)) || !(top > 0x1p-64) || !(top < 0x1p64)) return false;
+    if (!(low >= std::ldexp(top, -kFxMinLog)) || !(top > kFxMatrixLow) ||
+        !(top < kFxMatrixTop))
+        return false;
     int x;
     std::frexp(comp, &x);  // comp < 2^x
     const int S = 57 - x;

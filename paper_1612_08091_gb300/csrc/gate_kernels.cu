@@ -496,7 +496,8 @@ int dense_k_fx(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
         rows = std::max(rows, t);
     }
     // a zero or an extreme matrix: FP64
-    if (!(rows > 0x1p-64) || !(rows < 0x1p64)) return dense_k_plain<double2, K>(s, targets, cmask, m);
+    if (!(rows > qsim_fx::kFxMatrixLow) || !(rows < qsim_fx::kFxMatrixTop))
+        return dense_k_plain<double2, K>(s, targets, cmask, m);
     int x;
     std::frexp(rows, &x);  // rows < 2^x
     const int S = 52 - x;
