@@ -216,7 +216,9 @@ int sim_collapse(qsim *s, const int *qubits, int m, const int *bits, double *p);
  * phase of psi_j. */
 int sim_measure_all(qsim *s, double u, uint64_t *outcome);
 
-/* <psi| sum_k terms[k].coeff * P_k |psi>, accumulated in FP64.  Not in the
+/* <psi| sum_k terms[k].coeff * P_k |psi>, accumulated in FP64 (complex64: of
+ * FP32 sums over a few amplitudes; strings with an X part: of at most eight
+ * amplitude pairs).  Not in the
  * paper (its simulator exposes no observable); the Pauli-sum expectation the
  * variational workloads need.  The state is assumed normalised (no division
  * by the norm; complex64 block passes hold the norm, see sim_apply). */

@@ -17,6 +17,7 @@
 // pass for all terms; strings with an X/Y part grouped by their X mask, one
 // pass per group) use  P|i> = i^{#Y} (-1)^{popc(i & zmask)} |i ^ xmask>.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -559,13 +560,17 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_x(const Amp *__restrict_
 //   A  e = i | tid << 5                               (tile bits 0..4)
 //   B  e = (tid & 31) | i << 5 | (tid >> 5) << 10     (tile bits 5..9)
 //   C  e = tid | s << 8 | i << 10, 8 at a time        (tile bits 10..12)
-// so that both amplitudes of a pair are its own: 2 FMAs per pair and term,
-// about 13 per amplitude and pass, and four crossings of shared memory (one
-// asynchronous copy in, three reads).  Element e sits at position
+// so that both amplitudes of a pair are its own: four crossings of shared
+// memory (one asynchronous copy in, three reads).  Element e sits at position
 // e ^ ((e >> 5) & 7) << 1: an amplitude pair stays one aligned 16-byte slot,
-// eight lanes of layout A meet eight different slots.  Partial sums: FP32
-// over a term's 16 pairs in a thread and over the layout's terms, FP64 from
-// one tile to the next.
+// eight lanes of layout A meet eight different slots.
+// Rounding.  A term's pairs are added eight at a time in FP32, in a tree; two
+// such sums, their product with the coefficient and the terms of a tile are
+// added with their rounding errors kept (x_term), tiles in FP64.  So FP32
+// rounds what it rounds in k_expect_x, sums of eight pairs, and the
+// coefficients stay doubles.  Registers where a thread of k_expect_x has fewer
+// than eight pairs, and each sum then fewer than eight, take Fine: every pair
+// goes to FP64 on its own.
 // 29 qubits, 29 terms: 2.13 ms (0.71 ms a pass, 6.05 TB/s, 90 % of HBM)
 // against 38.2 ms with a read per term.  Fewer than two terms, complex128
 // and registers below one tile keep k_expect_x.
@@ -576,26 +581,53 @@ constexpr int kXMinRun = 3;  // runs of at least 2^3 amplitudes
 struct XTileArgs {
     uint64_t ntiles;       // 2^(n - 13)
     InsertSpec vspec;      // V, ascending
-    float c[kXBits];       // 2 c_q of the qubit at tile bit j (0: no term)
+    double c[kXBits];      // 2 c_q of the qubit at tile bit j (0: no term)
+    float ch[kXBits], cl[kXBits];  // the same as a pair of FP32
     uint32_t mask;         // tile bits with a term
 };
 
 __device__ __forceinline__ uint32_t xswz(uint32_t e) { return e ^ (((e >> 5) & 7u) << 1); }
 
-// sum of Re v_i conj(v_j) over the pairs of register bit r
+// the k-th of the pairs of register bit r: Re v_i conj(v_j)
 template <int N>
-__device__ __forceinline__ float x_pairs(const float2 (&v)[N], int r) {
-    float s0 = 0.f, s1 = 0.f;
+__device__ __forceinline__ float x_pair(const float2 (&v)[N], int r, int k) {
+    const int i = ((k >> r) << (r + 1)) | (k & ((1 << r) - 1));
+    const float2 a = v[i], b = v[i | (1 << r)];
+    return fmaf(a.x, b.x, a.y * b.y);
+}
+// sum of M pairs from the k0-th on, in a tree
+template <int M, int N>
+__device__ __forceinline__ float x_pairs(const float2 (&v)[N], int r, int k0) {
+    float t[M];
 #pragma unroll
-    for (int i = 0; i < N; ++i)
-        if (!((i >> r) & 1)) {
-            const float2 a = v[i], b = v[i | (1 << r)];
-            s0 = fmaf(a.x, b.x, s0);
-            s1 = fmaf(a.y, b.y, s1);
-        }
-    return s0 + s1;
+    for (int k = 0; k < M; ++k) t[k] = x_pair(v, r, k0 + k);
+#pragma unroll
+    for (int w = M / 2; w; w >>= 1)
+#pragma unroll
+        for (int k = 0; k < w; ++k) t[k] = __fadd_rn(t[k], t[k + w]);
+    return t[0];
+}
+// all pairs in FP64
+template <int N>
+__device__ __forceinline__ double x_pairs_fine(const float2 (&v)[N], int r) {
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) s += (double)x_pair(v, r, k);
+    return s;
+}
+// (hi, lo) += (ch + cl) (a + b), with the errors of the sums and of the
+// product; lo is meaningless where hi is not finite
+__device__ __forceinline__ void x_term(float &hi, float &lo, float a, float b, float ch, float cl) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    const float p = __fmul_rn(ch, s);
+    const float pe = fmaf(ch, e, fmaf(cl, s, fmaf(ch, s, -p)));
+    const float t = __fadd_rn(hi, p), tb = __fsub_rn(t, hi);
+    lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, tb)), __fsub_rn(p, tb)) + pe;
+    hi = t;
 }
 
+template <bool Fine>
 __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const float2 *__restrict__ psi,
                                                                           const XTileArgs A,
                                                                           double *__restrict__ partials) {
@@ -628,7 +660,18 @@ __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const
         asm volatile("cp.async.commit_group;" ::: "memory");
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
-        float e = 0.f;
+        float hi = 0.f, lo = 0.f;
+        // the terms of tile bits base..base + 4, 16 pairs each
+        auto five = [&](const float2(&v)[32], uint32_t mask, int base) {
+#pragma unroll
+            for (int r = 0; r < 5; ++r) {
+                if (!((mask >> r) & 1u)) continue;
+                if (Fine)
+                    acc = fma(A.c[base + r], x_pairs_fine(v, r), acc);
+                else
+                    x_term(hi, lo, x_pairs<8>(v, r, 0), x_pairs<8>(v, r, 8), A.ch[base + r], A.cl[base + r]);
+            }
+        };
         if (mA) {
             float2 v[32];
 #pragma unroll
@@ -637,30 +680,39 @@ __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const
                 v[2 * j] = make_float2(w.x, w.y);
                 v[2 * j + 1] = make_float2(w.z, w.w);
             }
-#pragma unroll
-            for (int r = 0; r < 5; ++r)
-                if ((mA >> r) & 1u) e = fmaf(A.c[r], x_pairs(v, r), e);
+            five(v, mA, 0);
         }
         if (mB) {
             float2 v[32];
 #pragma unroll
             for (uint32_t i = 0; i < 32; ++i) v[i] = xs[xswz((tid & 31u) | (i << 5) | ((tid >> 5) << 10))];
-#pragma unroll
-            for (int r = 0; r < 5; ++r)
-                if ((mB >> r) & 1u) e = fmaf(A.c[5 + r], x_pairs(v, r), e);
+            five(v, mB, 5);
         }
         if (mC) {
+            float h[3][4];  // four pairs each
 #pragma unroll
             for (uint32_t s = 0; s < 4; ++s) {
                 float2 v[8];
 #pragma unroll
                 for (uint32_t i = 0; i < 8; ++i) v[i] = xs[xswz(tid | (s << 8) | (i << 10))];
 #pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    if (!((mC >> r) & 1u)) continue;
+                    if (Fine)
+                        acc = fma(A.c[10 + r], x_pairs_fine(v, r), acc);
+                    else
+                        h[r][s] = x_pairs<4>(v, r, 0);
+                }
+            }
+            if (!Fine) {
+#pragma unroll
                 for (int r = 0; r < 3; ++r)
-                    if ((mC >> r) & 1u) e = fmaf(A.c[10 + r], x_pairs(v, r), e);
+                    if ((mC >> r) & 1u)
+                        x_term(hi, lo, __fadd_rn(h[r][0], h[r][1]), __fadd_rn(h[r][2], h[r][3]), A.ch[10 + r],
+                               A.cl[10 + r]);
             }
         }
-        acc += (double)e;
+        if (!Fine) acc += (double)hi + (isfinite(hi) ? (double)lo : 0.0);
     }
     acc = block_sum(acc, sh);
     if (threadIdx.x == 0) partials[blockIdx.x] = acc;
@@ -965,7 +1017,9 @@ int field_passes(qsim *s, uint64_t field, const double *c, unsigned *filled, Roo
     static bool attr[64] = {false};
     constexpr int smem = (int)(sizeof(float2) << kXBits);
     if (s->device < 0 || s->device >= 64 || !attr[s->device]) {
-        const cudaError_t e = cudaFuncSetAttribute(k_expect_x_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(k_expect_x_tiles<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_expect_x_tiles<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return cuda_err(s, e, "expect attribute");
         if (s->device >= 0 && s->device < 64) attr[s->device] = true;
     }
@@ -983,7 +1037,9 @@ int field_passes(qsim *s, uint64_t field, const double *c, unsigned *filled, Roo
             if ((V >> b) & 1ull) {
                 if (((field & ~done) >> b) & 1ull) {
                     A.mask |= 1u << k;
-                    A.c[k] = (float)(2.0 * c[b]);
+                    A.c[k] = 2.0 * c[b];
+                    A.ch[k] = (float)A.c[k];
+                    A.cl[k] = (float)(A.c[k] - (double)A.ch[k]);
                 }
                 A.vspec.pos[k++] = b;
             }
@@ -991,7 +1047,13 @@ int field_passes(qsim *s, uint64_t field, const double *c, unsigned *filled, Roo
         A.ntiles = 1ull << (n - kXBits);
         const unsigned grid = (unsigned)std::min<uint64_t>(A.ntiles, (uint64_t)kXCtasPerSm * s->sms);
         if (const int rc = room(grid)) return rc;
-        k_expect_x_tiles<<<grid, kXThreads, smem, s->stream>>>((const float2 *)s->state, A, ws_partials(s) + *filled);
+        // fewer than eight pairs a thread of k_expect_x
+        if (((1ull << n) >> 1) < 8ull * reduce_blocks(s) * kRedThreads)
+            k_expect_x_tiles<true>
+                <<<grid, kXThreads, smem, s->stream>>>((const float2 *)s->state, A, ws_partials(s) + *filled);
+        else
+            k_expect_x_tiles<false>
+                <<<grid, kXThreads, smem, s->stream>>>((const float2 *)s->state, A, ws_partials(s) + *filled);
         s->stats.launches++;
         *filled += grid;
         const cudaError_t e = cudaGetLastError();
@@ -1069,6 +1131,9 @@ int expect_t(qsim *s, const qsim_pauli *terms, int nterms, double *out) {
                     field |= terms[k].xmask;
                     c[__builtin_ctzll(terms[k].xmask)] += terms[k].coeff;
                 }
+            // coefficients that FP32 pairs do not hold, and sums of 0, term by term
+            for (int b = 0; b < n; ++b)
+                if (!(std::abs(c[b]) >= 0x1p-100) || !(std::abs(c[b]) <= 0x1p100)) field &= ~(1ull << b);
             // one term takes one read either way (k_expect_x then reads it)
             if (__builtin_popcountll(field) < 2) field = 0;
             if ((rc = field ? field_passes(s, field, c, &filled, room) : QSIM_OK)) return rc;
