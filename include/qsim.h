@@ -64,7 +64,7 @@ enum qsim_status {
 
 enum qsim_precision {
     QSIM_C128 = 0, /* complex128 amplitudes, FP64 arithmetic (one-qubit dense gates in
-                      60-bit integers where these err no more) */
+                      60-bit integers where a result, as a complex number, errs no more) */
     QSIM_C64 = 1   /* complex64 amplitudes; fused blocks on tensor cores */
 };
 

@@ -17,10 +17,18 @@
 // sum |m| max |x| plus its one rounding.  FP64 arithmetic rounds each product
 // to 2^-53 of itself.  Where every |m| is at least 2^-kFxMinLog of the
 // largest, a product with the group's largest amplitude is in every result,
-// so FP64's own error is of at least the same size: that is the condition
-// under which the FP64 gates take this path (make_fx).  Measured against
-// 128-bit sums on 300,000 random U3 gates: 4.7e-17 of the result's norm, FP64
-// 7.3e-17, whatever the spread of the inputs' exponents.
+// so FP64's own error of the result, as a complex number, is of at least the
+// same size: that is the condition under which the FP64 gates take this path
+// (make_fx).  Measured against 128-bit sums on 300,000 random U3 gates: 4.7e-17
+// of the result's norm, FP64 7.3e-17, whatever the spread of the inputs'
+// exponents.
+// A result's real and imaginary parts each have this error: with general
+// complex elements the smaller of the two is known to 2^-57 of the group, not
+// of itself.  Matrices whose elements are each real or imaginary (H, RX, RY and
+// their products with Paulis) do not mix all four components, and FP64 keeps
+// the two sets that they do mix apart: there each set has an exponent of its
+// own (Apart), so that a result's component is as exact, against the components
+// it comes from, as in FP64.  Zeros of either sign are exact.
 //
 // Groups whose exponent is near the ends of the range, and infinities and
 // NaN, are left to FP64 (fx_range).
@@ -62,14 +70,12 @@ __device__ __forceinline__ long long shr_s64(long long v, uint32_t s) {
 #endif
 }
 
-// floor(x 2^(1081 - E)) (one less for some exact negative values); E >= the
-// biased exponent of x
+// x 2^(1081 - E) without its fraction; E >= the biased exponent of x, E > 64
 __device__ __forceinline__ Fx to_fx(double x, int E) {
     const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
     const unsigned long long m = (((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | l) << 6;
-    const uint32_t sg = (uint32_t)((int)h >> 31);
-    long long v = (long long)(m ^ (((unsigned long long)sg << 32) | sg));
-    v = shr_s64(v, (uint32_t)(E - (int)((h >> 20) & 0x7FFu)));
+    const long long sg = (int)h >> 31;
+    const long long v = (shr_s64((long long)m, (uint32_t)(E - (int)((h >> 20) & 0x7FFu))) ^ sg) - sg;
     return Fx{(int)(v >> 28), (int)((uint32_t)v & 0xFFFFFFFu)};
 }
 
@@ -140,10 +146,13 @@ __device__ __forceinline__ double to_double_f(long long a, float c, int eadd) {
     return __hiloint2double(h ? h + eadd : 0, __double2loint(d));
 }
 
-// A 2x2 matrix in this form.
+// A 2x2 matrix in this form.  Element e of an Apart matrix is real or (bit e of
+// `imag`) imaginary; its re and im are then the factors of the results' real
+// and imaginary parts.
 struct MatFx {
     Fx re[4], im[4], nim[4];  // m 2^S; nim = -im
-    int shift, pad;           // -1025 - S
+    int shift, apart, imag;   // shift: -1025 - S
+    int pad;
     double2 m[4];             // the matrix itself, for groups outside the range
 };
 
@@ -167,10 +176,45 @@ __device__ __forceinline__ double2 row_fp64(const MatFx &M, int r, double2 a, do
     return qsim_dev::cfma(M.m[2 * r + 1], b, qsim_dev::cmul(M.m[2 * r], a));
 }
 
+// Two components that an Apart matrix mixes, with their exponent; E = 0 for
+// two zeros, -1 outside the range.
+struct Side {
+    Fx a, b;
+    int E;
+};
+__device__ __forceinline__ Side side(double a, double b) {
+    const int E = (int)(max(mag(a), mag(b)) >> 20);
+    if (fx_range(E)) return Side{to_fx(a, E), to_fx(b, E), E};
+    return Side{Fx{0, 0}, Fx{0, 0}, a == 0.0 && b == 0.0 ? 0 : -1};
+}
+__device__ __forceinline__ double side_sum(const MatFx &M, Fx wa, Fx wb, const Side &s) {
+    Acc t{0, 0};
+    mac(t, wa, s.a);
+    mac(t, wb, s.b);
+    return to_double(t, (s.E + M.shift) << 20);
+}
+// row r of an Apart M: p and q are the components that row 0 takes its real and
+// its imaginary part from
+__device__ __forceinline__ double2 apart_row(const MatFx &M, int r, const Side &p, const Side &q) {
+    const bool crossed = r && ((M.imag ^ (M.imag >> 2)) & 1);
+    return make_double2(side_sum(M, M.re[2 * r], M.re[2 * r + 1], crossed ? q : p),
+                        side_sum(M, M.im[2 * r], M.im[2 * r + 1], crossed ? p : q));
+}
+__device__ __forceinline__ bool apart_sides(const MatFx &M, double2 a, double2 b, Side &p, Side &q) {
+    const bool ia = M.imag & 1, ib = M.imag & 2;
+    p = side(ia ? a.y : a.x, ib ? b.y : b.x);
+    q = side(ia ? a.x : a.y, ib ? b.x : b.y);
+    return p.E >= 0 && q.E >= 0;
+}
+
 // (na, nb) = M (a, b)
 __device__ __forceinline__ void dense1(const MatFx &M, double2 a, double2 b, double2 &na, double2 &nb) {
     const int E = (int)(max(mag(a), mag(b)) >> 20);
-    if (fx_range(E)) {
+    Side p, q;
+    if (M.apart && apart_sides(M, a, b, p, q)) {
+        na = apart_row(M, 0, p, q);
+        nb = apart_row(M, 1, p, q);
+    } else if (!M.apart && fx_range(E)) {
         const Fx ar = to_fx(a.x, E), ai = to_fx(a.y, E), br = to_fx(b.x, E), bi = to_fx(b.y, E);
         na = row(M, 0, ar, ai, br, bi, E);
         nb = row(M, 1, ar, ai, br, bi, E);
@@ -182,7 +226,9 @@ __device__ __forceinline__ void dense1(const MatFx &M, double2 a, double2 b, dou
 // one row of it
 __device__ __forceinline__ double2 dense1_row(const MatFx &M, int r, double2 a, double2 b) {
     const int E = (int)(max(mag(a), mag(b)) >> 20);
-    if (!fx_range(E)) return row_fp64(M, r, a, b);
+    Side p, q;
+    if (M.apart && apart_sides(M, a, b, p, q)) return apart_row(M, r, p, q);
+    if (M.apart || !fx_range(E)) return row_fp64(M, r, a, b);
     return row(M, r, to_fx(a.x, E), to_fx(a.y, E), to_fx(b.x, E), to_fx(b.y, E), E);
 }
 
@@ -208,14 +254,22 @@ inline bool make_fx(const std::complex<double> *m, MatFx &M) {
     int x;
     std::frexp(comp, &x);  // comp < 2^x
     const int S = 57 - x;
+    M.apart = 1;
+    M.imag = M.pad = 0;
     for (int e = 0; e < 4; ++e) {
-        M.re[e] = host_fx(m[e].real(), S);
-        M.im[e] = host_fx(m[e].imag(), S);
+        M.apart &= m[e].real() == 0.0 || m[e].imag() == 0.0;
+        M.imag |= (m[e].real() == 0.0) << e;
+    }
+    // two rows that mix the components differently (no unitary does): FP64
+    if (M.apart && (__builtin_popcount(M.imag) & 1)) return false;
+    for (int e = 0; e < 4; ++e) {
+        const bool im = (M.imag >> e) & 1;
+        M.re[e] = host_fx(M.apart && im ? -m[e].imag() : m[e].real(), S);
+        M.im[e] = host_fx(M.apart && !im ? m[e].real() : m[e].imag(), S);
         M.nim[e] = host_fx(-m[e].imag(), S);
         M.m[e] = make_double2(m[e].real(), m[e].imag());
     }
     M.shift = -1025 - S;
-    M.pad = 0;
     return true;
 }
 
