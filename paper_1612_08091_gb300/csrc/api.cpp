@@ -331,6 +331,13 @@ int flush(qsim *s) {
             s->stats.amp_updates += std::ldexp(1.0, s->n - (int)q[i].controls.size());
             s->stats.alg_bytes += gate_bytes(s, q[i]);
         }
+        if (rc == QSIM_ENOTSUP) {
+            rc = QSIM_OK;
+            for (size_t i = done; i < q.size() && !rc; ++i) {
+                PlanItem one = single_item(q, s->n, (int)i);
+                rc = execute_item(s, one);
+            }
+        }
     } else if (s->fusion == QSIM_FUSE_NONE || (s->fusion == QSIM_FUSE_MLP && s->cost.loaded() && ch.kmax == 1)) {
         std::vector<PlanItem> plan;
         plan_none(q, s->n, plan);

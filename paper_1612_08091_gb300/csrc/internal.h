@@ -162,7 +162,8 @@ int cuda_err(qsim *s, cudaError_t e, const char *where);
 int launch_gate_plain(qsim *s, const GateRec &g);
 int launch_block_dense(qsim *s, const int *qubits, int k, const cd *m);
 // The whole queue on a small register in one launch or a few, gate by gate
-// (small_kernel.cu); *done: gates executed.
+// (small_kernel.cu); *done: gates executed.  QSIM_ENOTSUP where the device does
+// not take the launch: the rest are for the caller.
 bool small_queue_ok(const qsim *s);
 int launch_small_queue(qsim *s, size_t *done);
 // Emulated classical bijection on a register (perm_kernels.cu).

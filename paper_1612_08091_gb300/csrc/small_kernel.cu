@@ -149,24 +149,17 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(Amp *__restrict__ psi, 
 inline void put(double2 *d, cd z) { *d = make_double2(z.real(), z.imag()); }
 inline void put(float2 *d, cd z) { *d = make_float2((float)z.real(), (float)z.imag()); }
 
+// QSIM_ENOTSUP: nothing was launched (the caller runs the gates one by one)
 template <typename Amp, int RB>
 int launch_small(qsim *s, const unsigned char *dev, int ngates, uint32_t rec_bytes) {
-    static bool attr[64] = {false};
+    static signed char usable[64] = {0};  // per device: 1 yes, -1 no
     // at most 2 x 2^9 complex128 or 2 x 2^12 complex64 amplitudes, or those of kSmallOneCta qubits
     constexpr int kMaxSmem = (int)(2 * (sizeof(Amp) == 16 ? 8192 : 32768) + kSmallRecord);
     if (s->device < 0 || s->device >= 64) return QSIM_ENOTSUP;
-    if (!attr[s->device]) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_small<Amp, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-        if (e == cudaSuccess && RB)
-            e = cudaFuncSetAttribute(k_small<Amp, RB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return cuda_err(s, e, "small register kernel attribute");
-        attr[s->device] = true;
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1u << RB);
     cfg.blockDim = dim3(kSmallThreads);
-    cfg.dynamicSmemBytes = 2 * (sizeof(Amp) << (s->n - RB)) + rec_bytes;
+    cfg.dynamicSmemBytes = kMaxSmem;
     cfg.stream = s->stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -174,10 +167,25 @@ int launch_small(qsim *s, const unsigned char *dev, int ngates, uint32_t rec_byt
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = RB ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_small<Amp, RB>, (Amp *)s->state, s->n, dev, ngates, rec_bytes);
+    if (!usable[s->device]) {
+        cudaError_t e =
+            cudaFuncSetAttribute(k_small<Amp, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        // a cluster of 16 needs a GPC with as many free SMs
+        if (e == cudaSuccess && RB)
+            e = cudaFuncSetAttribute(k_small<Amp, RB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        int clusters = 1;
+        if (e == cudaSuccess && RB) e = cudaOccupancyMaxActiveClusters(&clusters, k_small<Amp, RB>, &cfg);
+        if (e != cudaSuccess) cudaGetLastError();
+        usable[s->device] = e == cudaSuccess && clusters > 0 ? 1 : -1;
+    }
+    if (usable[s->device] < 0) return QSIM_ENOTSUP;
+    cfg.dynamicSmemBytes = 2 * (sizeof(Amp) << (s->n - RB)) + rec_bytes;
+    if (cudaLaunchKernelEx(&cfg, k_small<Amp, RB>, (Amp *)s->state, s->n, dev, ngates, rec_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return QSIM_ENOTSUP;
+    }
     s->stats.launches++;
-    if (e != cudaSuccess) cudaGetLastError();
-    return cuda_err(s, e, "small register launch");
+    return QSIM_OK;
 }
 
 template <typename Amp>

@@ -30,6 +30,7 @@ inline int freed_sources = 0;      // sources of pending copies given back to th
 inline int sms = 152;              // multiprocessors of the device
 inline const char *fail_launch = nullptr;  // launches of kernels whose name holds this fail
 inline int fail_attribute = 0;     // cudaFuncSetAttribute fails
+inline int clusters = 1;           // clusters of any size that the device can hold
 inline cudaError_t last = cudaSuccess;
 inline std::map<const void *, std::string> &names() {
     static std::map<const void *, std::string> m;
@@ -166,6 +167,9 @@ cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) {
     return *n = 2, cudaSuccess;
+}
+cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *) {
+    return *n = fake::clusters, cudaSuccess;
 }
 cudaError_t cudaEventCreate(cudaEvent_t *) { return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *, unsigned) { return cudaSuccess; }

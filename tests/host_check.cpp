@@ -45,10 +45,45 @@ void check_training_sources() {
     sim_mlp_destroy(m);
 }
 
+const double kHadamard[8] = {0.7, 0, 0.7, 0, 0.7, 0, -0.7, 0};
+
+qsim *register_of(int n, int precision, int fusion = QSIM_FUSE_NONE) {
+    qsim_opts o = {};
+    o.fusion = fusion;
+    o.kmax = 4;
+    qsim *s = nullptr;
+    CHECK(sim_create(n, precision, &o, &s) == QSIM_OK);
+    CHECK(sim_reset(s, 0) == QSIM_OK);
+    fake::launches().clear();
+    return s;
+}
+
+// a queue on a small register where the cluster launch is not possible: the
+// gates run one by one (complex128: cannot be placed; complex64: the launch fails)
+void check_small_queue_falls_back() {
+    for (int precision : {QSIM_C128, QSIM_C64}) {
+        qsim *s = register_of(11, precision);
+        fake::clusters = precision == QSIM_C128 ? 0 : 1;
+        fake::fail_launch = precision == QSIM_C64 ? "k_small" : nullptr;
+        for (int k = 0; k < 5; ++k) CHECK(sim_apply(s, kHadamard, &k, 1, nullptr, 0) == QSIM_OK);
+        CHECK(sim_flush(s) == QSIM_OK);
+        CHECK(fake::launched("k_small") == 0 && fake::launched("k_dense1") == 5);
+        fake::clusters = 1;
+        fake::fail_launch = nullptr;
+        sim_destroy(s);
+    }
+    qsim *s = register_of(8, QSIM_C128);  // one CTA
+    for (int k = 0; k < 5; ++k) CHECK(sim_apply(s, kHadamard, &k, 1, nullptr, 0) == QSIM_OK);
+    CHECK(sim_flush(s) == QSIM_OK);
+    CHECK(fake::launched("k_small") == 1 && fake::launches().size() == 1);
+    sim_destroy(s);
+}
+
 }  // namespace
 
 int main() {
     check_training_sources();
+    check_small_queue_falls_back();
     std::printf(failures ? "%d failures\n" : "ok\n", failures);
     return failures != 0;
 }
