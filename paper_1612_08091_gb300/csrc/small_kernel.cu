@@ -247,8 +247,18 @@ int small_queue(qsim *s, size_t *done) {
 
 bool small_queue_ok(const qsim *s) {
     // fewer than 3 gates: as many launches cost less than the record's copy
-    return s->fusion == QSIM_FUSE_NONE && !s->profiling && !s->c128_df && s->queue.size() >= 3 &&
-           s->n <= (s->prec == QSIM_C128 ? 13 : 16);
+    if (s->fusion != QSIM_FUSE_NONE || s->profiling || s->c128_df || s->queue.size() < 3 ||
+        s->n > (s->prec == QSIM_C128 ? 13 : 16))
+        return false;
+    // in a stream capture gates are launched one by one, their matrices in the
+    // launches: the graph would copy the record again at each replay, from a
+    // staging buffer that later calls write to
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st == cudaStreamCaptureStatusNone;
 }
 
 int launch_small_queue(qsim *s, size_t *done) {

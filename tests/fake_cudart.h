@@ -30,6 +30,8 @@ inline int freed_sources = 0;      // sources of pending copies given back to th
 inline int sms = 152;              // multiprocessors of the device
 inline const char *fail_launch = nullptr;  // launches of kernels whose name holds this fail
 inline int fail_attribute = 0;     // cudaFuncSetAttribute fails
+inline int capturing = 0;          // streams are being captured
+inline int copies = 0;             // copies from host memory
 inline int clusters = 1;           // clusters of any size that the device can hold
 inline cudaError_t last = cudaSuccess;
 inline std::map<const void *, std::string> &names() {
@@ -142,6 +144,7 @@ cudaError_t cudaFreeHost(void *p) {
     return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void *dst, const void *src, size_t n, cudaMemcpyKind kind, cudaStream_t) {
+    fake::copies += kind == cudaMemcpyHostToDevice;
     if (kind == cudaMemcpyHostToDevice && fake::npending < fake::kMaxPending) {
         fake::pending[fake::npending++] = fake::Copy{dst, src, n};
         return cudaSuccess;
@@ -181,6 +184,10 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t *, unsigned) { return cudaSuc
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *st) {
+    *st = fake::capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *) { return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t *, cudaGraph_t, unsigned long long) { return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }

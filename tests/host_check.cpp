@@ -79,11 +79,27 @@ void check_small_queue_falls_back() {
     sim_destroy(s);
 }
 
+// plain gates in a stream capture: launches alone, no copy from host memory
+// that a replay would repeat
+void check_small_queue_under_capture() {
+    for (int n : {7, 11}) {
+        qsim *s = register_of(n, QSIM_C64);
+        for (int k = 0; k < 5; ++k) CHECK(sim_apply(s, kHadamard, &k, 1, nullptr, 0) == QSIM_OK);
+        fake::capturing = 1;
+        const int copies = fake::copies;
+        CHECK(sim_flush(s) == QSIM_OK);
+        fake::capturing = 0;
+        CHECK(fake::copies == copies && fake::launched("k_dense1") == 5 && fake::launches().size() == 5);
+        sim_destroy(s);
+    }
+}
+
 }  // namespace
 
 int main() {
     check_training_sources();
     check_small_queue_falls_back();
+    check_small_queue_under_capture();
     std::printf(failures ? "%d failures\n" : "ok\n", failures);
     return failures != 0;
 }
