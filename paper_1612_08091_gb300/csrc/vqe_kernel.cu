@@ -772,28 +772,6 @@ int count_large(const qsim_batch *b, int m) {
     return k;
 }
 
-// CTAs per cluster for the first circuits of the order, *joint of them, when
-// few circuits hold much of the work; 1 when there are enough circuits.  A CTA
-// alone with a circuit ends late if the circuit is more than a CTA's share of
-// the work; of 17 qubits on (16 tiles and more, so that the passes over one
-// tile and their preparation weigh less) sharing pays from half of that on.
-// Milliseconds with 1, 4 and 8 CTAs per circuit, 10..20 qubits: 40 circuits
-// 6.2, 2.1, 1.2; 200: 9.8, 3.9, 2.2; 1024: 14.4, 5.5, 6.3; 4096: 16.7, 19, 20;
-// 13..16 qubits: 1024 circuits 1.2, 1.5, 1.9.
-int cluster_size(const qsim_batch *b, int large, int ctas, int *joint) {
-    auto amps = [&](int k) { return (double)(1u << b->nq[b->order[k]]); };
-    double work = 0.0;
-    for (int k = 0; k < large; ++k) work += amps(k);
-    auto shared = [&](int k) {
-        const int n = b->nq[b->order[k]];
-        return n >= 16 && amps(k) * ctas * (n >= 17 ? 2 : 1) > work;
-    };
-    *joint = 0;
-    while (*joint < large && shared(*joint)) ++*joint;
-    const int cl = amps(0) * ctas > 4.0 * work ? 8 : 4;
-    return *joint > 0 && ctas >= cl ? cl : 1;
-}
-
 bool config_valid(const qsim_batch *b, int threads, int m) {
     (void)b;
     return (1 << m) <= reg_amps(threads) * threads;  // in-place permutation through registers
@@ -854,7 +832,7 @@ int launch(qsim_batch *b, int threads, int m, int grid) {
         a.counter = b->d_counter;
         a.begin = 0;
         a.end = large;
-        const int cl = cluster_size(b, large, ggrid, &a.split);
+        const int cl = cluster_size([b](int k) { return b->nq[b->order[k]]; }, large, ggrid, &a.split);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(ggrid / cl * cl);
         cfg.blockDim = dim3(kWinThreads);

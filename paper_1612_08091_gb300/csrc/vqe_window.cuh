@@ -243,4 +243,30 @@ VQE_HD inline void make_pass(Progress &s, int w, Pass &p) {
     }
 }
 
+// CTAs per cluster for the first circuits of the order (qubits(0) >= qubits(1)
+// >= .. qubits(large - 1)), *joint of them, when few circuits hold much of the
+// work; 1 and none when there are enough circuits.  A CTA
+// alone with a circuit ends late if the circuit is more than a CTA's share of
+// the work; of 17 qubits on (16 tiles and more, so that the passes over one
+// tile and their preparation weigh less) sharing pays from half of that on.
+// Milliseconds with 1, 4 and 8 CTAs per circuit, 10..20 qubits: 40 circuits
+// 6.2, 2.1, 1.2; 200: 9.8, 3.9, 2.2; 1024: 14.4, 5.5, 6.3; 4096: 16.7, 19, 20;
+// 13..16 qubits: 1024 circuits 1.2, 1.5, 1.9.
+template <class Qubits>
+inline int cluster_size(Qubits qubits, int large, int ctas, int *joint) {
+    auto amps = [&](int k) { return (double)(1u << qubits(k)); };
+    double work = 0.0;
+    for (int k = 0; k < large; ++k) work += amps(k);
+    auto shared = [&](int k) {
+        const int n = qubits(k);
+        return n >= 16 && amps(k) * ctas * (n >= 17 ? 2 : 1) > work;
+    };
+    *joint = 0;
+    while (*joint < large && shared(*joint)) ++*joint;
+    const int cl = amps(0) * ctas > 4.0 * work ? 8 : 4;
+    if (*joint > 0 && ctas >= cl) return cl;
+    *joint = 0;
+    return 1;
+}
+
 }  // namespace qsim_vqe

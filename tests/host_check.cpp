@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../include/qsim.h"
+#include "../paper_1612_08091_gb300/csrc/vqe_window.cuh"
 
 namespace {
 
@@ -94,12 +95,25 @@ void check_small_queue_under_capture() {
     }
 }
 
+// every circuit of a batch is some CTA's: circuits are set aside for clusters
+// only where clusters are launched
+void check_batch_clusters() {
+    for (int ctas = 1; ctas <= 304; ctas += ctas < 16 ? 1 : 16)
+        for (int top = 13; top <= 24; ++top)
+            for (int large : {1, 2, 5, 40, 400}) {
+                int joint = -1;
+                const int cl = qsim_vqe::cluster_size([&](int k) { return top - (k > 0 ? 1 : 0); }, large, ctas, &joint);
+                CHECK(cl == 1 ? joint == 0 : joint > 0 && joint <= large && cl <= ctas);
+            }
+}
+
 }  // namespace
 
 int main() {
     check_training_sources();
     check_small_queue_falls_back();
     check_small_queue_under_capture();
+    check_batch_clusters();
     std::printf(failures ? "%d failures\n" : "ok\n", failures);
     return failures != 0;
 }
