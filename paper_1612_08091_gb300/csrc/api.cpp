@@ -653,7 +653,10 @@ int sim_apply_gates(qsim *s, int count, const int *kinds, const int *nt, const i
     if (!s) return QSIM_EINVAL;
     if (count < 0 || (count > 0 && (!kinds || !nt || !nc || !targets)))
         return set_err(s, QSIM_EINVAL, "bad gate arguments");
-    s->queue.reserve(s->queue.size() + (size_t)count);
+    // room for all of them at once; at least twice as much as before, so that
+    // many short lists grow the queue in linear time too
+    const size_t need = s->queue.size() + (size_t)count;
+    if (need > s->queue.capacity()) s->queue.reserve(std::max(need, 2 * s->queue.capacity()));
     for (int i = 0; i < count; ++i) {
         double m[32];
         const int t = kinds[i] == QSIM_G_SWAP ? 2 : 1, np = named_params(kinds[i]);

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../include/qsim.h"
+#include "../paper_1612_08091_gb300/csrc/internal.h"
 #include "../paper_1612_08091_gb300/csrc/vqe_window.cuh"
 
 namespace {
@@ -107,6 +108,20 @@ void check_batch_clusters() {
             }
 }
 
+// gates queued in many short lists: the queue moves seldom
+void check_queue_growth() {
+    qsim *s = register_of(20, QSIM_C128);
+    int moves = 0;
+    for (int i = 0; i < 4096; ++i) {
+        const int kind = QSIM_G_H, nt = 1, nc = 0, target = i % 20;
+        const size_t before = s->queue.capacity();
+        CHECK(sim_apply_gates(s, 1, &kind, &nt, &nc, &target, nullptr, nullptr, nullptr) == QSIM_OK);
+        moves += s->queue.capacity() != before;
+    }
+    CHECK(s->queue.size() == 4096 && moves <= 13);
+    sim_destroy(s);
+}
+
 }  // namespace
 
 int main() {
@@ -114,6 +129,7 @@ int main() {
     check_small_queue_falls_back();
     check_small_queue_under_capture();
     check_batch_clusters();
+    check_queue_growth();
     std::printf(failures ? "%d failures\n" : "ok\n", failures);
     return failures != 0;
 }
