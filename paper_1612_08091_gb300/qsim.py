@@ -9,6 +9,7 @@ is no CPU fallback: without the built library or a GPU, construction fails.
 import ctypes
 import itertools
 import math
+import operator
 import os
 
 import numpy as np
@@ -134,6 +135,16 @@ _KINDS = ["H", "X", "Y", "Z", "S", "T", "SWAP", "RX", "RY", "RZ", "R", "U3"]
 _KIND_CODE = {k: i for i, k in enumerate(_KINDS)}
 _KIND_PARAMS = [0] * 7 + [1] * 4 + [3]
 _KIND_TARGETS = [2 if k == "SWAP" else 1 for k in _KINDS]
+_OP_KIND = operator.attrgetter("kind")
+_OP_FIELDS = operator.attrgetter("kind", "targets", "controls", "params")
+_NUMBERS = {float, int, np.float64}
+
+
+def _is_named(op):
+    try:
+        return op.kind in _KIND_CODE
+    except Exception:
+        return False
 
 
 def _ints(seq):
@@ -225,31 +236,45 @@ class Simulator:
         self.apply(_gates.gate_matrix(op.kind, op.params), op.targets, op.controls)
 
     def run(self, ops):
-        """Queue a list of circuitgen-style ops.  Gates named by kind go to
-        the library in one call (sim_apply_gates), which forms their
-        matrices: 0.6 us a gate instead of 5.6 through apply_op."""
-        for named, group in itertools.groupby(ops, key=lambda op: getattr(op, "kind", None) in _KIND_CODE):
+        """Queue circuitgen-style ops.  Of a list or tuple, gates named by
+        kind go to the library in one call (sim_apply_gates), which forms
+        their matrices: 0.6 us a gate instead of 5.6 through apply_op.  The
+        ops of other iterables are queued one by one as they come: the next
+        one may depend on what the handle then holds."""
+        if not isinstance(ops, (list, tuple)):
+            for op in ops:
+                self.apply_op(op)
+            return
+        try:
+            named = set(map(_OP_KIND, ops)) <= _KIND_CODE.keys()
+        except Exception:  # an op without a kind: apply_op refuses it, at its place
+            named = False
+        if named and self._run_named(ops):
+            return
+        for named, group in itertools.groupby(ops, key=_is_named):
             group = list(group)
             for op in group[self._run_named(group) if named else 0:]:
                 self.apply_op(op)
 
     def _run_named(self, ops):
-        """Queue ops of known kinds if they are plain (kind, targets,
-        controls, params) tuples with finite parameters; returns their number,
-        or 0: what it leaves, apply_op takes or refuses."""
+        """Queue ops of known kinds whose fields are plain (as many targets
+        and parameters as the kind has, finite numbers); returns their
+        number, or 0: what it leaves, apply_op takes or refuses."""
         try:
-            kinds, targets, controls, params = zip(*ops)
+            kinds, targets, controls, params = zip(*map(_OP_FIELDS, ops))
             codes = list(map(_KIND_CODE.__getitem__, kinds))
             nt, nc = list(map(len, targets)), list(map(len, controls))
             if list(map(len, params)) != list(map(_KIND_PARAMS.__getitem__, codes)):
                 return 0
             flat = itertools.chain.from_iterable
             targets, controls, params = list(flat(targets)), list(flat(controls)), list(flat(params))
-            if nt != list(map(_KIND_TARGETS.__getitem__, codes)) or not all(map(math.isfinite, params)):
+            if nt != list(map(_KIND_TARGETS.__getitem__, codes)) or not set(map(type, params)) <= _NUMBERS:
+                return 0
+            if not all(map(math.isfinite, params)):
                 return 0
             ints = np.array(codes + nt + nc + targets + controls, dtype=np.int32)
             reals = np.array(params, dtype=np.float64)
-        except (TypeError, ValueError, OverflowError, KeyError):
+        except (AttributeError, TypeError, ValueError, OverflowError, KeyError):
             return 0
         at = ints.ctypes.data
         ip, step = ctypes.POINTER(ctypes.c_int), 4 * len(codes)
