@@ -786,7 +786,7 @@ int occupancy_global(const qsim_batch *b, int *grid) {
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWinThreads, kWinSmem);
     if (e != cudaSuccess || per_sm < 1) return QSIM_ENOTSUP;
-    *grid = std::min(b->sms * per_sm, b->max_grid);
+    *grid = b->sms * std::min(per_sm, kWinCtas);  // a buffer each
     return QSIM_OK;
 }
 
@@ -905,10 +905,10 @@ int sim_batch_workspace_bytes(int count, const int *nqubits, const int *layers, 
         cudaGetLastError();
         return QSIM_ECUDA;
     }
-    const size_t max_grid = (size_t)sms * 4;
+    const size_t buffers = (size_t)sms * kWinCtas;  // one per CTA of k_vqe_window
     const size_t gstride = nmax > 12 ? ((size_t)1 << nmax) : 0;
     size_t s = align256(sizeof(double) * nang) + align256(sizeof(double) * count) + 3 * align256(sizeof(int) * count) +
-               align256(sizeof(long long) * count) + 256 + max_grid * gstride * sizeof(float2);
+               align256(sizeof(long long) * count) + 256 + buffers * gstride * sizeof(float2);
     *bytes = s;
     return QSIM_OK;
 }

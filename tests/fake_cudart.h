@@ -31,6 +31,8 @@ inline int sms = 152;              // multiprocessors of the device
 inline const char *fail_launch = nullptr;  // launches of kernels whose name holds this fail
 inline int fail_attribute = 0;     // cudaFuncSetAttribute fails
 inline int capturing = 0;          // streams are being captured
+inline int ctas_per_sm = 2;        // occupancy of any kernel
+inline unsigned grid = 0;          // CTAs of the last cudaLaunchKernelEx
 inline int copies = 0;             // copies from host memory
 inline int clusters = 1;           // clusters of any size that the device can hold
 inline cudaError_t last = cudaSuccess;
@@ -108,7 +110,10 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) {
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **, size_t, cudaStream_t) {
     return fake::launch((const void *)k);
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *, const void *f, void **) { return fake::launch(f); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **) {
+    fake::grid = c->gridDim.x;
+    return fake::launch(f);
+}
 cudaError_t cudaGetLastError() {
     const cudaError_t e = fake::last;
     fake::last = cudaSuccess;
@@ -169,7 +174,7 @@ cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) {
-    return *n = 2, cudaSuccess;
+    return *n = fake::ctas_per_sm, cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *) {
     return *n = fake::clusters, cudaSuccess;

@@ -122,6 +122,24 @@ void check_queue_growth() {
     sim_destroy(s);
 }
 
+// a batch reserves a state for every CTA that works on one, and no more
+void check_batch_buffers() {
+    const std::vector<int> nq(400, 15), nl(400, 2);
+    std::vector<double> angles(400 * 60, 0.1), energies(400);
+    for (int per_sm : {1, 2, 4}) {
+        fake::ctas_per_sm = per_sm;
+        size_t bytes = 0;
+        CHECK(sim_batch_workspace_bytes(400, nq.data(), nl.data(), &bytes) == QSIM_OK);
+        qsim_batch *b = nullptr;
+        CHECK(sim_batch_create(400, nq.data(), nl.data(), 0.7, nullptr, nullptr, 0, &b) == QSIM_OK);
+        CHECK(sim_batch_run(b, angles.data(), energies.data()) == QSIM_OK);
+        const size_t state = sizeof(float) * 2 << 15, rest = sizeof(double) * angles.size() + 65536;
+        CHECK(fake::grid * state < bytes && bytes <= 2 * fake::sms * state + rest);
+        sim_batch_destroy(b);
+    }
+    fake::ctas_per_sm = 2;
+}
+
 }  // namespace
 
 int main() {
@@ -130,6 +148,7 @@ int main() {
     check_small_queue_under_capture();
     check_batch_clusters();
     check_queue_growth();
+    check_batch_buffers();
     std::printf(failures ? "%d failures\n" : "ok\n", failures);
     return failures != 0;
 }
