@@ -28,7 +28,7 @@
 // their products with Paulis) do not mix all four components, and FP64 keeps
 // the two sets that they do mix apart: there each set has an exponent of its
 // own (Apart), so that a result's component is as exact, against the components
-// it comes from, as in FP64.  Zeros of either sign are exact.
+// it comes from, as in FP64, and zeros of either sign are exact.
 //
 // Groups whose exponent is near the ends of the range, and infinities and
 // NaN, are left to FP64 (fx_range).
@@ -70,8 +70,19 @@ __device__ __forceinline__ long long shr_s64(long long v, uint32_t s) {
 #endif
 }
 
-// x 2^(1081 - E) without its fraction; E >= the biased exponent of x, E > 64
+// floor(x 2^(1081 - E)) (one less for some exact negative values and -0.0);
+// E >= the biased exponent of x
 __device__ __forceinline__ Fx to_fx(double x, int E) {
+    const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+    const unsigned long long m = (((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | l) << 6;
+    const uint32_t sg = (uint32_t)((int)h >> 31);
+    long long v = (long long)(m ^ (((unsigned long long)sg << 32) | sg));
+    v = shr_s64(v, (uint32_t)(E - (int)((h >> 20) & 0x7FFu)));
+    return Fx{(int)(v >> 28), (int)((uint32_t)v & 0xFFFFFFFu)};
+}
+// the same rounded towards zero (E > 64): exact zeros and negative values
+// (with it a gate that mixes all components takes 3.5 % longer)
+__device__ __forceinline__ Fx to_fx_exact(double x, int E) {
     const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
     const unsigned long long m = (((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | l) << 6;
     const long long sg = (int)h >> 31;
@@ -111,37 +122,39 @@ __device__ __forceinline__ double to_double(const Acc &s, int eadd) {
 }
 
 // ---------------------------------------------------------------------------
-// gates on several qubits: 51 bits, the cross sums in FP32
+// gates on several qubits: 55 bits, the cross sums in FP32
 // ---------------------------------------------------------------------------
-// For the handles that allow double-float accuracy.  v = x 2^(1073 - E) = hi
-// 2^25 + lo with 26 bits and a sign in hi; a matrix element w = m 2^S in the
-// same form (lo rounded to nearest, -2^24..2^24), scaled so that its largest
-// row sum of |re| + |im| is below 2^52.  The sum of hi hi' is exact in 64 bits
-// (one multiply-add a product, four cycles of a pipe that plain FP32 does not
-// need); the cross terms, 2^-25 of it, go to an FP32 sum, which is off by some
-// 2^-24 of that.  Error of a result: some 2^-48 of the group's largest
-// amplitude.
+// For the handles that allow double-float accuracy.  v = x 2^(1077 - E) = hi
+// 2^25 + lo with 30 bits and a sign in hi, lo rounded to nearest (-2^24..2^24);
+// a matrix element w = m 2^S in the same form, scaled so that its largest row
+// sum of |re| + |im| is below 2^55.  The sum of hi hi' is exact in 64 bits (one
+// multiply-add a product, four cycles of a pipe that plain FP32 does not
+// need); the cross terms, 2^-30 of it, go to two FP32 sums.  Error of a result:
+// 2^-54 (standard deviation) to 2^-51 of U, the largest row sum times the
+// group's largest component, each rounded up to a power of two (random 2- to
+// 4-qubit unitaries).
 struct FxF {  // an amplitude's component
     int hi;
-    float fhi, flo;  // hi rounded, lo exact
+    float fhi, flo;  // hi and lo, hi rounded
 };
 __device__ __forceinline__ FxF to_fxf(double x, int E) {
     const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+    const unsigned long long m = (((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | l) << 2;
     const uint32_t sg = (uint32_t)((int)h >> 31);
-    const unsigned long long m =
-        ((unsigned long long)(((h & 0xFFFFFu) | 0x100000u) ^ sg) << 32) | (unsigned long long)(l ^ sg);
-    const long long v = shr_s64((long long)m, (uint32_t)(E + 2 - (int)((h >> 20) & 0x7FFu)));
+    const long long v = shr_s64((long long)(m ^ (((unsigned long long)sg << 32) | sg)),
+                                (uint32_t)(E - (int)((h >> 20) & 0x7FFu)));
     FxF r;
-    r.hi = (int)(v >> 25);
+    r.hi = (int)((v + (1 << 24)) >> 25);
     r.fhi = (float)r.hi;
-    r.flo = (float)((uint32_t)v & 0x1FFFFFFu);
+    r.flo = (float)((int)v - (int)((uint32_t)r.hi << 25));
     return r;
 }
-// a 2^50 + c 2^25 as a double: units of 2^(E - 1073 - S); eadd = (E - 1023 - S)
-// 2^20.  |c| < 2^55.2: sum |w.hi| < 2^27 times lo < 2^25, and up to 32 terms
-// of |w.lo| <= 2^24 times |hi| <= 2^26.
+// a 2^50 + c 2^25 as a double: units of 2^(E - 1077 - S); eadd = (E - 1027 - S)
+// 2^20.  |c| <= 2^54 + 2^59: sum |w.hi| <= 2^30 times |lo| <= 2^24, and up to 32
+// terms of |w.lo| <= 2^24 times |hi| <= 2^30; it is rounded to 2^8 units of a,
+// 2^-52 of the largest a.
 __device__ __forceinline__ double to_double_f(long long a, float c, int eadd) {
-    const double d = (double)(a + (long long)__float2int_rn(c * 0x1p-25f));
+    const double d = (double)mad_wide(__float2int_rn(c * 0x1p-33f), 256, a);
     const int h = __double2hiint(d);
     return __hiloint2double(h ? h + eadd : 0, __double2loint(d));
 }
@@ -184,7 +197,7 @@ struct Side {
 };
 __device__ __forceinline__ Side side(double a, double b) {
     const int E = (int)(max(mag(a), mag(b)) >> 20);
-    if (fx_range(E)) return Side{to_fx(a, E), to_fx(b, E), E};
+    if (fx_range(E)) return Side{to_fx_exact(a, E), to_fx_exact(b, E), E};
     return Side{Fx{0, 0}, Fx{0, 0}, a == 0.0 && b == 0.0 ? 0 : -1};
 }
 __device__ __forceinline__ double side_sum(const MatFx &M, Fx wa, Fx wb, const Side &s) {

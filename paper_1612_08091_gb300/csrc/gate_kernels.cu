@@ -254,23 +254,84 @@ __global__ void __launch_bounds__(256) k_phase_df(double2 *__restrict__ psi, uin
         if (g0 + u * blockDim.x < ngroups) psi[i[u]] = qsim_df::to_double(qsim_df::cmul(M.m[3], qsim_df::split(v[u])));
 }
 
+// complex128 5-qubit dense gate or fused block in double-float arithmetic, and
+// narrower ones that the integer form does not fit: the group's 2^k amplitudes
+// split into FP32 pairs, each output the sum of 2^k exact-product complex MACs
+// with two-sum additions, rounded once to double.  About 40 FP32 operations per
+// MAC instead of 4 FP64 FMAs (FP64 runs at 1/58 of the FP32 rate here).
+template <int K>
+__device__ __forceinline__ void dense_pairs(double2 *p, const qsim_df::C2 *m, const uint64_t *off) {
+    constexpr int D = 1 << K;
+    qsim_df::C2 v[D];
+#pragma unroll
+    for (int r = 0; r < D; ++r) v[r] = qsim_df::split(p[off[r]]);
+#pragma unroll 1
+    for (int r = 0; r < D; ++r) {
+        // four partial sums: each addition rounds the low parts
+        qsim_df::C2 acc[4];
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            const qsim_df::C2 z = qsim_df::cmul(m[r * D + c], v[c]);
+            acc[c & 3] = c < 4 ? z : qsim_df::cadd(acc[c & 3], z);
+        }
+        p[off[r]] =
+            qsim_df::to_double(qsim_df::cadd(qsim_df::cadd(acc[0], acc[1]), qsim_df::cadd(acc[2], acc[3])));
+    }
+}
+
+// the same in FP64 arithmetic
+template <int K>
+__device__ __forceinline__ void dense_fp64(double2 *p, const qsim_df::C2 *m, const uint64_t *off) {
+    constexpr int D = 1 << K;
+    double2 v[D];
+#pragma unroll
+    for (int r = 0; r < D; ++r) v[r] = p[off[r]];
+#pragma unroll 1
+    for (int r = 0; r < D; ++r) {
+        double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            const qsim_df::C2 w = m[r * D + c];
+            acc = cfma(make_double2((double)w.re.hi + w.re.lo, (double)w.im.hi + w.im.lo), v[c], acc);
+        }
+        p[off[r]] = acc;
+    }
+}
+
+template <int K> struct MatKDF { qsim_df::C2 m[(1 << K) * (1 << K)]; uint64_t off[1 << K]; };
+
+template <int K>
+__global__ void __launch_bounds__(128) k_denseK_df(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
+                                                   uint64_t cmask, const MatKDF<K> M) {
+    const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (g >= ngroups) return;
+    dense_pairs<K>(psi + (insert_zeros(g, ins) | cmask), M.m, M.off);
+}
+
 // complex128 k-qubit dense gate or fused block where the handle allows
 // double-float accuracy, in shared-exponent integers and FP32 (fx128.cuh): a
 // thread takes a group's 2^k amplitudes; a complex product is 4 integer
 // multiply-adds and 8 FP32 ones, on two halves of the FMA pipe, where pairs of
-// FP32 took 48 operations; one FP64 conversion per result.  26 qubits, 4-qubit
-// blocks: 0.80 ms a pass (2.69 TB/s) against 1.59 ms, bound by issue (69 %) and
-// the integer multiply-adds (60 % of their pipe); a 27-pass circuit ends 6.0e-14
-// from 64 bits, with pairs 6.2e-14.  (With the cross sums in integers too, 9
-// multiply-adds a product: 1.4e-15, but 1.09 ms a pass.)
+// FP32 took 48 operations; one FP64 conversion per result.
+// The error of this form is relative to the group's largest amplitude, that of
+// pairs (2^-45) to a result's own products.  So each row's sum of |m| |v| is
+// looked at first (a lower bound from the least elements of a quarter's rows;
+// where that is too small, the sum): where all are at least kFxRow of U
+// (fx128.cuh) the error is below 2^-45 of them; where one is not (amplitudes of
+// very different sizes under rows that do not mix them), the warp computes in
+// pairs, as the 5-qubit kernel.
 template <int K> struct MatKFx {
     // each element's re and im (hi, hi rounded, lo) for 16- and 8-byte loads
     int4 a[(1 << K) * (1 << K)];    // re hi, im hi, and both as floats
     float2 b[(1 << K) * (1 << K)];  // re lo, im lo
+    qsim_df::C2 m[(1 << K) * (1 << K)];
+    float w[(1 << K) * (1 << K)];   // |element|, the largest row sum being 1/2 to 1
+    float low[4][1 << K];           // the least of each quarter of a column
     uint64_t off[1 << K];
-    int shift;                    // -1023 - S
-    double unit;                  // 2^-S
+    int shift;                    // -1027 - S
+    int pairs;                    // rows that hardly mix: in pairs throughout
 };
+constexpr float kFxRow = 0x1p-6f;
 
 template <int K>
 __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
@@ -293,18 +354,7 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
 #pragma unroll
         for (int r = 0; r < D; ++r) zero = zero && v[r].x == 0.0 && v[r].y == 0.0;
         if (zero) return;
-        // amplitudes near the ends of the range: FP64
-#pragma unroll 1
-        for (int r = 0; r < D; ++r) {
-            double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int c = 0; c < D; ++c) {
-                const int4 w = M.a[r * D + c];
-                const float2 l = M.b[r * D + c];
-                acc = cfma(make_double2((w.x * 0x1p25 + l.x) * M.unit, (w.y * 0x1p25 + l.y) * M.unit), v[c], acc);
-            }
-            p[M.off[r]] = acc;
-        }
+        dense_fp64<K>(p, M.m, M.off);  // amplitudes near the ends of the range
         return;
     }
     FxF xr[D], xi[D];
@@ -313,11 +363,45 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
         xr[r] = to_fxf(v[r].x, E);
         xi[r] = to_fxf(v[r].y, E);
     }
+    {
+        float size[D], low = M.pairs ? 0.f : 0x1p30f;
+#pragma unroll
+        for (int c = 0; c < D; ++c) size[c] = fmaxf(fabsf(xr[c].fhi), fabsf(xi[c].fhi));
+        // at first a lower bound for the rows of a quarter
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float t = 0.f;
+#pragma unroll
+            for (int c = 0; c < D; ++c) t = fmaf(M.low[q][c], size[c], t);
+            low = fminf(low, t);
+        }
+        bool pairs = __any_sync(__activemask(), low < kFxRow * 0x1p30f);
+        if (pairs && !M.pairs) {
+            low = 0x1p30f;
+#pragma unroll 2
+            for (int r = 0; r < D; ++r) {
+                float t = 0.f;
+#pragma unroll
+                for (int c = 0; c < D; ++c) t = fmaf(M.w[r * D + c], size[c], t);
+                low = fminf(low, t);
+            }
+            pairs = __any_sync(__activemask(), low < kFxRow * 0x1p30f);
+        }
+        if (pairs) {
+            // pairs hold 2^-126 to 2^127
+            if (E > 1023 - 60 && E < 1023 + 60)
+                dense_pairs<K>(p, M.m, M.off);
+            else
+                dense_fp64<K>(p, M.m, M.off);
+            return;
+        }
+    }
     const int eadd = (E + M.shift) << 20;
 #pragma unroll 2
     for (int r = 0; r < D; ++r) {
         long long rr = 0, ii = 0, ri = 0;  // sums of mr xr, mi xi, mr xi + mi xr
-        float cr = 0.f, ci = 0.f;          // cross sums of the two results
+        float cr = 0.f, ci = 0.f;          // cross sums of the two results: hi by lo
+        float dr = 0.f, di = 0.f;          // and lo by hi
 #pragma unroll
         for (int c = 0; c < D; ++c) {
             const int4 w = M.a[r * D + c];
@@ -328,41 +412,15 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
             ri = mad_wide(w.x, xi[c].hi, ri);
             ri = mad_wide(w.y, xr[c].hi, ri);
             cr = fmaf(frh, xr[c].flo, cr);
-            cr = fmaf(l.x, xr[c].fhi, cr);
+            dr = fmaf(l.x, xr[c].fhi, dr);
             cr = fmaf(-fih, xi[c].flo, cr);
-            cr = fmaf(-l.y, xi[c].fhi, cr);
+            dr = fmaf(-l.y, xi[c].fhi, dr);
             ci = fmaf(frh, xi[c].flo, ci);
-            ci = fmaf(l.x, xi[c].fhi, ci);
+            di = fmaf(l.x, xi[c].fhi, di);
             ci = fmaf(fih, xr[c].flo, ci);
-            ci = fmaf(l.y, xr[c].fhi, ci);
+            di = fmaf(l.y, xr[c].fhi, di);
         }
-        p[M.off[r]] = make_double2(to_double_f(rr - ii, cr, eadd), to_double_f(ri, ci, eadd));
-    }
-}
-
-// complex128 5-qubit dense gate or fused block in double-float arithmetic:
-// the group's 2^k amplitudes split into FP32 pairs, each output the sum of
-// 2^k exact-product complex MACs with two-sum additions, rounded once to
-// double.  About 40 FP32 operations per MAC instead of 4 FP64 FMAs (FP64
-// runs at 1/58 of the FP32 rate here).
-template <int K> struct MatKDF { qsim_df::C2 m[(1 << K) * (1 << K)]; uint64_t off[1 << K]; };
-
-template <int K>
-__global__ void __launch_bounds__(128) k_denseK_df(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
-                                                   uint64_t cmask, const MatKDF<K> M) {
-    constexpr int D = 1 << K;
-    const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (g >= ngroups) return;
-    const uint64_t base = insert_zeros(g, ins) | cmask;
-    qsim_df::C2 v[D];
-#pragma unroll
-    for (int r = 0; r < D; ++r) v[r] = qsim_df::split(psi[base + M.off[r]]);
-#pragma unroll 1
-    for (int r = 0; r < D; ++r) {
-        qsim_df::C2 acc = qsim_df::cmul(M.m[r * D], v[0]);
-#pragma unroll
-        for (int c = 1; c < D; ++c) acc = qsim_df::cadd(acc, qsim_df::cmul(M.m[r * D + c], v[c]));
-        psi[base + M.off[r]] = qsim_df::to_double(acc);
+        p[M.off[r]] = make_double2(to_double_f(rr - ii, cr + dr, eadd), to_double_f(ri, ci + di, eadd));
     }
 }
 
@@ -490,17 +548,24 @@ int dense_k_fx(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
         M.off[r] = o;
     }
     double rows = 0.0;  // largest sum of |re| + |im| of a row
+    bool mixes = true;
     for (int r = 0; r < D; ++r) {
-        double t = 0.0;
-        for (int c = 0; c < D; ++c) t += std::abs(m[r * D + c].real()) + std::abs(m[r * D + c].imag());
+        double t = 0.0, sum = 0.0, top = 0.0;
+        for (int c = 0; c < D; ++c) {
+            const cd z = m[r * D + c];
+            t += std::abs(z.real()) + std::abs(z.imag());
+            sum += std::abs(z);
+            top = std::max(top, std::abs(z));
+        }
         rows = std::max(rows, t);
+        mixes = mixes && sum >= 1.125 * top;
     }
     // a zero or an extreme matrix: FP64
     if (!(rows > qsim_fx::kFxMatrixLow) || !(rows < qsim_fx::kFxMatrixTop))
         return dense_k_plain<double2, K>(s, targets, cmask, m);
     int x;
     std::frexp(rows, &x);  // rows < 2^x
-    const int S = 52 - x;
+    const int S = 55 - x;
     for (int i = 0; i < D * D; ++i) {
         auto part = [&](double v, int &hi, float &fhi, float &flo) {
             const long long w = std::llrint(std::ldexp(v, S));
@@ -513,9 +578,18 @@ int dense_k_fx(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
         part(m[i].imag(), M.a[i].y, fi, M.b[i].y);
         std::memcpy(&M.a[i].z, &fr, 4);
         std::memcpy(&M.a[i].w, &fi, 4);
+        M.m[i] = qsim_df::C2{host_split(m[i].real()), host_split(m[i].imag())};
+        M.w[i] = (float)std::ldexp(std::abs(m[i]), -x);
     }
-    M.shift = -1023 - S;
-    M.unit = std::ldexp(1.0, -S);
+    for (int q = 0; q < 4; ++q)
+        for (int c = 0; c < D; ++c) {
+            M.low[q][c] = M.w[q * (D / 4) * D + c];
+            for (int r = q * (D / 4); r < (q + 1) * (D / 4); ++r) M.low[q][c] = std::min(M.low[q][c], M.w[r * D + c]);
+        }
+    M.shift = -1027 - S;
+    // a row of one amplitude (permutations, controlled gates): the sums that the
+    // kernel looks at are small in most warps, and pairs multiply by 1 exactly
+    M.pairs = !mixes;
     const InsertSpec ins = make_spec(tmask | cmask);
     const uint64_t ngroups = 1ull << (s->n - ins.m);
     k_denseK_fx<K><<<blocks_for(ngroups, 128), 128, 0, s->stream>>>((double2 *)s->state, ngroups, ins, cmask, M);
@@ -530,8 +604,10 @@ int dense_k(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
         // pairs, whose plans the narrower blocks beat either way (27 qubits,
         // depth 10: 56 ms with 4-qubit blocks, 69 ms with integer 5-qubit ones)
         if (s->c128_df) {
-            if constexpr (K <= 4) return dense_k_fx<K>(s, targets, cmask, m);
-            return dense_k_df<K>(s, targets, cmask, m);
+            if constexpr (K <= 4)
+                return dense_k_fx<K>(s, targets, cmask, m);
+            else
+                return dense_k_df<K>(s, targets, cmask, m);
         }
     }
     return dense_k_plain<Amp, K>(s, targets, cmask, m);
