@@ -564,8 +564,8 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_x(const Amp *__restrict_
 // memory (one asynchronous copy in, three reads).  Element e sits at position
 // e ^ ((e >> 5) & 7) << 1: an amplitude pair stays one aligned 16-byte slot,
 // eight lanes of layout A meet eight different slots.
-// Rounding.  A term's pairs are added eight at a time in FP32, in a tree; two
-// such sums, their product with the coefficient and the terms of a tile are
+// Rounding.  A term's pairs are added eight at a time in FP32 (four and four);
+// two such sums, their product with the coefficient and the terms of a tile are
 // added with their rounding errors kept (x_term), tiles in FP64.  So FP32
 // rounds what it rounds in k_expect_x, sums of eight pairs, and the
 // coefficients stay doubles.  Registers where a thread of k_expect_x has fewer
@@ -581,38 +581,39 @@ constexpr int kXMinRun = 3;  // runs of at least 2^3 amplitudes
 struct XTileArgs {
     uint64_t ntiles;       // 2^(n - 13)
     InsertSpec vspec;      // V, ascending
-    double c[kXBits];      // 2 c_q of the qubit at tile bit j (0: no term)
+    double c[kXBits];      // 2 c_q of the qubit at tile bit j, times 1 / scale (0: no term)
     float ch[kXBits], cl[kXBits];  // the same as a pair of FP32
+    double scale;          // a power of two: the largest c_q is about 1
     uint32_t mask;         // tile bits with a term
 };
 
 __device__ __forceinline__ uint32_t xswz(uint32_t e) { return e ^ (((e >> 5) & 7u) << 1); }
 
-// the k-th of the pairs of register bit r: Re v_i conj(v_j)
+// s + Re v_i conj(v_j) of the k-th of the pairs of register bit r
 template <int N>
-__device__ __forceinline__ float x_pair(const float2 (&v)[N], int r, int k) {
+__device__ __forceinline__ float x_pair(const float2 (&v)[N], int r, int k, float s) {
     const int i = ((k >> r) << (r + 1)) | (k & ((1 << r) - 1));
     const float2 a = v[i], b = v[i | (1 << r)];
-    return fmaf(a.x, b.x, a.y * b.y);
+    return fmaf(a.x, b.x, fmaf(a.y, b.y, s));
 }
-// sum of M pairs from the k0-th on, in a tree
-template <int M, int N>
-__device__ __forceinline__ float x_pairs(const float2 (&v)[N], int r, int k0) {
-    float t[M];
+// sum of four pairs from the k0-th on
+template <int N>
+__device__ __forceinline__ float x_four(const float2 (&v)[N], int r, int k0) {
+    float t = 0.f;
 #pragma unroll
-    for (int k = 0; k < M; ++k) t[k] = x_pair(v, r, k0 + k);
-#pragma unroll
-    for (int w = M / 2; w; w >>= 1)
-#pragma unroll
-        for (int k = 0; k < w; ++k) t[k] = __fadd_rn(t[k], t[k + w]);
-    return t[0];
+    for (int k = 0; k < 4; ++k) t = x_pair(v, r, k0 + k, t);
+    return t;
+}
+template <int N>
+__device__ __forceinline__ float x_eight(const float2 (&v)[N], int r, int k0) {
+    return __fadd_rn(x_four(v, r, k0), x_four(v, r, k0 + 4));
 }
 // all pairs in FP64
 template <int N>
 __device__ __forceinline__ double x_pairs_fine(const float2 (&v)[N], int r) {
     double s = 0.0;
 #pragma unroll
-    for (int k = 0; k < N / 2; ++k) s += (double)x_pair(v, r, k);
+    for (int k = 0; k < N / 2; ++k) s += (double)x_pair(v, r, k, 0.f);
     return s;
 }
 // (hi, lo) += (ch + cl) (a + b), with the errors of the sums and of the
@@ -669,7 +670,7 @@ __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const
                 if (Fine)
                     acc = fma(A.c[base + r], x_pairs_fine(v, r), acc);
                 else
-                    x_term(hi, lo, x_pairs<8>(v, r, 0), x_pairs<8>(v, r, 8), A.ch[base + r], A.cl[base + r]);
+                    x_term(hi, lo, x_eight(v, r, 0), x_eight(v, r, 8), A.ch[base + r], A.cl[base + r]);
             }
         };
         if (mA) {
@@ -701,7 +702,7 @@ __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const
                     if (Fine)
                         acc = fma(A.c[10 + r], x_pairs_fine(v, r), acc);
                     else
-                        h[r][s] = x_pairs<4>(v, r, 0);
+                        h[r][s] = x_four(v, r, 0);
                 }
             }
             if (!Fine) {
@@ -714,7 +715,7 @@ __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const
         }
         if (!Fine) acc += (double)hi + (isfinite(hi) ? (double)lo : 0.0);
     }
-    acc = block_sum(acc, sh);
+    acc = block_sum(acc * A.scale, sh);
     if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 
@@ -1008,7 +1009,7 @@ int collapse_t(qsim *s, uint64_t mask, uint64_t value, double scale) {
 // read; the high ones spread evenly, so that the runs are as long as they
 // can be.
 template <typename Room>
-int field_passes(qsim *s, uint64_t field, const double *c, unsigned *filled, Room room) {
+int field_passes(qsim *s, uint64_t field, const double *c, double scale, unsigned *filled, Room room) {
     const int n = s->n, per = kXBits - kXMinRun;
     int hi[kMaxQubits], nhi = 0;
     for (int b = kXBits; b < n; ++b)
@@ -1026,6 +1027,7 @@ int field_passes(qsim *s, uint64_t field, const double *c, unsigned *filled, Roo
     uint64_t done = 0;
     for (int p = -1; p < passes; ++p) {
         XTileArgs A{};
+        A.scale = scale;
         uint64_t V = 0;
         if (p >= 0)  // high qubits p * nhi / passes ..
             for (int j = p * nhi / passes; j < (p + 1) * nhi / passes; ++j) V |= 1ull << hi[j];
@@ -1037,7 +1039,7 @@ int field_passes(qsim *s, uint64_t field, const double *c, unsigned *filled, Roo
             if ((V >> b) & 1ull) {
                 if (((field & ~done) >> b) & 1ull) {
                     A.mask |= 1u << k;
-                    A.c[k] = 2.0 * c[b];
+                    A.c[k] = 2.0 * c[b] / scale;
                     A.ch[k] = (float)A.c[k];
                     A.cl[k] = (float)(A.c[k] - (double)A.ch[k]);
                 }
@@ -1131,12 +1133,16 @@ int expect_t(qsim *s, const qsim_pauli *terms, int nterms, double *out) {
                     field |= terms[k].xmask;
                     c[__builtin_ctzll(terms[k].xmask)] += terms[k].coeff;
                 }
-            // coefficients that FP32 pairs do not hold, and sums of 0, term by term
+            // relative to the largest coefficient FP32 pairs hold the others down to
+            // 2^-100 of it; smaller ones, and sums of 0, term by term
+            double top = 0.0;
+            for (int b = 0; b < n; ++b) top = std::max(top, std::abs(c[b]));
+            const double scale = top > 0x1p-900 && top < 0x1p900 ? std::ldexp(1.0, std::ilogb(top)) : 0.0;
             for (int b = 0; b < n; ++b)
-                if (!(std::abs(c[b]) >= 0x1p-100) || !(std::abs(c[b]) <= 0x1p100)) field &= ~(1ull << b);
+                if (!(std::abs(c[b]) > 0x1p-100 * scale) || scale == 0.0) field &= ~(1ull << b);
             // one term takes one read either way (k_expect_x then reads it)
             if (__builtin_popcountll(field) < 2) field = 0;
-            if ((rc = field ? field_passes(s, field, c, &filled, room) : QSIM_OK)) return rc;
+            if ((rc = field ? field_passes(s, field, c, scale, &filled, room) : QSIM_OK)) return rc;
         }
     }
     // strings with an X part, grouped by X mask
