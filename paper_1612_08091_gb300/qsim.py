@@ -135,9 +135,16 @@ _KINDS = ["H", "X", "Y", "Z", "S", "T", "SWAP", "RX", "RY", "RZ", "R", "U3"]
 _KIND_CODE = {k: i for i, k in enumerate(_KINDS)}
 _KIND_PARAMS = [0] * 7 + [1] * 4 + [3]
 _KIND_TARGETS = [2 if k == "SWAP" else 1 for k in _KINDS]
-_OP_KIND = operator.attrgetter("kind")
-_OP_FIELDS = operator.attrgetter("kind", "targets", "controls", "params")
+_FIELDS = ("kind", "targets", "controls", "params")
+_OP_FIELDS = operator.attrgetter(*_FIELDS)
 _NUMBERS = {float, int, np.float64}
+
+
+def _plain_tuples(ops):
+    """Named tuples of one type with these fields in this order."""
+    types = set(map(type, ops))
+    t = types.pop() if len(types) == 1 else None
+    return t is not None and t.__bases__ == (tuple,) and getattr(t, "_fields", None) == _FIELDS
 
 
 def _is_named(op):
@@ -245,11 +252,7 @@ class Simulator:
             for op in ops:
                 self.apply_op(op)
             return
-        try:
-            named = set(map(_OP_KIND, ops)) <= _KIND_CODE.keys()
-        except Exception:  # an op without a kind: apply_op refuses it, at its place
-            named = False
-        if named and self._run_named(ops):
+        if self._run_named(ops):
             return
         for named, group in itertools.groupby(ops, key=_is_named):
             group = list(group)
@@ -261,7 +264,7 @@ class Simulator:
         and parameters as the kind has, finite numbers); returns their
         number, or 0: what it leaves, apply_op takes or refuses."""
         try:
-            kinds, targets, controls, params = zip(*map(_OP_FIELDS, ops))
+            kinds, targets, controls, params = zip(*(ops if _plain_tuples(ops) else map(_OP_FIELDS, ops)))
             codes = list(map(_KIND_CODE.__getitem__, kinds))
             nt, nc = list(map(len, targets)), list(map(len, controls))
             if list(map(len, params)) != list(map(_KIND_PARAMS.__getitem__, codes)):
@@ -274,7 +277,7 @@ class Simulator:
                 return 0
             ints = np.array(codes + nt + nc + targets + controls, dtype=np.int32)
             reals = np.array(params, dtype=np.float64)
-        except (AttributeError, TypeError, ValueError, OverflowError, KeyError):
+        except Exception:  # nothing queued yet: one by one, refused at its place
             return 0
         at = ints.ctypes.data
         ip, step = ctypes.POINTER(ctypes.c_int), 4 * len(codes)
