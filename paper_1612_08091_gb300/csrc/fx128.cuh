@@ -220,21 +220,27 @@ __device__ __forceinline__ bool apart_sides(const MatFx &M, double2 a, double2 b
     return p.E >= 0 && q.E >= 0;
 }
 
-// (na, nb) = M (a, b)
+// (na, nb) = M (a, b); Apart as M.apart
+template <bool Apart>
 __device__ __forceinline__ void dense1(const MatFx &M, double2 a, double2 b, double2 &na, double2 &nb) {
-    const int E = (int)(max(mag(a), mag(b)) >> 20);
-    Side p, q;
-    if (M.apart && apart_sides(M, a, b, p, q)) {
-        na = apart_row(M, 0, p, q);
-        nb = apart_row(M, 1, p, q);
-    } else if (!M.apart && fx_range(E)) {
-        const Fx ar = to_fx(a.x, E), ai = to_fx(a.y, E), br = to_fx(b.x, E), bi = to_fx(b.y, E);
-        na = row(M, 0, ar, ai, br, bi, E);
-        nb = row(M, 1, ar, ai, br, bi, E);
+    if constexpr (Apart) {
+        Side p, q;
+        if (apart_sides(M, a, b, p, q)) {
+            na = apart_row(M, 0, p, q);
+            nb = apart_row(M, 1, p, q);
+            return;
+        }
     } else {
-        na = row_fp64(M, 0, a, b);
-        nb = row_fp64(M, 1, a, b);
+        const int E = (int)(max(mag(a), mag(b)) >> 20);
+        if (fx_range(E)) {
+            const Fx ar = to_fx(a.x, E), ai = to_fx(a.y, E), br = to_fx(b.x, E), bi = to_fx(b.y, E);
+            na = row(M, 0, ar, ai, br, bi, E);
+            nb = row(M, 1, ar, ai, br, bi, E);
+            return;
+        }
     }
+    na = row_fp64(M, 0, a, b);
+    nb = row_fp64(M, 1, a, b);
 }
 // one row of it
 __device__ __forceinline__ double2 dense1_row(const MatFx &M, int r, double2 a, double2 b) {

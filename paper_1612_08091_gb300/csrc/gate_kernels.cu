@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(256) k_dense1(Amp *__restrict__ psi, uint64_t 
 // qubits 0.43 ms on a full state (5.0 TB/s, 74 % of HBM; 0.31 ms while most
 // groups are zero) against 1.03 ms in FP64 arithmetic; bound by the integer
 // multiply-add pipe.
-template <int kGroups>
+template <int kGroups, bool Apart>
 __global__ void __launch_bounds__(256) k_dense1_fx(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                    uint64_t cmask, uint64_t tbit, const qsim_fx::MatFx M) {
     const uint64_t g0 = blockIdx.x * (uint64_t)(blockDim.x * kGroups) + threadIdx.x;
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256) k_dense1_fx(double2 *__restrict__ psi, ui
     for (int u = 0; u < kGroups; ++u) {
         if (g0 + u * blockDim.x >= ngroups) continue;
         double2 na, nb;
-        qsim_fx::dense1(M, a[u], b[u], na, nb);
+        qsim_fx::dense1<Apart>(M, a[u], b[u], na, nb);
         psi[i0[u]] = na;
         psi[i0[u] | tbit] = nb;
     }
@@ -654,12 +654,12 @@ int gate_plain(qsim *s, const GateRec &g) {
             if constexpr (sizeof(Amp) == 16) {
                 qsim_fx::MatFx F;
                 if (qsim_fx::make_fx(g.m.data(), F)) {
-                    if (narrow(s, ngroups, kWideFx))
-                        k_dense1_fx<1><<<blocks_for(ngroups, kNarrowThreads), kNarrowThreads, 0, s->stream>>>(
-                            psi, ngroups, ins, g.cmask, tbit, F);
-                    else
-                        k_dense1_fx<kWideFx><<<blocks_for(ngroups, 256 * kWideFx), 256, 0, s->stream>>>(
-                            psi, ngroups, ins, g.cmask, tbit, F);
+                    const bool nr = narrow(s, ngroups, kWideFx);
+                    auto kernel = nr ? (F.apart ? k_dense1_fx<1, true> : k_dense1_fx<1, false>)
+                                     : (F.apart ? k_dense1_fx<kWideFx, true> : k_dense1_fx<kWideFx, false>);
+                    const int threads = nr ? kNarrowThreads : 256;
+                    kernel<<<blocks_for(ngroups, nr ? threads : threads * kWideFx), threads, 0, s->stream>>>(
+                        psi, ngroups, ins, g.cmask, tbit, F);
                     break;
                 }
             }
