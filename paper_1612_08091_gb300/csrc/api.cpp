@@ -323,17 +323,26 @@ int flush(qsim *s) {
         s->last_plan_predicted_ms = ch.predicted_ms;
     }
     if (small_queue_ok(s)) {
-        size_t done = 0;
-        rc = launch_small_queue(s, &done);
-        for (size_t i = 0; i < done; ++i) {
-            if (!q[i].unitary) norm_anchor(s, -1.0);
-            s->stats.passes++;
-            s->stats.amp_updates += std::ldexp(1.0, s->n - (int)q[i].controls.size());
-            s->stats.alg_bytes += gate_bytes(s, q[i]);
-        }
-        if (rc == QSIM_ENOTSUP) {
-            rc = QSIM_OK;
-            for (size_t i = done; i < q.size() && !rc; ++i) {
+        bool fits = true;
+        rc = QSIM_OK;
+        for (size_t i = 0; i < q.size() && !rc;) {
+            const size_t end = fits ? small_run(s, i) : i;
+            if (end - i >= (size_t)kSmallMinRun) {
+                size_t done = i;
+                rc = launch_small_queue(s, i, end, &done);
+                for (; i < done; ++i) {
+                    if (!q[i].unitary) norm_anchor(s, -1.0);
+                    s->stats.passes++;
+                    s->stats.amp_updates += std::ldexp(1.0, s->n - (int)q[i].controls.size());
+                    s->stats.alg_bytes += gate_bytes(s, q[i]);
+                }
+                if (rc == QSIM_ENOTSUP) {
+                    rc = QSIM_OK;
+                    fits = false;
+                }
+                continue;
+            }
+            for (const size_t to = std::max(end, i + 1); i < to && !rc; ++i) {
                 PlanItem one = single_item(q, s->n, (int)i);
                 rc = execute_item(s, one);
             }

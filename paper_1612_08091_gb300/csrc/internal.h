@@ -161,11 +161,15 @@ int cuda_err(qsim *s, cudaError_t e, const char *where);
 // Launchers (gate_kernels.cu) -----------------------------------------------
 int launch_gate_plain(qsim *s, const GateRec &g);
 int launch_block_dense(qsim *s, const int *qubits, int k, const cd *m);
-// The whole queue on a small register in one launch or a few, gate by gate
-// (small_kernel.cu); *done: gates executed.  QSIM_ENOTSUP where the device does
-// not take the launch: the rest are for the caller.
+// Gates of the queue on a small register in one launch or a few, gate by gate
+// (small_kernel.cu): whether this queue may; the end of the gates from `begin`
+// on that run faster there; launch [begin, end).  *done: the end of those
+// executed.  QSIM_ENOTSUP where the device does not take the launch: the rest
+// are for the caller.
+constexpr int kSmallMinRun = 3;  // as many launches cost less than the record's copy
 bool small_queue_ok(const qsim *s);
-int launch_small_queue(qsim *s, size_t *done);
+size_t small_run(const qsim *s, size_t begin);
+int launch_small_queue(qsim *s, size_t begin, size_t end, size_t *done);
 // Emulated classical bijection on a register (perm_kernels.cu).
 // *kind: which kernel ran: 0 tiled, 1 cycle walk through registers, 2 cycle
 // walk through the bulk-copy engine

@@ -90,7 +90,11 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(Amp *__restrict__ psi, 
                 }
                 if constexpr (sizeof(Amp) == 16) {
                     if (G.fx) {
-                        qsim_fx::dense1(*(const qsim_fx::MatFx *)m, v0, v1, x[i0], x[i1]);
+                        const qsim_fx::MatFx &F = *(const qsim_fx::MatFx *)m;
+                        if (F.apart)
+                            qsim_fx::dense1<true>(F, v0, v1, x[i0], x[i1]);
+                        else
+                            qsim_fx::dense1<false>(F, v0, v1, x[i0], x[i1]);
                         continue;
                     }
                 }
@@ -188,15 +192,16 @@ int launch_small(qsim *s, const unsigned char *dev, int ngates, uint32_t rec_byt
     return QSIM_OK;
 }
 
+// Gates [*done, end) of the queue.
 template <typename Amp>
-int small_queue(qsim *s, size_t *done) {
+int small_queue(qsim *s, size_t end, size_t *done) {
     const std::vector<GateRec> &q = s->queue;
     std::vector<unsigned char> mats;
     std::vector<SmallGate> gates;
-    for (size_t i = 0; i < q.size();) {
+    for (size_t i = *done; i < end;) {
         gates.clear();
         mats.clear();
-        for (; i < q.size(); ++i) {
+        for (; i < end; ++i) {
             const GateRec &g = q[i];
             const size_t T = (size_t)1 << g.t;
             const size_t count = g.kind == GK_X ? 0 : g.kind == GK_PHASE ? 1 : g.kind == GK_DIAG1 ? 2 : T * T;
@@ -246,8 +251,7 @@ int small_queue(qsim *s, size_t *done) {
 }  // namespace
 
 bool small_queue_ok(const qsim *s) {
-    // fewer than 3 gates: as many launches cost less than the record's copy
-    if (s->fusion != QSIM_FUSE_NONE || s->profiling || s->c128_df || s->queue.size() < 3 ||
+    if (s->fusion != QSIM_FUSE_NONE || s->profiling || s->c128_df || s->queue.size() < (size_t)kSmallMinRun ||
         s->n > (s->prec == QSIM_C128 ? 13 : 16))
         return false;
     // in a stream capture gates are launched one by one, their matrices in the
@@ -261,7 +265,26 @@ bool small_queue_ok(const qsim *s) {
     return st == cudaStreamCaptureStatusNone;
 }
 
-int launch_small_queue(qsim *s, size_t *done) {
-    *done = 0;
-    return s->prec == QSIM_C128 ? small_queue<double2>(s, done) : small_queue<float2>(s, done);
+// Where a gate's outputs come from amplitudes of other CTAs, 16 SMs read 2^t of
+// them each; a launch of its own has the whole chip.  complex64, us a gate here
+// and launched: 2 targets 4.2 of 13 qubits, 6.9 of 14 (4.4 launched); 3 targets
+// 4.4 of 12 (4.4); 4 targets 6.2 of 8 (4.6); a dense gate on a rank qubit 4.4 of
+// 14, 7.6 of 15 (4.4); X there 3.3 of 15, 5.5 of 16 (4.4).  complex128 is bound
+// by FP64 either way: 2 to 5 targets of 13 qubits 6.2, 11.5, 22, 47 (6.5, 12.7,
+// 42, 156).
+size_t small_run(const qsim *s, size_t begin) {
+    auto pays = [s](const GateRec &g) {
+        if (s->prec == QSIM_C128 || g.kind == GK_PHASE || g.kind == GK_DIAG1) return true;
+        if (g.t == 1 && (s->n <= kSmallOneCta || g.targets[0] < s->n - kSmallRankBits)) return true;
+        if (g.kind == GK_X) return s->n <= 15;
+        return s->n <= (g.t == 1 ? 14 : g.t == 2 ? 13 : g.t == 3 ? 12 : 0);
+    };
+    size_t i = begin;
+    while (i < s->queue.size() && pays(s->queue[i])) ++i;
+    return i;
+}
+
+int launch_small_queue(qsim *s, size_t begin, size_t end, size_t *done) {
+    *done = begin;
+    return s->prec == QSIM_C128 ? small_queue<double2>(s, end, done) : small_queue<float2>(s, end, done);
 }

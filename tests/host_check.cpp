@@ -81,6 +81,28 @@ void check_small_queue_falls_back() {
     sim_destroy(s);
 }
 
+// complex64 gates that the one launch makes slower go on their own, those
+// between them together
+void check_small_queue_runs() {
+    const double swap[32] = {1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1, 0, 0, 0, 0, 0, 1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1, 0};
+    for (int n : {13, 14}) {
+        qsim *s = register_of(n, QSIM_C64);
+        const int pair[2] = {1, 4};
+        for (int k = 0; k < 5; ++k) CHECK(sim_apply(s, kHadamard, &k, 1, nullptr, 0) == QSIM_OK);
+        CHECK(sim_apply(s, swap, pair, 2, nullptr, 0) == QSIM_OK);
+        for (int k = 0; k < 2; ++k) CHECK(sim_apply(s, kHadamard, &k, 1, nullptr, 0) == QSIM_OK);
+        CHECK(sim_apply(s, swap, pair, 2, nullptr, 0) == QSIM_OK);
+        for (int k = 0; k < 5; ++k) CHECK(sim_apply(s, kHadamard, &k, 1, nullptr, 0) == QSIM_OK);
+        CHECK(sim_flush(s) == QSIM_OK);
+        if (n == 13)
+            CHECK(fake::launches().size() == 1 && fake::launched("k_small") == 1);
+        else
+            CHECK(fake::launches().size() == 6 && fake::launched("k_small") == 2 && fake::launched("k_denseK") == 2 &&
+                  fake::launched("k_dense1") == 2);
+        sim_destroy(s);
+    }
+}
+
 // plain gates in a stream capture: launches alone, no copy from host memory
 // that a replay would repeat
 void check_small_queue_under_capture() {
@@ -145,6 +167,7 @@ void check_batch_buffers() {
 int main() {
     check_training_sources();
     check_small_queue_falls_back();
+    check_small_queue_runs();
     check_small_queue_under_capture();
     check_batch_clusters();
     check_queue_growth();
