@@ -184,8 +184,10 @@ int sim_flush(qsim *s);
  * a bijection (QSIM_EINVAL otherwise).  Where all controls are |1>, the
  * amplitude of register value x moves to register value f(x).  Flushes the
  * queue, then runs at once (one pass over the touched groups; fixed points
- * of f are not touched when the register and controls lie above the lowest
- * 64 bytes of amplitudes and f's cycles give at least one task per SM). */
+ * of f are not touched where the amplitudes walk along f's cycles: when the
+ * register and controls lie above the lowest 4 KB of amplitudes, or above the
+ * lowest 64 bytes and the walk is the faster, and f's cycles give at least one
+ * task per SM). */
 int sim_apply_permutation(qsim *s, const uint64_t *perm, const int *qubits, int m, const int *controls, int c);
 
 /* P(qubit = 1) = sum of |psi_i|^2 over indices with bit q set, accumulated

@@ -36,13 +36,16 @@
 // walked from e_{L-1} down to e_0 with the loads of the next eight elements
 // in flight (a load of e_j always precedes the store to e_j).  Fixed points
 // of f are not touched, and the work is (cycle, slice) tasks, longest cycles
-// first.  (A tile of a 12-qubit register above qubit 2 has room for runs of 32
-// bytes only, 128 KB for one CTA per SM: 1.55 ms on 28 qubits against 0.86 ms,
-// 5.0 TB/s, for the walk.)  Above the lowest 16 KB
-// the same walk runs through the bulk-copy engine (k_permute_cycles_bulk).
+// first.  Below 4 KB the pieces cost the walk more than a tile's fixed points and
+// short runs cost it, or less (walk_pays): 12-qubit registers on 28 qubits have
+// room in a tile for runs of 32 bytes only, 128 KB for one CTA per SM, 1.55 ms
+// against 1.02 for swaps and 0.68 for the adder's blocks; 5- to 8-qubit ones from
+// qubit 3 on take 0.9 ms in tiles and 1.2 to 2.0 in pieces of 64 bytes.  Above
+// the lowest 16 KB the same walk runs through the bulk-copy engine (k_permute_cycles_bulk).
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -276,9 +279,100 @@ __global__ void __launch_bounds__(32) k_permute_cycles_bulk(unsigned char *__res
     }
 }
 
+// The cycles of f: elements cycle by cycle, the longest cycle first, fixed
+// points left out.
+struct Cycles {
+    std::vector<uint32_t> elem;
+    std::vector<uint32_t> start;  // of each cycle, and the end
+    size_t count() const { return start.size() - 1; }
+    uint32_t longest() const { return count() ? start[1] : 0; }
+};
+void find_cycles(const uint64_t *perm, int D, Cycles &c) {
+    std::vector<uint32_t> found, begin;
+    std::vector<char> seen(D, 0);
+    for (int v = 0; v < D; ++v) {
+        if (seen[v] || (int)perm[v] == v) continue;
+        begin.push_back((uint32_t)found.size());
+        for (uint32_t x = (uint32_t)v; !seen[x]; x = (uint32_t)perm[x]) {
+            seen[x] = 1;
+            found.push_back(x);
+        }
+    }
+    const size_t n = begin.size();
+    begin.push_back((uint32_t)found.size());
+    // longest first: a counting sort by length
+    std::vector<uint32_t> at(D + 2, 0), order(n);
+    for (size_t j = 0; j < n; ++j) ++at[D - (begin[j + 1] - begin[j]) + 1];
+    for (int l = 0; l <= D; ++l) at[l + 1] += at[l];
+    for (size_t j = 0; j < n; ++j) order[at[D - (begin[j + 1] - begin[j])]++] = (uint32_t)j;
+    c.elem.clear();
+    c.elem.reserve(found.size());
+    c.start.assign(1, 0);
+    for (uint32_t j : order) {
+        c.elem.insert(c.elem.end(), found.begin() + begin[j], found.begin() + begin[j + 1]);
+        c.start.push_back((uint32_t)c.elem.size());
+    }
+}
+
+// Whether the walk beats the tiles where the lowest register or control qubit
+// leaves pieces below 4 KB (from 4 KB on it always does, given the tasks).  Both
+// kernels' rates in TB/s, of the bytes of the whole tiles and of the moved
+// amplitudes, measured on 28 (complex128 27) qubits, by register width: the
+// tiles for pieces of 64, 128 and 256 bytes or more; the walk also by the mean
+// cycle: 2 (two scattered pieces a task), 3 to 40, longer.  E.g. 5 qubits from
+// qubit 3 on, random: tiles 0.90 ms, walk 1.97; 12 qubits from 5 on, swaps: 1.56
+// and 1.02; 12 qubits, one cycle of 4096: 1.54 and 2.34.
+const float kTileRate[2][8][3] = {
+    {{4.7f, 4.8f, 4.8f}, {4.65f, 5.0f, 5.25f}, {4.8f, 5.15f, 5.3f}, {4.9f, 5.2f, 5.4f},
+     {4.9f, 5.2f, 5.3f}, {5.3f, 4.2f, 4.1f}, {4.1f, 2.9f, 2.85f}, {2.95f, 2.8f, 2.75f}},  // complex64
+    {{4.8f, 4.85f, 4.85f}, {4.75f, 4.7f, 4.8f}, {4.5f, 4.8f, 4.85f}, {4.4f, 4.83f, 4.9f},
+     {4.4f, 4.8f, 4.85f}, {4.65f, 4.85f, 4.8f}, {4.85f, 4.4f, 4.3f}, {4.3f, 3.55f, 3.45f}}};
+const float kWalkRate[8][3][3] = {
+    {{5.7f, 6.3f, 6.3f}, {5.9f, 6.3f, 6.3f}, {5.6f, 6.3f, 6.3f}},  // 1, 2 qubits
+    {{4.8f, 5.1f, 5.1f}, {5.3f, 6.2f, 6.2f}, {5.4f, 6.3f, 6.3f}},  // 3
+    {{4.1f, 5.0f, 5.0f}, {5.2f, 6.1f, 6.1f}, {5.4f, 6.3f, 6.3f}},  // 4
+    {{4.0f, 3.9f, 4.4f}, {5.0f, 5.8f, 5.3f}, {5.2f, 6.2f, 5.7f}},  // 5, 6
+    {{4.0f, 3.7f, 4.0f}, {4.8f, 6.0f, 4.5f}, {5.0f, 6.3f, 5.2f}},  // 7, 8
+    {{3.3f, 3.4f, 3.3f}, {4.2f, 5.4f, 4.3f}, {4.4f, 5.9f, 5.1f}},  // 9, 10
+    {{3.2f, 3.4f, 3.2f}, {4.2f, 4.8f, 3.9f}, {4.3f, 5.2f, 4.6f}},  // 11
+    {{3.1f, 3.7f, 2.0f}, {4.1f, 4.6f, 2.2f}, {4.2f, 5.0f, 2.2f}}};  // 12
+int width_row(int m) { return m <= 2 ? 0 : m <= 4 ? m - 2 : m <= 10 ? (m - 5) / 2 + 3 : m - 5; }
+
+struct WalkChoice {
+    bool small;       // the state stays in L2
+    double tiles_us;  // what the tiles take
+    double bytes;     // read and written by whole tiles
+    int row, piece;
+};
+WalkChoice walk_choice(const qsim *s, int m, uint64_t fixed, uint64_t cmask) {
+    WalkChoice w;
+    const size_t b = amp_bytes(s);
+    w.bytes = 2.0 * (double)b * std::ldexp(1.0, s->n - __builtin_popcountll(cmask));
+    w.small = std::ldexp((double)b, s->n) <= (double)(64u << 20);
+    w.row = width_row(m);
+    const uint64_t piece = (uint64_t)b << __builtin_ctzll(fixed);
+    w.piece = piece < 128 ? 0 : piece < 256 ? 1 : 2;
+    w.tiles_us = w.bytes / (1e6 * kTileRate[b == 16][w.row][w.piece]);
+    return w;
+}
+// before the cycles are known: in L2 both take some 20 us and what the host
+// does for each register value decides; else the search takes no more than a
+// tenth of the tiles' time
+bool walk_worth_a_search(const WalkChoice &w, int D) { return w.small ? D <= 64 : w.tiles_us >= D / 16.0; }
+bool walk_pays(const WalkChoice &w, int D, const Cycles &c) {
+    if (w.small) return true;
+    const double mean = (double)c.elem.size() / (double)c.count();
+    const int kind = mean < 3.0 ? 0 : mean <= 40.0 ? 1 : 2;
+    // a step of a cycle waits for its loads: 0.6 us
+    const double walk_us = std::max(w.bytes * (double)c.elem.size() / D / (1e6 * kWalkRate[w.row][w.piece][kind]),
+                                    0.6 * c.longest());
+    return walk_us < w.tiles_us;
+}
+
 // The cycle walk when the register and the controls leave the lowest 64
-// bytes of amplitudes contiguous and there are enough tasks to fill the GPU;
-// returns QSIM_ENOTSUP otherwise (the tiled kernel then runs).
+// bytes of amplitudes contiguous, there are enough tasks to fill the GPU, and
+// from pieces of 4 KB on or where it is the faster; returns QSIM_ENOTSUP
+// otherwise (the tiled kernel then runs).
 template <typename Amp>
 int permute_cycles(qsim *s, const uint64_t *perm, const int *qubits, int m, uint64_t qmask, uint64_t cmask,
                    bool *bulk) {
@@ -291,29 +385,32 @@ int permute_cycles(qsim *s, const uint64_t *perm, const int *qubits, int m, uint
     // a thread's 16 bytes, and pieces of at least 64 bytes, contiguous
     if ((fixed & ((1ull << (2 + amp_shift)) - 1ull)) != 0 || nfree < slice_bits) return QSIM_ENOTSUP;
     const int D = 1 << m;
-    // the cycles of f, longest first
-    std::vector<std::vector<uint32_t>> cycles;
-    std::vector<char> seen(D, 0);
-    size_t total = 0;
-    for (int v = 0; v < D; ++v) {
-        if (seen[v] || (int)perm[v] == v) continue;
-        std::vector<uint32_t> cy;
-        for (uint32_t x = (uint32_t)v; !seen[x]; x = (uint32_t)perm[x]) {
-            seen[x] = 1;
-            cy.push_back(x);
-        }
-        total += cy.size();
-        cycles.push_back(std::move(cy));
-    }
-    if (cycles.empty()) return QSIM_OK;  // f is the identity
+    int first = 0;
+    while (first < D && perm[first] == (uint64_t)first) ++first;
+    if (first == D) return QSIM_OK;  // f is the identity
+    const bool pieces = (fixed & ((1ull << slice_bits) - 1ull)) != 0;  // below 4 KB
+    const WalkChoice choice = walk_choice(s, m, fixed, cmask);
+    if (pieces && !walk_worth_a_search(choice, D)) return QSIM_ENOTSUP;
+    Cycles cycles;
+    find_cycles(perm, D, cycles);
+    const size_t ncyc = cycles.count(), total = cycles.elem.size();
     const uint64_t nslices = 1ull << (nfree - slice_bits);
-    if ((uint64_t)cycles.size() * nslices < (uint64_t)s->sms) return QSIM_ENOTSUP;
+    if ((uint64_t)ncyc * nslices < (uint64_t)s->sms) return QSIM_ENOTSUP;
+    if (pieces && !walk_pays(choice, D, cycles)) return QSIM_ENOTSUP;
     // the bulk-copy walk: 16 KB slices, at least two tasks per SM
     const bool use_bulk = (fixed & ((1ull << bulk_bits) - 1ull)) == 0 && nfree >= bulk_bits &&
-                          (uint64_t)cycles.size() * (1ull << (nfree - bulk_bits)) >= 2ull * (uint64_t)s->sms;
-    std::stable_sort(cycles.begin(), cycles.end(),
-                     [](const std::vector<uint32_t> &a, const std::vector<uint32_t> &b) { return a.size() > b.size(); });
-    const size_t ncyc = cycles.size();
+                          (uint64_t)ncyc * (1ull << (nfree - bulk_bits)) >= 2ull * (uint64_t)s->sms;
+    // register-value offsets, in amplitudes: bits 0..5 and 6..11 of the value
+    uint64_t olo[64], ohi[64];
+    for (int v = 0; v < 64; ++v) {
+        olo[v] = ohi[v] = 0;
+        for (int b = 0; b < 6; ++b)
+            if ((v >> b) & 1) {
+                if (b < m) olo[v] |= 1ull << qubits[b];
+                if (b + 6 < m) ohi[v] |= 1ull << qubits[b + 6];
+            }
+    }
+    auto offset = [&](uint32_t v) { return olo[v & 63u] | ohi[v >> 6]; };
     InsertSpec ins{};
     ins.m = 0;
     for (int b = 0; b < 64; ++b)
@@ -322,23 +419,14 @@ int permute_cycles(qsim *s, const uint64_t *perm, const int *qubits, int m, uint
         // record: offsets in 16 KB slice units (uint32), then cycle starts
         const size_t bslice_amps = (size_t)kBulkSlice / sizeof(Amp);
         std::vector<uint32_t> rb(total + ncyc + 1);
-        size_t k = 0;
-        for (size_t j = 0; j < ncyc; ++j) {
-            rb[total + j] = (uint32_t)k;
-            for (uint32_t v : cycles[j]) {
-                uint64_t a = 0;
-                for (int b = 0; b < m; ++b)
-                    if ((v >> b) & 1u) a |= 1ull << qubits[b];
-                rb[k++] = (uint32_t)(a / bslice_amps);
-            }
-        }
-        rb[total + ncyc] = (uint32_t)k;
+        for (size_t k = 0; k < total; ++k) rb[k] = (uint32_t)(offset(cycles.elem[k]) / bslice_amps);
+        std::copy(cycles.start.begin(), cycles.start.end(), rb.begin() + total);
         unsigned char *dev = nullptr;
         int rc = stage_operand(s, rb.data(), rb.size() * sizeof(uint32_t), &dev);
         if (rc) return rc;
         const uint64_t bslices = 1ull << (nfree - bulk_bits);
         const uint64_t ntasks = (uint64_t)ncyc * bslices;
-        const size_t smem = (size_t)(kBulkStages + 1) * kBulkSlice + sizeof(uint32_t) * cycles[0].size();
+        const size_t smem = (size_t)(kBulkStages + 1) * kBulkSlice + sizeof(uint32_t) * cycles.longest();
         static bool attr[64] = {false};
         if (s->device >= 0 && s->device < 64 && !attr[s->device]) {
             cudaError_t e = cudaFuncSetAttribute(k_permute_cycles_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -358,24 +446,15 @@ int permute_cycles(qsim *s, const uint64_t *perm, const int *qubits, int m, uint
     std::vector<unsigned char> rec(sizeof(uint64_t) * total + sizeof(uint32_t) * (ncyc + 1));
     uint64_t *coff = (uint64_t *)rec.data();
     uint32_t *cstart = (uint32_t *)(rec.data() + sizeof(uint64_t) * total);
-    size_t k = 0;
-    for (size_t j = 0; j < ncyc; ++j) {
-        cstart[j] = (uint32_t)k;
-        for (uint32_t v : cycles[j]) {
-            uint64_t a = 0;
-            for (int b = 0; b < m; ++b)
-                if ((v >> b) & 1u) a |= 1ull << qubits[b];
-            coff[k++] = a >> amp_shift;
-        }
-    }
-    cstart[ncyc] = (uint32_t)k;
+    for (size_t k = 0; k < total; ++k) coff[k] = offset(cycles.elem[k]) >> amp_shift;
+    std::copy(cycles.start.begin(), cycles.start.end(), cstart);
     unsigned char *dev = nullptr;
     int rc = stage_operand(s, rec.data(), rec.size(), &dev);
     if (rc) return rc;
     const uint64_t ntasks = (uint64_t)ncyc * nslices;
     // 64 registers a thread: four CTAs of 256 threads resident per SM
     const uint64_t grid = ntasks < (uint64_t)s->sms * 4 ? ntasks : (uint64_t)s->sms * 4;
-    const size_t smem = sizeof(uint64_t) * cycles[0].size();  // the longest cycle (<= 2^12 entries)
+    const size_t smem = sizeof(uint64_t) * cycles.longest();  // the longest cycle (<= 2^12 entries)
     k_permute_cycles<<<(unsigned)grid, kCycThreads, smem, s->stream>>>(
         (float4 *)s->state, ins, cmask >> amp_shift, (const uint64_t *)dev,
         (const uint32_t *)(dev + sizeof(uint64_t) * total), (uint32_t)ncyc, nslices, amp_shift);

@@ -118,6 +118,50 @@ void check_small_queue_under_capture() {
     }
 }
 
+// which kernel moves a register's values: tiles, or the walk along the cycles,
+// whichever was measured to be the faster on the register's qubits and cycles
+void check_permutation_choice() {
+    enum Kind { SWAPS, ADD, LONG, CADD, EIGHTS, IDENTITY };
+    auto kernel = [](int n, int precision, int m, int q0, Kind kind) {
+        qsim *s = register_of(n, precision);
+        std::vector<uint64_t> f(1u << m);
+        std::vector<int> qubits(m);
+        const uint64_t D = f.size(), h = D / 2;
+        for (int j = 0; j < m; ++j) qubits[j] = q0 + j;
+        for (uint64_t v = 0; v < D; ++v) {
+            f[v] = v;
+            if (kind == SWAPS) f[v] = v ^ (D - 1);
+            if (kind == ADD) f[v] = (v + 1) % D;
+            if (kind == LONG) f[v] = (5 * v + 3) % D;  // one cycle of D values, far apart
+            if (kind == EIGHTS) f[v] = (v + D / 8) % D;  // cycles of 8
+            if (kind == CADD && v >= h) f[v] = h + (v - h + 3) % h;
+        }
+        CHECK(sim_apply_permutation(s, f.data(), qubits.data(), m, nullptr, 0) == QSIM_OK);
+        const int walks = fake::launched("k_permute_cycles"), tiles = fake::launched("k_permute") - walks;
+        sim_destroy(s);
+        return walks ? 'w' : tiles ? 't' : '-';
+    };
+    for (int precision : {QSIM_C64, QSIM_C128}) {
+        const int n = precision == QSIM_C64 ? 28 : 27, low = precision == QSIM_C64 ? 3 : 2;  // pieces of 64 bytes
+        for (int m : {5, 6, 7, 8, 10}) {
+            CHECK(kernel(n, precision, m, low, SWAPS) == 't');  // 1.2 ms and more against 0.9
+            CHECK(kernel(n, precision, m, low, LONG) == 't');
+        }
+        CHECK(kernel(n, precision, 12, low, LONG) == 't');      // 2.0 to 2.9 ms against 1.0 to 1.5
+        CHECK(kernel(n, precision, 12, low + 4, LONG) == 't');  // 2.1 to 2.5 against 1.2 to 1.6
+        CHECK(kernel(n, precision, 12, low + 3, SWAPS) == 'w'); // 1.0 against 1.6 (1.2)
+        CHECK(kernel(n, precision, 12, low, EIGHTS) == (precision == QSIM_C64 ? 'w' : 't'));  // 1.1 against 1.44 (1.0)
+        CHECK(kernel(n, precision, 3, low, ADD) == 'w');        // 0.7 against 0.93
+        CHECK(kernel(n, precision, 2, low + 1, SWAPS) == 'w');
+        CHECK(kernel(n, precision, 8, low + 1, CADD) == 'w');   // half the values: 0.5 against 0.85
+        CHECK(kernel(n, precision, 6, low + 7, LONG) == 'w');   // pieces of 8 KB
+        CHECK(kernel(n, precision, 8, low, IDENTITY) == '-');
+        CHECK(kernel(n - 6, precision, 12, low + 1, SWAPS) == 't');  // in L2: what the host does per value
+        CHECK(kernel(n - 6, precision, 4, low + 1, SWAPS) == 'w');
+        CHECK(kernel(n, precision, 4, 0, ADD) == 't');
+    }
+}
+
 // every circuit of a batch is some CTA's: circuits are set aside for clusters
 // only where clusters are launched
 void check_batch_clusters() {
@@ -169,6 +213,7 @@ int main() {
     check_small_queue_falls_back();
     check_small_queue_runs();
     check_small_queue_under_capture();
+    check_permutation_choice();
     check_batch_clusters();
     check_queue_growth();
     check_batch_buffers();
