@@ -499,9 +499,11 @@ def run_ours(args):
             if roof is not None:
                 roof["note"] = ("double-float arithmetic: the plain complex128 >= 80% target is met in this "
                                 "arithmetic only" if df else
-                                "fp64 arithmetic: the dense gate is bound by the FP64 pipe (~2.1 TB/s), not HBM")
+                                "dense one-qubit gates in shared-exponent integers: bound by integer multiply-adds, "
+                                "not HBM")
             return {"value": rate, "unit": UNIT, "precision": "c128", "hbm_roofline": roof,
-                    "arithmetic": "double-float (fp32 pairs, ~2^-45 relative)" if df else "fp64",
+                    "arithmetic": "double-float (fp32 pairs, or integers to the same accuracy; ~2^-45 relative)"
+                                  if df else "fp64; dense one-qubit gates in integers of at least its accuracy",
                     "fusion": fusion if fusion == "none" else "%s, kmax %d" % (fusion, kmax),
                     "sample": "first %d gates of the same %d-qubit circuit, %s (the whole circuit: "
                               "bench.py --workload plain)"
@@ -782,7 +784,8 @@ def run_planner(args):
            "learned": dict(arm(ml, upd), gain_over_greedy_k5=g5["s"] / ml["s"], gain_over_greedy_k6=g6["s"] / ml["s"]),
            "greedy_k5": arm(g5, upd),
            "greedy_k6": arm(g6, upd),
-           "plain_c128": {"ms": 1e3 * t_plain, "value": upd / t_plain, "runs": 1, "arithmetic": "fp64",
+           "plain_c128": {"ms": 1e3 * t_plain, "value": upd / t_plain, "runs": 1,
+                          "arithmetic": "fp64; dense one-qubit gates in integers of at least its accuracy",
                           "what": "whole circuit, one launch per gate, complex128",
                           "learned_speedup": t_plain / ml["s"]},
            "check": {"max_p1_difference_learned_vs_plain_c128": float(np.max(np.abs(ml["p1"] - np.asarray(p1_plain)))),

@@ -4,8 +4,8 @@
 // phases, multi-controlled Z) only multiply each amplitude by a phase that
 // depends on the bits of its index on the gate's qubits, and they commute
 // with one another.  A run of them over a qubit set S (|S| <= 12) is one
-// table d of 2^|S| factors (built on the host in FP64: the product of the
-// gates' diagonal entries for every assignment of S), and the pass is
+// table d of 2^|S| factors (the product of the gates' diagonal entries for
+// every assignment of S, in FP64), and the pass is
 //     psi_i <- d[bits of i on S] * psi_i.
 // The phase ladders of the QFT (ProjectQ paper, Sec. 3: the constant adder
 // is QFT, phase shifts, inverse QFT) and the controlled z-rotation chain of

@@ -146,7 +146,7 @@ __device__ __forceinline__ FxF to_fxf(double x, int E) {
     FxF r;
     r.hi = (int)((v + (1 << 24)) >> 25);
     r.fhi = (float)r.hi;
-    r.flo = (float)((int)v - (int)((uint32_t)r.hi << 25));
+    r.flo = (float)(int)((uint32_t)v - ((uint32_t)r.hi << 25));
     return r;
 }
 // a 2^50 + c 2^25 as a double: units of 2^(E - 1077 - S); eadd = (E - 1027 - S)

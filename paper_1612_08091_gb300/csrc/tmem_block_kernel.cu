@@ -24,7 +24,7 @@
 // BF16x3.  X = X1 + X2 and R = R1 + R2 (+ R3) are split into bfloat16 parts;
 // the products X1 R1 + X2 R1 + X1 R2 (or five with X2 R2 + X1 R3) accumulate
 // in FP32 in tensor memory.  The state split loses about 2^-17 relatively
-// per element and pass; the gate split is computed on the host in FP64.
+// per element and pass; the gate split is computed in FP64 (k_build_operand).
 //
 // Where the operands live.  R's bf16 parts are operand B in shared memory:
 // K-major, 128-byte swizzle, in 64-element K halves of N x 128 bytes.  The

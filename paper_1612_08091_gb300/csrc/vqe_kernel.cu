@@ -104,11 +104,9 @@ __device__ __forceinline__ unsigned ladder_src(unsigned y, unsigned mask) { retu
 // at a time in registers: each thread loads the 16 amplitudes of a group,
 // applies the four rotations there and stores them back, so a layer of k
 // one-qubit rotations costs ceil(k/4) passes over shared memory instead of k.
-// Rotation j pairs the elements i and i ^ mask[j] (single bits here; the
-// pair pass of the global-memory path, whose buffers are in source order,
-// has its own compile-time version, pair_group).  The masks' bits must
-// differ; a group is a base with zeros at its bits XOR any subset of its
-// masks.  A group of fewer than four rotations is padded with identity
+// Rotation j pairs the elements i and i ^ mask[j] (single bits).  The masks'
+// bits must differ; a group is a base with zeros at its bits XOR any subset of
+// its masks.  A group of fewer than four rotations is padded with identity
 // rotations on other bits.
 __device__ __forceinline__ void cswap(int &a, int &b) {
     const int lo = a < b ? a : b, hi = a < b ? b : a;
@@ -720,7 +718,7 @@ __global__ void __launch_bounds__(kWinThreads, kWinCtas) k_vqe_window(const VqeA
 // host side: the batch object, its graph and the tile autotuner
 // ---------------------------------------------------------------------------
 struct qsim_batch {
-    int count = 0, nmax = 0, nmin = 0;
+    int count = 0, nmax = 0;
     long long nangles = 0;
     double h = 0.7;
     std::vector<int> nq, nl, order;
@@ -772,8 +770,7 @@ int count_large(const qsim_batch *b, int m) {
     return k;
 }
 
-bool config_valid(const qsim_batch *b, int threads, int m) {
-    (void)b;
+bool config_valid(int threads, int m) {
     return (1 << m) <= reg_amps(threads) * threads;  // in-place permutation through registers
 }
 
@@ -930,12 +927,10 @@ int sim_batch_create(int count, const int *nqubits, const int *layers, double h,
     b->aoff.resize(count);
     long long off = 0;
     b->nmax = 0;
-    b->nmin = 64;
     for (int i = 0; i < count; ++i) {
         b->aoff[i] = off;
         off += 2LL * nqubits[i] * layers[i];
         b->nmax = std::max(b->nmax, nqubits[i]);
-        b->nmin = std::min(b->nmin, nqubits[i]);
     }
     b->nangles = off;
     // largest first: by qubits, then layers (so the circuits above any
@@ -1055,7 +1050,7 @@ int sim_batch_autotune(qsim_batch *b, const double *angles, int reps, int *threa
     int bt = b->threads, bm = b->m;
     for (const auto &cand : kCandidates) {
         const int threads = cand[0], m = cand[1];
-        if (!config_valid(b, threads, m)) continue;
+        if (!config_valid(threads, m)) continue;
         int grid = 0;
         if (occupancy(b, threads, m, &grid)) continue;
         std::vector<float> t;
@@ -1096,7 +1091,7 @@ int sim_batch_autotune(qsim_batch *b, const double *angles, int reps, int *threa
 int sim_batch_set_config(qsim_batch *b, int threads, int m) {
     if (!b) return QSIM_EINVAL;
     if (threads != 256 && threads != 512 && threads != 1024) return berr(b, QSIM_EINVAL, "threads must be 256/512/1024");
-    if (m < 12 || m > 14 || !config_valid(b, threads, m)) return berr(b, QSIM_EINVAL, "invalid tile configuration");
+    if (m < 12 || m > 14 || !config_valid(threads, m)) return berr(b, QSIM_EINVAL, "invalid tile configuration");
     b->threads = threads;
     b->m = m;
     if (b->graph) {
