@@ -254,32 +254,88 @@ __global__ void __launch_bounds__(256) k_phase_df(double2 *__restrict__ psi, uin
         if (g0 + u * blockDim.x < ngroups) psi[i[u]] = qsim_df::to_double(qsim_df::cmul(M.m[3], qsim_df::split(v[u])));
 }
 
-// complex128 5-qubit dense gate or fused block in double-float arithmetic, and
-// narrower ones that the integer form does not fit: the group's 2^k amplitudes
-// split into FP32 pairs, each output the sum of 2^k exact-product complex MACs
+// complex128 5-qubit dense gate or fused block in double-float arithmetic: the
+// group's 2^k amplitudes split into FP32 pairs, each output the sum of 2^k exact-product complex MACs
 // with two-sum additions, rounded once to double.  About 40 FP32 operations per
 // MAC instead of 4 FP64 FMAs (FP64 runs at 1/58 of the FP32 rate here).
+template <int K> struct MatKDF { qsim_df::C2 m[(1 << K) * (1 << K)]; uint64_t off[1 << K]; };
+
 template <int K>
-__device__ __forceinline__ void dense_pairs(double2 *p, const qsim_df::C2 *m, const uint64_t *off) {
+__global__ void __launch_bounds__(128) k_denseK_df(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
+                                                   uint64_t cmask, const MatKDF<K> M) {
     constexpr int D = 1 << K;
+    const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (g >= ngroups) return;
+    const uint64_t base = insert_zeros(g, ins) | cmask;
     qsim_df::C2 v[D];
 #pragma unroll
-    for (int r = 0; r < D; ++r) v[r] = qsim_df::split(p[off[r]]);
+    for (int r = 0; r < D; ++r) v[r] = qsim_df::split(psi[base + M.off[r]]);
 #pragma unroll 1
     for (int r = 0; r < D; ++r) {
         // four partial sums: each addition rounds the low parts
         qsim_df::C2 acc[4];
 #pragma unroll
         for (int c = 0; c < D; ++c) {
-            const qsim_df::C2 z = qsim_df::cmul(m[r * D + c], v[c]);
+            const qsim_df::C2 z = qsim_df::cmul(M.m[r * D + c], v[c]);
             acc[c & 3] = c < 4 ? z : qsim_df::cadd(acc[c & 3], z);
         }
-        p[off[r]] =
+        psi[base + M.off[r]] =
             qsim_df::to_double(qsim_df::cadd(qsim_df::cadd(acc[0], acc[1]), qsim_df::cadd(acc[2], acc[3])));
     }
 }
 
-// the same in FP64 arithmetic
+// complex128 gate or fused block on 2 to 4 qubits whose matrix has one element
+// in each row and column (CNOTs, SWAPs, phases), double-float option: every
+// amplitude goes to its place, times its element in FP64 unless that is 1.  26
+// qubits, a block of CNOTs: bound by HBM, where pairs took 1.59 ms and the integer
+// form, which rounds to the group's largest amplitude, 0.80.
+template <int K> struct MatKMono {
+    double2 w[1 << K];
+    uint64_t from[1 << K], to[1 << K];
+    uint32_t ones;
+};
+
+template <int K>
+__global__ void __launch_bounds__(128) k_monomial(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
+                                                  uint64_t cmask, const MatKMono<K> M) {
+    constexpr int D = 1 << K;
+    const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (g >= ngroups) return;
+    double2 *const p = psi + (insert_zeros(g, ins) | cmask);
+    double2 v[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) v[c] = p[M.from[c]];
+#pragma unroll
+    for (int c = 0; c < D; ++c) p[M.to[c]] = (M.ones >> c) & 1u ? v[c] : cmul(M.w[c], v[c]);
+}
+
+// complex128 k-qubit dense gate or fused block where the handle allows
+// double-float accuracy, in shared-exponent integers and FP32 (fx128.cuh): a
+// thread takes a group's 2^k amplitudes; a complex product is 4 integer
+// multiply-adds and 8 FP32 ones, on two halves of the FMA pipe, where pairs of
+// FP32 took 48 operations; one FP64 conversion per result.
+// The error of this form is relative to the group's largest amplitude, that of
+// pairs (2^-45) to a result's own products.  So each row's sum of |m| |v| is
+// looked at (first a lower bound from the least elements of a quarter's rows for
+// all of them, then, in a warp where that is too small, each): from kFxRow of U
+// (fx128.cuh) on the error is below 2^-44.6 of it; where it is smaller
+// (amplitudes of very different sizes under rows that do not mix them), the
+// result is formed again in pairs, from the inputs kept in shared memory.
+template <int K> struct MatKFx {
+    // each element's re and im (hi, hi rounded, lo) for 16- and 8-byte loads
+    int4 a[(1 << K) * (1 << K)];    // re hi, im hi, and both as floats
+    float2 b[(1 << K) * (1 << K)];  // re lo, im lo
+    qsim_df::C2 m[(1 << K) * (1 << K)];
+    float w[(1 << K) * (1 << K)];   // |element|, the largest row sum being 1/2 to 1
+    float low[4][1 << K];           // the least of each quarter of a column
+    uint64_t off[1 << K];
+    int shift;                    // -1027 - S
+};
+// times the square root of the number of amplitudes that are not 0, as the error
+// (fx128.cuh): 2^-8 to 2^-6
+constexpr float kFxRow = 0x1p-8f;
+
+// All rows in FP64, from the matrix in pairs.
 template <int K>
 __device__ __forceinline__ void dense_fp64(double2 *p, const qsim_df::C2 *m, const uint64_t *off) {
     constexpr int D = 1 << K;
@@ -298,46 +354,36 @@ __device__ __forceinline__ void dense_fp64(double2 *p, const qsim_df::C2 *m, con
     }
 }
 
-template <int K> struct MatKDF { qsim_df::C2 m[(1 << K) * (1 << K)]; uint64_t off[1 << K]; };
-
+// One row times the inputs of this thread (E: their exponent; nz: which are not
+// 0), in pairs, or FP64 beyond their range.
 template <int K>
-__global__ void __launch_bounds__(128) k_denseK_df(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
-                                                   uint64_t cmask, const MatKDF<K> M) {
-    const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (g >= ngroups) return;
-    dense_pairs<K>(psi + (insert_zeros(g, ins) | cmask), M.m, M.off);
+__device__ __forceinline__ double2 row_apart(const qsim_df::C2 *m, const double2 (*in)[128], uint32_t nz, int E) {
+    constexpr int D = 1 << K;
+    const int t = threadIdx.x;
+    if (E > 1023 - 60 && E < 1023 + 60) {
+        qsim_df::C2 acc[4] = {};
+#pragma unroll 1
+        for (int c = 0; c < D; c += 4) {
+            if (!((nz >> c) & 15u)) continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                acc[j] = qsim_df::cadd(acc[j], qsim_df::cmul(m[c + j], qsim_df::split(in[c + j][t])));
+        }
+        return qsim_df::to_double(qsim_df::cadd(qsim_df::cadd(acc[0], acc[1]), qsim_df::cadd(acc[2], acc[3])));
+    }
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int c = 0; c < D; ++c)
+        acc = cfma(make_double2((double)m[c].re.hi + m[c].re.lo, (double)m[c].im.hi + m[c].im.lo), in[c][t], acc);
+    return acc;
 }
-
-// complex128 k-qubit dense gate or fused block where the handle allows
-// double-float accuracy, in shared-exponent integers and FP32 (fx128.cuh): a
-// thread takes a group's 2^k amplitudes; a complex product is 4 integer
-// multiply-adds and 8 FP32 ones, on two halves of the FMA pipe, where pairs of
-// FP32 took 48 operations; one FP64 conversion per result.
-// The error of this form is relative to the group's largest amplitude, that of
-// pairs (2^-45) to a result's own products.  So each row's sum of |m| |v| is
-// looked at first (a lower bound from the least elements of a quarter's rows;
-// where that is too small, the sum): where all are at least kFxRow of U
-// (fx128.cuh) the error is below 2^-45 of them; where one is not (amplitudes of
-// very different sizes under rows that do not mix them), the warp computes in
-// pairs, as the 5-qubit kernel.
-template <int K> struct MatKFx {
-    // each element's re and im (hi, hi rounded, lo) for 16- and 8-byte loads
-    int4 a[(1 << K) * (1 << K)];    // re hi, im hi, and both as floats
-    float2 b[(1 << K) * (1 << K)];  // re lo, im lo
-    qsim_df::C2 m[(1 << K) * (1 << K)];
-    float w[(1 << K) * (1 << K)];   // |element|, the largest row sum being 1/2 to 1
-    float low[4][1 << K];           // the least of each quarter of a column
-    uint64_t off[1 << K];
-    int shift;                    // -1027 - S
-    int pairs;                    // rows that hardly mix: in pairs throughout
-};
-constexpr float kFxRow = 0x1p-6f;
 
 template <int K>
 __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, uint64_t ngroups, const InsertSpec ins,
                                                    uint64_t cmask, const MatKFx<K> M) {
     using namespace qsim_fx;
     constexpr int D = 1 << K;
+    __shared__ double2 s_in[D][128];
     const uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (g >= ngroups) return;
     double2 *const p = psi + (insert_zeros(g, ins) | cmask);
@@ -363,11 +409,16 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
         xr[r] = to_fxf(v[r].x, E);
         xi[r] = to_fxf(v[r].y, E);
     }
+    uint32_t apart = 0, nz = 0;  // rows to be formed apart, amplitudes that are not 0
+    bool look;
     {
-        float size[D], low = M.pairs ? 0.f : 0x1p30f;
+        float size[D], low = 0x1p30f, count = 0.f;
 #pragma unroll
-        for (int c = 0; c < D; ++c) size[c] = fmaxf(fabsf(xr[c].fhi), fabsf(xi[c].fhi));
-        // at first a lower bound for the rows of a quarter
+        for (int c = 0; c < D; ++c) {
+            size[c] = fmaxf(fabsf(xr[c].fhi), fabsf(xi[c].fhi));
+            count += size[c] > 0.f ? 1.f : 0.f;
+        }
+        const float line = kFxRow * 0x1p30f * sqrtf(count);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             float t = 0.f;
@@ -375,25 +426,22 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
             for (int c = 0; c < D; ++c) t = fmaf(M.low[q][c], size[c], t);
             low = fminf(low, t);
         }
-        bool pairs = __any_sync(__activemask(), low < kFxRow * 0x1p30f);
-        if (pairs && !M.pairs) {
-            low = 0x1p30f;
+        look = __any_sync(__activemask(), low < line);
+        if (look) {
+            // (read again, one by one: v kept, or all at once, takes 40 registers more)
+#pragma unroll 1
+            for (int r = 0; r < D; ++r) {
+                const double2 z = p[M.off[r]];
+                s_in[r][threadIdx.x] = z;
+                nz |= (uint32_t)(z.x != 0.0 || z.y != 0.0) << r;
+            }
 #pragma unroll 2
             for (int r = 0; r < D; ++r) {
                 float t = 0.f;
 #pragma unroll
                 for (int c = 0; c < D; ++c) t = fmaf(M.w[r * D + c], size[c], t);
-                low = fminf(low, t);
+                apart |= (uint32_t)(t < line) << r;
             }
-            pairs = __any_sync(__activemask(), low < kFxRow * 0x1p30f);
-        }
-        if (pairs) {
-            // pairs hold 2^-126 to 2^127
-            if (E > 1023 - 60 && E < 1023 + 60)
-                dense_pairs<K>(p, M.m, M.off);
-            else
-                dense_fp64<K>(p, M.m, M.off);
-            return;
         }
     }
     const int eadd = (E + M.shift) << 20;
@@ -422,6 +470,9 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
         }
         p[M.off[r]] = make_double2(to_double_f(rr - ii, cr + dr, eadd), to_double_f(ri, ci + di, eadd));
     }
+#pragma unroll 1
+    for (int r = 0; r < D && look; ++r)
+        if ((apart >> r) & 1u) p[M.off[r]] = row_apart<K>(M.m + r * D, s_in, nz, E);
 }
 
 qsim_df::F2 host_split(double x) {
@@ -548,17 +599,33 @@ int dense_k_fx(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
         M.off[r] = o;
     }
     double rows = 0.0;  // largest sum of |re| + |im| of a row
-    bool mixes = true;
+    int in_row[D] = {0}, in_col[D] = {0}, row_of[D] = {0};
     for (int r = 0; r < D; ++r) {
-        double t = 0.0, sum = 0.0, top = 0.0;
+        double t = 0.0;
         for (int c = 0; c < D; ++c) {
             const cd z = m[r * D + c];
             t += std::abs(z.real()) + std::abs(z.imag());
-            sum += std::abs(z);
-            top = std::max(top, std::abs(z));
+            if (z != 0.0) ++in_row[r], ++in_col[c], row_of[c] = r;
         }
         rows = std::max(rows, t);
-        mixes = mixes && sum >= 1.125 * top;
+    }
+    bool mono = true;
+    for (int r = 0; r < D; ++r) mono = mono && in_row[r] == 1 && in_col[r] == 1;
+    if (mono) {
+        MatKMono<K> P;
+        P.ones = 0;
+        for (int c = 0; c < D; ++c) {
+            const cd z = m[row_of[c] * D + c];
+            P.w[c] = amp<double2>(z);
+            P.from[c] = M.off[c];
+            P.to[c] = M.off[row_of[c]];
+            if (z == 1.0) P.ones |= 1u << c;
+        }
+        const InsertSpec ins = make_spec(tmask | cmask);
+        const uint64_t ngroups = 1ull << (s->n - ins.m);
+        k_monomial<K><<<blocks_for(ngroups, 128), 128, 0, s->stream>>>((double2 *)s->state, ngroups, ins, cmask, P);
+        s->stats.launches++;
+        return cuda_err(s, cudaGetLastError(), "monomial gate launch");
     }
     // a zero or an extreme matrix: FP64
     if (!(rows > qsim_fx::kFxMatrixLow) || !(rows < qsim_fx::kFxMatrixTop))
@@ -587,9 +654,6 @@ int dense_k_fx(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
             for (int r = q * (D / 4); r < (q + 1) * (D / 4); ++r) M.low[q][c] = std::min(M.low[q][c], M.w[r * D + c]);
         }
     M.shift = -1027 - S;
-    // a row of one amplitude (permutations, controlled gates): the sums that the
-    // kernel looks at are small in most warps, and pairs multiply by 1 exactly
-    M.pairs = !mixes;
     const InsertSpec ins = make_spec(tmask | cmask);
     const uint64_t ngroups = 1ull << (s->n - ins.m);
     k_denseK_fx<K><<<blocks_for(ngroups, 128), 128, 0, s->stream>>>((double2 *)s->state, ngroups, ins, cmask, M);

@@ -25,6 +25,8 @@ def matrix(kind, k, rng):
         return unitary(d, rng)
     if kind == "permutation":
         return np.eye(d)[rng.permutation(d)].astype(complex)
+    if kind == "phases":
+        return np.eye(d)[rng.permutation(d)] * np.where(rng.random(d) < 0.5, 1.0, np.exp(1j * rng.uniform(0, 6, d)))
     if kind == "controlled":  # the last qubit's gate where all others are 1
         m = np.eye(d, dtype=complex)
         m[d // 2 - 1::d // 2, d // 2 - 1::d // 2] = unitary(2, rng)
@@ -35,7 +37,7 @@ def matrix(kind, k, rng):
 
 
 @pytest.mark.parametrize("k", [2, 3, 4])
-@pytest.mark.parametrize("kind", ["mixing", "permutation", "controlled", "product", "1e-3", "0.05", "0.3"])
+@pytest.mark.parametrize("kind", ["mixing", "permutation", "phases", "controlled", "product", "1e-3", "0.05", "0.3"])
 @pytest.mark.parametrize("spread,zeros,scale", [(0, 0.0, 0), (8, 0.0, 0), (40, 0.0, 0), (0, 0.8, 0), (12, 0.5, 0),
                                                 (10, 0.2, 900), (10, 0.2, 200), (10, 0.2, -850), (10, 0.2, -200)])
 def test_rows(k, kind, spread, zeros, scale):
