@@ -568,11 +568,13 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_x(const Amp *__restrict_
 // two such sums, their product with the coefficient and the terms of a tile are
 // added with their rounding errors kept (x_term), tiles in FP64.  So FP32
 // rounds what it rounds in k_expect_x, sums of eight pairs, and the
-// coefficients stay doubles.  Registers where a thread of k_expect_x has fewer
-// than eight pairs, and each sum then fewer than eight, take Fine: every pair
-// goes to FP64 on its own.
-// 29 qubits, 29 terms: 2.13 ms (0.71 ms a pass, 6.05 TB/s, 90 % of HBM)
-// against 38.2 ms with a read per term.  Fewer than two terms, complex128
+// coefficients are pairs of FP32.  Registers where a thread of k_expect_x has
+// fewer than eight pairs, and each sum then fewer than eight, take Fine: every
+// pair is added on its own, its rounding error kept.
+// 29 qubits, 29 terms: 2.46 ms (0.82 ms a pass, 5.2 TB/s) against 38.2 ms with a
+// read per term; 2.13 ms with one FP32 sum for all terms of a tile, whose error
+// was 4 times as large on states whose pairs have one sign.  Fine, 18 qubits: 6
+// us of 106 (44 us with FP64 additions).  Fewer than two terms, complex128
 // and registers below one tile keep k_expect_x.
 constexpr int kXBits = 13;
 constexpr int kXThreads = 256;
@@ -581,8 +583,7 @@ constexpr int kXMinRun = 3;  // runs of at least 2^3 amplitudes
 struct XTileArgs {
     uint64_t ntiles;       // 2^(n - 13)
     InsertSpec vspec;      // V, ascending
-    double c[kXBits];      // 2 c_q of the qubit at tile bit j, times 1 / scale (0: no term)
-    float ch[kXBits], cl[kXBits];  // the same as a pair of FP32
+    float ch[kXBits], cl[kXBits];  // 2 c_q / scale of the qubit at tile bit j, as a pair of FP32 (0: no term)
     double scale;          // a power of two: the largest c_q is about 1
     uint32_t mask;         // tile bits with a term
 };
@@ -608,24 +609,24 @@ template <int N>
 __device__ __forceinline__ float x_eight(const float2 (&v)[N], int r, int k0) {
     return __fadd_rn(x_four(v, r, k0), x_four(v, r, k0 + 4));
 }
-// all pairs in FP64
-template <int N>
-__device__ __forceinline__ double x_pairs_fine(const float2 (&v)[N], int r) {
-    double s = 0.0;
-#pragma unroll
-    for (int k = 0; k < N / 2; ++k) s += (double)x_pair(v, r, k, 0.f);
-    return s;
+// (s, e) += w, e collecting the rounding errors
+__device__ __forceinline__ void two_sum(float &s, float &e, float w) {
+    const float t = __fadd_rn(s, w), b = __fsub_rn(t, s);
+    e += __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(w, b));
+    s = t;
 }
-// (hi, lo) += (ch + cl) (a + b), with the errors of the sums and of the
-// product; lo is meaningless where hi is not finite
-__device__ __forceinline__ void x_term(float &hi, float &lo, float a, float b, float ch, float cl) {
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+// all pairs, each added on its own
+template <int N>
+__device__ __forceinline__ void x_fine(const float2 (&v)[N], int r, float &s, float &e) {
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) two_sum(s, e, x_pair(v, r, k, 0.f));
+}
+// (hi, lo) += (ch + cl) (s + e), with the errors of the product and the sum; lo
+// is meaningless where hi is not finite
+__device__ __forceinline__ void x_term(float &hi, float &lo, float s, float e, float ch, float cl) {
     const float p = __fmul_rn(ch, s);
-    const float pe = fmaf(ch, e, fmaf(cl, s, fmaf(ch, s, -p)));
-    const float t = __fadd_rn(hi, p), tb = __fsub_rn(t, hi);
-    lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, tb)), __fsub_rn(p, tb)) + pe;
-    hi = t;
+    lo += fmaf(ch, e, fmaf(cl, s, fmaf(ch, s, -p)));
+    two_sum(hi, lo, p);
 }
 
 template <bool Fine>
@@ -667,10 +668,14 @@ __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const
 #pragma unroll
             for (int r = 0; r < 5; ++r) {
                 if (!((mask >> r) & 1u)) continue;
-                if (Fine)
-                    acc = fma(A.c[base + r], x_pairs_fine(v, r), acc);
-                else
-                    x_term(hi, lo, x_eight(v, r, 0), x_eight(v, r, 8), A.ch[base + r], A.cl[base + r]);
+                float s = 0.f, e = 0.f;
+                if (Fine) {
+                    x_fine(v, r, s, e);
+                } else {
+                    s = x_eight(v, r, 0);
+                    two_sum(s, e, x_eight(v, r, 8));
+                }
+                x_term(hi, lo, s, e, A.ch[base + r], A.cl[base + r]);
             }
         };
         if (mA) {
@@ -690,7 +695,7 @@ __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const
             five(v, mB, 5);
         }
         if (mC) {
-            float h[3][4];  // four pairs each
+            float h[3][4] = {}, fs[3] = {}, fe[3] = {};  // four pairs each, or all sixteen
 #pragma unroll
             for (uint32_t s = 0; s < 4; ++s) {
                 float2 v[8];
@@ -700,20 +705,22 @@ __global__ void __launch_bounds__(kXThreads, kXCtasPerSm) k_expect_x_tiles(const
                 for (int r = 0; r < 3; ++r) {
                     if (!((mC >> r) & 1u)) continue;
                     if (Fine)
-                        acc = fma(A.c[10 + r], x_pairs_fine(v, r), acc);
+                        x_fine(v, r, fs[r], fe[r]);
                     else
                         h[r][s] = x_four(v, r, 0);
                 }
             }
-            if (!Fine) {
 #pragma unroll
-                for (int r = 0; r < 3; ++r)
-                    if ((mC >> r) & 1u)
-                        x_term(hi, lo, __fadd_rn(h[r][0], h[r][1]), __fadd_rn(h[r][2], h[r][3]), A.ch[10 + r],
-                               A.cl[10 + r]);
+            for (int r = 0; r < 3; ++r) {
+                if (!((mC >> r) & 1u)) continue;
+                if (!Fine) {
+                    fs[r] = __fadd_rn(h[r][0], h[r][1]);
+                    two_sum(fs[r], fe[r], __fadd_rn(h[r][2], h[r][3]));
+                }
+                x_term(hi, lo, fs[r], fe[r], A.ch[10 + r], A.cl[10 + r]);
             }
         }
-        if (!Fine) acc += (double)hi + (isfinite(hi) ? (double)lo : 0.0);
+        acc += (double)hi + (isfinite(hi) ? (double)lo : 0.0);
     }
     acc = block_sum(acc * A.scale, sh);
     if (threadIdx.x == 0) partials[blockIdx.x] = acc;
@@ -1039,9 +1046,9 @@ int field_passes(qsim *s, uint64_t field, const double *c, double scale, unsigne
             if ((V >> b) & 1ull) {
                 if (((field & ~done) >> b) & 1ull) {
                     A.mask |= 1u << k;
-                    A.c[k] = 2.0 * c[b] / scale;
-                    A.ch[k] = (float)A.c[k];
-                    A.cl[k] = (float)(A.c[k] - (double)A.ch[k]);
+                    const double ck = 2.0 * c[b] / scale;
+                    A.ch[k] = (float)ck;
+                    A.cl[k] = (float)(ck - (double)A.ch[k]);
                 }
                 A.vspec.pos[k++] = b;
             }
