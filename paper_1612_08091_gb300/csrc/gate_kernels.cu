@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(128) k_monomial(double2 *__restrict__ psi, uin
 // (amplitudes of very different sizes under rows that do not mix them), the
 // result is formed again in pairs, from the inputs kept in shared memory.
 // 26 qubits, 4-qubit blocks: 0.99 to 1.17 ms a pass on a full state; a circuit of
-// 27 passes 22.3 ms, 5.6e-15 from 64 bits, in pairs 43.7 ms and 6.2e-14.  (51 bits
+// 27 passes 21.5 ms, 5.7e-15 from 64 bits, in pairs 43.7 ms and 6.2e-14.  (51 bits
 // and no look at the rows: 21.7 ms, 6.0e-14, and amplitudes far below the group's
 // largest kept few bits.)  Bound by issue and the integer multiply-adds.
 template <int K> struct MatKFx {
@@ -331,7 +331,7 @@ template <int K> struct MatKFx {
     float2 b[(1 << K) * (1 << K)];  // re lo, im lo
     qsim_df::C2 m[(1 << K) * (1 << K)];
     float w[(1 << K) * (1 << K)];   // |element|, the largest row sum being 1/2 to 1
-    float low[4][1 << K];           // the least of each quarter of a column
+    float low[4][1 << K];           // the least of a quarter of the rows
     uint64_t off[1 << K];
     int shift;                    // -1027 - S
 };
@@ -414,7 +414,6 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
         xi[r] = to_fxf(v[r].y, E);
     }
     uint32_t apart = 0, nz = 0;  // rows to be formed apart, amplitudes that are not 0
-    bool look;
     {
         float size[D], low = 0x1p30f, count = 0.f;
 #pragma unroll
@@ -430,15 +429,7 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
             for (int c = 0; c < D; ++c) t = fmaf(M.low[q][c], size[c], t);
             low = fminf(low, t);
         }
-        look = __any_sync(__activemask(), low < line);
-        if (look) {
-            // (read again, one by one: v kept, or all at once, takes 40 registers more)
-#pragma unroll 1
-            for (int r = 0; r < D; ++r) {
-                const double2 z = p[M.off[r]];
-                s_in[r][threadIdx.x] = z;
-                nz |= (uint32_t)(z.x != 0.0 || z.y != 0.0) << r;
-            }
+        if (__any_sync(__activemask(), low < line)) {
 #pragma unroll 2
             for (int r = 0; r < D; ++r) {
                 float t = 0.f;
@@ -446,6 +437,15 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
                 for (int c = 0; c < D; ++c) t = fmaf(M.w[r * D + c], size[c], t);
                 apart |= (uint32_t)(t < line) << r;
             }
+        }
+    }
+    if (apart) {
+        // (read again, one by one: v kept, or all at once, takes 40 registers more)
+#pragma unroll 1
+        for (int r = 0; r < D; ++r) {
+            const double2 z = p[M.off[r]];
+            s_in[r][threadIdx.x] = z;
+            nz |= (uint32_t)(z.x != 0.0 || z.y != 0.0) << r;
         }
     }
     const int eadd = (E + M.shift) << 20;
@@ -475,8 +475,10 @@ __global__ void __launch_bounds__(128) k_denseK_fx(double2 *__restrict__ psi, ui
         p[M.off[r]] = make_double2(to_double_f(rr - ii, cr + dr, eadd), to_double_f(ri, ci + di, eadd));
     }
 #pragma unroll 1
-    for (int r = 0; r < D && look; ++r)
-        if ((apart >> r) & 1u) p[M.off[r]] = row_apart<K>(M.m + r * D, s_in, nz, E);
+    for (; apart; apart &= apart - 1u) {
+        const int r = __ffs(apart) - 1;
+        p[M.off[r]] = row_apart<K>(M.m + r * D, s_in, nz, E);
+    }
 }
 
 qsim_df::F2 host_split(double x) {
@@ -652,10 +654,19 @@ int dense_k_fx(qsim *s, const int *targets, uint64_t cmask, const cd *m) {
         M.m[i] = qsim_df::C2{host_split(m[i].real()), host_split(m[i].imag())};
         M.w[i] = (float)std::ldexp(std::abs(m[i]), -x);
     }
+    // the least elements of a quarter's rows, rows that mix the same columns together
+    uint32_t cols[D] = {0};
+    int row[D];
+    for (int r = 0; r < D; ++r) {
+        row[r] = r;
+        for (int c = 0; c < D; ++c) cols[r] |= (uint32_t)(M.w[r * D + c] > 0x1p-20f) << c;
+    }
+    std::stable_sort(row, row + D, [&](int a, int b) { return cols[a] < cols[b]; });
     for (int q = 0; q < 4; ++q)
         for (int c = 0; c < D; ++c) {
-            M.low[q][c] = M.w[q * (D / 4) * D + c];
-            for (int r = q * (D / 4); r < (q + 1) * (D / 4); ++r) M.low[q][c] = std::min(M.low[q][c], M.w[r * D + c]);
+            float low = M.w[row[q * (D / 4)] * D + c];
+            for (int k = 1; k < D / 4; ++k) low = std::min(low, M.w[row[q * (D / 4) + k] * D + c]);
+            M.low[q][c] = low;
         }
     M.shift = -1027 - S;
     const InsertSpec ins = make_spec(tmask | cmask);
