@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(128) k_denseK_df(double2 *__restrict__ psi, ui
 // in each row and column (CNOTs, SWAPs, phases), double-float option: every
 // amplitude goes to its place, times its element in FP64 unless that is 1.  26
 // qubits, a block of CNOTs: 0.49 ms (4.4 TB/s; 16 amplitudes a thread, few
-// threads) where the integer form below takes 0.99 and rounds.
+// threads) where the integer form below takes 0.98 and rounds.
 template <int K> struct MatKMono {
     double2 w[1 << K];
     uint64_t from[1 << K], to[1 << K];
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(128) k_monomial(double2 *__restrict__ psi, uin
 // (fx128.cuh) on the error is below 2^-44.6 of it; where it is smaller
 // (amplitudes of very different sizes under rows that do not mix them), the
 // result is formed again in pairs, from the inputs kept in shared memory.
-// 26 qubits, 4-qubit blocks: 0.99 to 1.17 ms a pass on a full state; a circuit of
+// 26 qubits, 4-qubit blocks: 0.98 to 1.04 ms a pass on a full state; a circuit of
 // 27 passes 21.5 ms, 5.7e-15 from 64 bits, in pairs 43.7 ms and 6.2e-14.  (51 bits
 // and no look at the rows: 21.7 ms, 6.0e-14, and amplitudes far below the group's
 // largest kept few bits.)  Bound by issue and the integer multiply-adds.
